@@ -311,10 +311,10 @@ cavity_status cavity_lu_solve(cavity_ctx* ctx, const void* lu, int n, int lda, c
  * operator variants to ~1e-7 relative, the group width within the solver
  * tolerance).  Set per context, at any time between calls; the
  * paper_2008_01966_gb300.autotune module times them and caches its choice.
- *  CAVITY_OPT_PASS_B_2048, CAVITY_OPT_PASS_C_2048: FP32 operator passes B and
- *      C on lines of 2048 points (512-point grid sides): 0 = each line on a
- *      pair of warps (one radix-2 step, then a 1024-point warp transform per
- *      warp; default), 1 = the block (Stockham) transform.
+ *  CAVITY_OPT_PASS_B_2048, CAVITY_OPT_PASS_C_2048: FP32 operator on grids with
+ *      nx = 512 (B) or ny = 512 (C): 0 = lines of 2048 points in the registers
+ *      of a group of lanes (default), 1 = the generic passes with the block
+ *      (Stockham) transform.
  *  CAVITY_OPT_GROUP_WIDTH: directions per group of the mixed solve's block
  *      Krylov iterations (one basis per group), 1..16; default 16.
  *  CAVITY_OPT_COARSE_MODES: two-level preconditioner of the mixed solve's

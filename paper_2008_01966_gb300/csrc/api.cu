@@ -92,6 +92,7 @@ extern "C" cavity_status cavity_setup(const cavity_desc* desc, void* cuda_stream
   ctx->TW = 2 * std::max(g.Px, g.Py);
   cavity_status s = launch_twiddles(ctx);
   if (s == CAVITY_OK && g.fft_ok) s = launch_ehat(ctx);
+  if (s == CAVITY_OK && g.fft_ok) s = launch_lane_tables(ctx);
   if (s == CAVITY_OK) {
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {
@@ -116,7 +117,7 @@ extern "C" void cavity_destroy(cavity_ctx* ctx) {
                   ctx->top64, ctx->top32, ctx->pinv64, ctx->pinv32, ctx->prof32, ctx->profq32,
                   ctx->minpiv, ctx->ws, ctx->ws2, ctx->stage, ctx->tw_p, ctx->ehat_xp[0],
                   ctx->ehat_xp[1], ctx->ehat_yp[0], ctx->ehat_yp[1], ctx->khat_p, ctx->top_p, ctx->prof_rec,
-                  ctx->dn_scr};
+                  ctx->dn_scr, ctx->khat32s, ctx->lane_tab[0], ctx->lane_tab[1]};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   dense_free(ctx->dn);
@@ -202,7 +203,10 @@ extern "C" cavity_status cavity_prepare(cavity_ctx* ctx, double kappa0, int nlay
   bool kappa_same = ctx->khat64 && ctx->kappa0 == kappa0;
   ctx->kappa0 = kappa0;
   ctx->layers = L;
-  if (!kappa_same) CKS(launch_khat(ctx, kappa0));
+  if (!kappa_same) {
+    CKS(launch_khat(ctx, kappa0));
+    if (ctx->g.fft_ok) CKS(launch_khat_split(ctx));
+  }
   CKS(launch_zsweep(ctx, kappa0));
   if (ctx->g.fft_ok) {   // the Krylov path's preconditioner and operator tables
     CKS(launch_precond(ctx));

@@ -144,6 +144,8 @@ struct cavity_ctx {
   std::vector<LayerDev> layers;
   double2* khat64 = nullptr;   // quarter box [j2][j1] (Py/2 x Px/2), scaled by 1/(Lx Ly)
   float2* khat32 = nullptr;
+  float2* khat32s = nullptr;   // khat32 by parity of j1 for the FP32 passes (tbc_f32.cu)
+  float2* lane_tab[2] = {nullptr, nullptr};  // their twiddle tables per axis (gfft.cuh)
   double2* khat_raw = nullptr; // unscaled copy [j1][j2] for export
   double2* prof = nullptr;     // (nz-1) x nap profiles P, level-major
   double2* profq = nullptr;    // (nz-1) x (n1+n2) profiles Q (layered only)
@@ -314,6 +316,15 @@ cavity_status launch_rhs(cavity_ctx* ctx, int ndir, const double* theta,
 template <typename T>
 cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
                            long long ystride = -1);
+template <>
+cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, float2* y, void* work,
+                                  long long ystride);
+// sides (log2) that the FP32 operator's own passes take (tbc_f32.cu), their
+// tables (once per context) and their copy of the kernel table (per kappa0)
+#define F32_LOG_MIN 4
+inline bool f32_fast_size(int ln) { return ln >= F32_LOG_MIN; }
+cavity_status launch_lane_tables(cavity_ctx* ctx);
+cavity_status launch_khat_split(cavity_ctx* ctx);
 size_t apply_work_bytes(const Geo& g, int ndir, int elem_bytes);
 // y = A x in pair-of-FP32 arithmetic (~1e-12), FP64 vectors in and out;
 // work: apply_pair_work_bytes

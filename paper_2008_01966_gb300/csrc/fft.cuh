@@ -492,48 +492,3 @@ __device__ __forceinline__ void fft_warp_lines(C<T>* base, int lstride, int firs
     fft_warp<T, INV, LW, S::RV, Op>(line, 1 << LOGN, LOGN, t, active, tw, twlog, l, op);
   }
 }
-
-// Named barrier of the two warps of a two-warp transform (ids 1..15; 0 is
-// __syncthreads).
-__device__ __forceinline__ void pair_sync(int id) {
-  asm volatile("bar.sync %0, 64;" ::"r"(id) : "memory");
-}
-
-// Two-warp transform of one FP32 line of length n = 2^LOGN (2048): one radix-2
-// step (decimation in frequency) and a warp transform of length n/2 per warp.
-// Warp h (0 or 1) forms u_h[i] = x[i] + x[i + n/2] (h = 0) or
-// (x[i] - x[i + n/2]) w_n^i (h = 1) and transforms it: X[2k + h] = DFT_{n/2}(u_h)[k].
-// Both warps read the whole line (op.ld) before either writes; their tiles
-// lie in disjoint halves of the line (the line's padded length is at least
-// n + n/8); both finish reading their tiles before either stores (op.st with
-// the output index 2k + h).  bar_id: a named barrier owned by the two warps.
-template <typename T, bool INV, int LOGN, typename Op = LineId<T>>
-__device__ __forceinline__ void fft_warp2(C<T>* line, int h, int l, const C<T>* __restrict__ tw,
-                                          int twlog, int bar_id, int lidx = 0,
-                                          const Op& op = Op()) {
-  constexpr int n = 1 << LOGN, nh = n / 2;
-  using S = LineShape<T, LOGN - 1>;
-  static_assert(S::WARP && S::LW == 32, "two-warp transform of 2 x 1024 points");
-  constexpr int LW = S::LW, RV = S::RV;
-  C<T> v[RV];
-  const int shift = twlog - LOGN;
-#pragma unroll
-  for (int r = 0; r < RV; ++r) {
-    const int i = l + LW * r;
-    const C<T> a = op.ld(lidx, line, i), b = op.ld(lidx, line, i + nh);
-    v[r] = h == 0 ? cadd<T>(a, b) : cmul<T>(csub<T>(a, b), twid<T, INV>(tw, i << shift));
-  }
-  pair_sync(bar_id);
-  constexpr int TILE = RV * (LW + 1);
-  static_assert(TILE <= nh + nh / 8, "tiles fit in the two halves of the padded line");
-  fft_warp_core<T, INV, LW, RV>(v, line + h * (nh + nh / 8), nh, LOGN - 1, l, true, tw, twlog);
-  pair_sync(bar_id);
-  constexpr int Q = RV / LW;
-#pragma unroll
-  for (int q = 0; q < Q; ++q) {
-    const int k1 = l + LW * q;
-#pragma unroll
-    for (int k2 = 0; k2 < LW; ++k2) op.st(lidx, line, 2 * (k1 + RV * k2) + h, v[q * LW + k2]);
-  }
-  __syncwarp();
-}

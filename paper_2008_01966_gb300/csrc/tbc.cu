@@ -6,10 +6,6 @@
 
 #include "tbc_apply.cuh"
 
-// the FP32 operator is instantiated in tbc_f32.cu
-extern template cavity_status launch_apply<float>(cavity_ctx*, int, const float2*, float2*, void*,
-                                                 long long);
-
 // ------------------------------------------------------------------ setup
 __global__ void k_twiddles(double2* tw64, float2* tw32, int TW) {
   int k = blockIdx.x * blockDim.x + threadIdx.x;

@@ -19,7 +19,9 @@
 // Templated on the arithmetic type: FP64 for the FP64 path and the residuals,
 // FP32 for the inner Krylov iterations of the mixed path.  Every pass kernel
 // is instantiated per grid size so that its line transforms have compile-time
-// lengths; tbc.cu instantiates the FP64 operator, tbc_f32.cu the FP32 one.
+// lengths; tbc.cu instantiates the FP64 operator, tbc_df*.cu the pair-of-FP32 one.
+// The FP32 operator has passes of its own (tbc_f32.cu) and takes these only on
+// sides of 4 or 8 intervals, or when a pass option asks for them.
 #pragma once
 #include <algorithm>
 #include <atomic>
@@ -135,33 +137,6 @@ struct ParityProducts : G {
   }
 };
 
-// last write of the forward transform when each parity line transforms its
-// own copy of the column: the product with its parity's kernel, in place
-template <typename T>
-struct OwnParity : LineId<T> {
-  const C<T>* eh;                 // [r][P]
-  int P, L;
-  __device__ __forceinline__ void st(int l, C<T>* line, int k, C<T> v) const {
-    const int r = l >= L ? 1 : 0;
-    line[pidx(k)] = cmul<T>(v, eh[r * P + k]);
-  }
-};
-
-// pass A with one copy of the row per parity line: gather of row (l mod L),
-// product with the kernel of parity (l >= L), in place
-template <typename T, int LNY>
-struct GatherOwnA : GatherA<T, LNY> {
-  const C<T>* eh;                 // [r][P]
-  int P, L;
-  __device__ __forceinline__ C<T> ld(int l, const C<T>* line, int n) const {
-    return GatherA<T, LNY>::ld(l >= L ? l - L : l, line, n);
-  }
-  __device__ __forceinline__ void st(int l, C<T>* line, int k, C<T> v) const {
-    const int r = l >= L ? 1 : 0;
-    line[pidx(k)] = cmul<T>(v, eh[r * P + k]);
-  }
-};
-
 // last write of the inverse transforms of pass A: Vy(k1, j), j = 2t + r mod Py
 template <typename T, int LNY>
 struct ScatterA : LineId<T> {
@@ -193,42 +168,21 @@ __global__ void TBC_BOUNDS_LN(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __re
   sc.row0 = row0;
   sc.nx = p.nx;
   sc.L = L;
-  if constexpr (LineShape<T, LPY>::WARP && 2 * L * LineShape<T, LPY>::TPL == LINES_THREADS) {
-    // every warp transforms its own lines (parity 0 or 1 of a row) from the
-    // gather to the scatter, the row's forward transform done by both of its
-    // lines' warps: no idle warps and no block barrier
-    GatherOwnA<T, LNY> fwd;
-    fwd.E1 = x + (size_t)d * p.nap;
-    fwd.E2 = fwd.E1 + p.n1;
-    fwd.row0 = row0;
-    fwd.nx = p.nx;
-    fwd.f = f;
-    fwd.pib = (T)p.pib;
-    fwd.pia = (T)p.pia;
-    fwd.eh = f != 0 ? eh_c : eh_s;
-    fwd.P = Py;
-    fwd.L = L;
-    constexpr int LPW = 32 / LineShape<T, LPY>::TPL;
-    const int first = (threadIdx.x >> 5) * LPW;
-    fft_warp_lines<T, false, LPY>(buf, ls, first, LPW, tw, p.twlog, fwd);
-    fft_warp_lines<T, true, LPY>(buf, ls, first, LPW, tw, p.twlog, sc);
-  } else {
-    ParityProducts<T, GatherA<T, LNY>> fwd;
-    fwd.E1 = x + (size_t)d * p.nap;
-    fwd.E2 = fwd.E1 + p.n1;
-    fwd.row0 = row0;
-    fwd.nx = p.nx;
-    fwd.f = f;
-    fwd.pib = (T)p.pib;
-    fwd.pia = (T)p.pia;
-    fwd.eh = f != 0 ? eh_c : eh_s;
-    fwd.P = Py;
-    fwd.L = L;
-    fwd.ls = ls;
-    fwd.buf = buf;
-    fft_lines<T, false, LPY>(buf, ls, L, tw, p.twlog, fwd);
-    fft_lines<T, true, LPY>(buf, ls, 2 * L, tw, p.twlog, sc);
-  }
+  ParityProducts<T, GatherA<T, LNY>> fwd;
+  fwd.E1 = x + (size_t)d * p.nap;
+  fwd.E2 = fwd.E1 + p.n1;
+  fwd.row0 = row0;
+  fwd.nx = p.nx;
+  fwd.f = f;
+  fwd.pib = (T)p.pib;
+  fwd.pia = (T)p.pia;
+  fwd.eh = f != 0 ? eh_c : eh_s;
+  fwd.P = Py;
+  fwd.L = L;
+  fwd.ls = ls;
+  fwd.buf = buf;
+  fft_lines<T, false, LPY>(buf, ls, L, tw, p.twlog, fwd);
+  fft_lines<T, true, LPY>(buf, ls, 2 * L, tw, p.twlog, sc);
 }
 
 // ------------------------------------------------------------------ pass B
@@ -304,9 +258,6 @@ __global__ void TBC_BOUNDS_LN(LNX) k_tbcB(const C<T>* __restrict__ Vy, C<T>* __r
   const int j0 = blockIdx.x * L;
   const int tid = threadIdx.x, nthr = blockDim.x;
   const bool xcos = (f != 1);
-  // the per-warp chain (below) needs the column in both of its lines
-  constexpr int NCOPY = (LineShape<T, LPX>::WARP && LineShape<T, LPX - 1>::WARP &&
-                         2 * L * LineShape<T, LPX>::TPL == LINES_THREADS) ? 2 : 1;
   // shared memory: 2L lines, then the two parity kernels [2][Px], then the
   // kernel-table rows |j2| of the L columns [L][Px/2] (staged once per block,
   // so the fused products read shared memory instead of waiting on loads)
@@ -337,14 +288,11 @@ __global__ void TBC_BOUNDS_LN(LNX) k_tbcB(const C<T>* __restrict__ Vy, C<T>* __r
       const C<T> c = j < Py ? src[(size_t)k1 * Py + j] : czero<T>();
       const C<T> c0 = k1 == 0 ? (xcos ? cscale<T>(c, (T)2) : czero<T>()) : c;
       const C<T> cm = xcos ? c : mk<T>(-c.x, -c.y);
-#pragma unroll
-      for (int r = 0; r < NCOPY; ++r) {
-        C<T>* line = buf + (size_t)(r * L + l) * ls;
-        line[pidx(k1)] = c0;
-        if (k1 > 0) line[pidx(Px - k1)] = cm;
-      }
+      C<T>* line = buf + (size_t)l * ls;
+      line[pidx(k1)] = c0;
+      if (k1 > 0) line[pidx(Px - k1)] = cm;
     }
-    for (int idx = tid; idx < NCOPY * L * (2 * nx + 1); idx += nthr) {
+    for (int idx = tid; idx < L * (2 * nx + 1); idx += nthr) {
       const int l = idx / (2 * nx + 1), k = nx + idx - l * (2 * nx + 1);
       buf[(size_t)l * ls + pidx(k)] = czero<T>();
     }
@@ -355,33 +303,15 @@ __global__ void TBC_BOUNDS_LN(LNX) k_tbcB(const C<T>* __restrict__ Vy, C<T>* __r
   kb.j0 = j0;
   kb.Py = Py;
   kb.L = L;
-  if constexpr (LineShape<T, LPX>::WARP && LineShape<T, LPX - 1>::WARP &&
-                2 * L * LineShape<T, LPX>::TPL == LINES_THREADS) {
-    // every warp runs the whole chain on its own lines (a parity-0 or a
-    // parity-1 line of a column): the forward transform of the column is done
-    // by both of its lines' warps, so no warp idles and no block barrier is
-    // needed until the two parities are combined
-    constexpr int LPW = 32 / LineShape<T, LPX>::TPL;
-    const int first = (tid >> 5) * LPW;
-    OwnParity<T> fwd;
-    fwd.eh = eh_use;
-    fwd.P = Px;
-    fwd.L = L;
-    fft_warp_lines<T, false, LPX>(buf, ls, first, LPW, tw, p.twlog, fwd);
-    fft_warp_lines<T, true, LPX>(buf, ls, first, LPW, tw, p.twlog, kb);
-    fft_warp_lines<T, true, LPX - 1>(buf, ls, first, LPW, tw, p.twlog);
-    __syncthreads();
-  } else {
-    ParityProducts<T, LineId<T>> fwd;
-    fwd.eh = eh_use;
-    fwd.P = Px;
-    fwd.L = L;
-    fwd.ls = ls;
-    fwd.buf = buf;
-    fft_lines<T, false, LPX>(buf, ls, L, tw, p.twlog, fwd);
-    fft_lines<T, true, LPX>(buf, ls, 2 * L, tw, p.twlog, kb);
-    fft_lines<T, true, LPX - 1>(buf, ls, 2 * L, tw, p.twlog);
-  }
+  ParityProducts<T, LineId<T>> fwd;
+  fwd.eh = eh_use;
+  fwd.P = Px;
+  fwd.L = L;
+  fwd.ls = ls;
+  fwd.buf = buf;
+  fft_lines<T, false, LPX>(buf, ls, L, tw, p.twlog, fwd);
+  fft_lines<T, true, LPX>(buf, ls, 2 * L, tw, p.twlog, kb);
+  fft_lines<T, true, LPX - 1>(buf, ls, 2 * L, tw, p.twlog);
   C<T>* dst = W + (size_t)(d * 3 + f) * (nx + 1) * Py;
   const int sh = p.twlog - LPX;
   for (int idx = tid; idx < L * (nx + 1); idx += nthr) {
@@ -511,182 +441,6 @@ __global__ void TBC_BOUNDS_LN(LNX) k_tbcD(const C<T>* __restrict__ Z, C<T>* __re
   fft_lines<T, false, LNX + 1>(buf, ls, L, tw, p.twlog, cd);
 }
 
-// ------------------------------------------------------------------ passes B, C at 2048 points
-// FP32 lines of 2048 points (the 512 x 512 grid: Px = Py = 2048) do not fit
-// one warp's registers; each line is transformed by two warps (fft_warp2:
-// one radix-2 step, then a 1024-point warp transform per warp), so these
-// passes keep the warp transforms of the smaller grids -- no block barrier
-// inside a transform, one shared-memory round trip per 1024-point half.
-// Pass B: two columns per block of eight warps, each parity line on a warp
-// pair; pass C: four rows per block, each on a warp pair; the named barrier
-// of pair g is 1 + g.  (Pass A keeps the block transform at this size: a
-// two-warp version measured 0.46 against 0.29 ms per 8-direction launch.)
-template <int N2> struct W2 {
-  static constexpr int LS = padded_len(N2);
-  static constexpr int L = 2;           // rows / columns per block
-};
-
-// pass B: grid (Py / 2 column pairs, 3 fields, ndir).  The parity kernels
-// are read from global memory (32 KB, L1 resident); shared memory holds the
-// four lines and the kernel-table rows of the two columns.
-template <typename T>
-struct OwnParityG : LineId<T> {
-  const C<T>* __restrict__ eh;    // [r][P], global
-  int P, L;
-  __device__ __forceinline__ void st(int l, C<T>* line, int k, C<T> v) const {
-    const int r = l >= L ? 1 : 0;
-    line[pidx(k)] = cmul<T>(v, __ldg(eh + r * P + k));
-  }
-};
-
-// KhatB for the two-warp pass: the lanes of a warp write outputs 2 apart, so
-// they read the kernel table 4 apart in j1; the rows are staged with
-// j1 -> (j1 mod 4) (Px/8 + 4) + j1 / 4 (row length KH_ROW), which makes
-// those reads consecutive and the staging writes free of bank conflicts
-template <int LNX>
-struct KhatBPerm : LineId<float> {
-  static constexpr int KH_ROW = 4 * ((4 << LNX) / 8 + 4);
-  const float2* kh;               // rows |j2| of the block's columns, permuted
-  int j0, Py, L;
-  __device__ __forceinline__ static int perm(int j1) {
-    constexpr int Px = 4 << LNX;
-    return (j1 & 3) * (Px / 8 + 4) + (j1 >> 2);
-  }
-  __device__ __forceinline__ void st(int lr, float2* line, int k, float2 v) const {
-    constexpr int Px = 4 << LNX, hp = Px / 2, qp = Px / 4;
-    int t, u;
-    if (k < qp) { t = k; u = k; }
-    else if (k >= Px - qp) { t = k - Px; u = k - hp; }
-    else return;
-    const int r = lr >= L ? 1 : 0, l = lr - r * L;
-    const int j = j0 + l;
-    const int j1 = 2 * t + r;
-    float2 o = czero<float>();
-    if (j1 != -hp && j < Py && j != Py / 2) {
-      const int j1a = j1 < 0 ? -j1 : j1;
-      o = cmul<float>(v, kh[l * KH_ROW + perm(j1a)]);
-    }
-    line[pidx(u)] = o;
-  }
-};
-
-template <int LNX>
-__global__ void __launch_bounds__(LINES_THREADS, 2)
-    k_tbcB_w2(const float2* __restrict__ Vy, float2* __restrict__ W, TbcP p,
-              const float2* __restrict__ tw, const float2* __restrict__ eh_c,
-              const float2* __restrict__ eh_s, const float2* __restrict__ kh) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  float2* buf = (float2*)sm_raw;
-  constexpr int LPX = LNX + 2, Px = 1 << LPX, nx = 1 << LNX, ls = W2<Px>::LS, L = W2<Px>::L;
-  const int Py = p.Py;
-  const int f = blockIdx.y, d = blockIdx.z;
-  const int j0 = blockIdx.x * L;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const int warp = tid >> 5, lane = tid & 31;
-  const bool xcos = (f != 1);
-  float2* kh_sm = buf + (size_t)2 * L * ls;
-  for (int idx = tid; idx < L * (Px / 2); idx += nthr) {
-    const int l = idx >> (LPX - 1), j1 = idx & (Px / 2 - 1);
-    const int j = j0 + l;
-    const int j2a = j < Py / 2 ? j : Py - j;
-    kh_sm[l * KhatBPerm<LNX>::KH_ROW + KhatBPerm<LNX>::perm(j1)] =
-        (j < Py && j != Py / 2) ? kh[(size_t)j2a * (Px / 2) + j1] : czero<float>();
-  }
-  // both parity lines of each column receive the mirrored column; the slots
-  // [nx, Px - nx] are cleared
-  {
-    const float2* src = Vy + (size_t)(d * 3 + f) * nx * Py;
-    for (int idx = tid; idx < L * nx; idx += nthr) {
-      const int k1 = idx >> 1, l = idx & 1;
-      const int j = j0 + l;
-      const float2 c = j < Py ? src[(size_t)k1 * Py + j] : czero<float>();
-      const float2 c0 = k1 == 0 ? (xcos ? cscale<float>(c, 2.f) : czero<float>()) : c;
-      const float2 cm = xcos ? c : mk<float>(-c.x, -c.y);
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        float2* line = buf + (size_t)(r * L + l) * ls;
-        line[pidx(k1)] = c0;
-        if (k1 > 0) line[pidx(Px - k1)] = cm;
-      }
-    }
-    for (int idx = tid; idx < 2 * L * (2 * nx + 1); idx += nthr) {
-      const int l = idx / (2 * nx + 1), k = nx + idx - l * (2 * nx + 1);
-      buf[(size_t)l * ls + pidx(k)] = czero<float>();
-    }
-    __syncthreads();
-  }
-  const int lr = warp >> 1, h = warp & 1;
-  float2* line = buf + (size_t)lr * ls;
-  OwnParityG<float> fwd;
-  fwd.eh = xcos ? eh_c : eh_s;
-  fwd.P = Px;
-  fwd.L = L;
-  fft_warp2<float, false, LPX>(line, h, lane, tw, p.twlog, 1 + lr, lr, fwd);
-  pair_sync(1 + lr);
-  KhatBPerm<LNX> kb;
-  kb.kh = kh_sm;
-  kb.j0 = j0;
-  kb.Py = Py;
-  kb.L = L;
-  fft_warp2<float, true, LPX>(line, h, lane, tw, p.twlog, 1 + lr, lr, kb);
-  pair_sync(1 + lr);
-  if (h == 0) fft_warp<float, true, 32, 32>(line, Px / 2, LPX - 1, lane, true, tw, p.twlog);
-  __syncthreads();
-  float2* dst = W + (size_t)(d * 3 + f) * (nx + 1) * Py;
-  const int sh = p.twlog - LPX;
-  for (int idx = tid; idx < L * (nx + 1); idx += nthr) {
-    const int q = idx >> 1, l = idx & 1;
-    const int j = j0 + l;
-    if (j >= Py) continue;
-    const float2 z0 = buf[(size_t)l * ls + pidx(q)];
-    const float2 z1 = buf[(size_t)(L + l) * ls + pidx(q)];
-    dst[(size_t)q * Py + j] = cadd<float>(z0, cmul<float>(z1, twid<float, true>(tw, q << sh)));
-  }
-}
-
-// pass C: grid (ceil((nx+1) / 4) row groups, 3 fields, ndir); four rows per
-// block, the inverse torus transform of a row (2048 points) on a warp pair,
-// then its projection (1024 points) on the pair's first warp
-template <int LNY>
-__global__ void __launch_bounds__(LINES_THREADS, 2)
-    k_tbcC_w2(const float2* __restrict__ W, float2* __restrict__ Z, TbcP p,
-              const float2* __restrict__ tw) {
-  extern __shared__ __align__(16) unsigned char sm_raw[];
-  float2* buf = (float2*)sm_raw;
-  constexpr int LPY = LNY + 2, Py = 1 << LPY, ny = 1 << LNY, ls = W2<Py>::LS;
-  constexpr int RB = 4;   // rows per block
-  const int f = blockIdx.y, d = blockIdx.z;
-  const int r0 = blockIdx.x * RB;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int l = warp >> 1, h = warp & 1;
-  const bool ycos = (f != 0);
-  RowC<float, LNY> rc;
-  rc.src = W + (size_t)(d * 3 + f) * (p.nx + 1) * Py;
-  rc.r0 = r0;
-  rc.nx = p.nx;
-  rc.ycos = ycos;
-  float2* line = buf + (size_t)l * ls;
-  fft_warp2<float, true, LPY>(line, h, lane, tw, p.twlog, 1 + l, l, rc);
-  pair_sync(1 + l);
-  if (h == 0) {
-    StoreZ<float, LNY> sz;
-    sz.Z = Z + (size_t)(d * 3 + f) * (p.nx + 1) * (ny + 1);
-    sz.r0 = r0;
-    sz.nx = p.nx;
-    sz.ycos = ycos;
-    sz.w = (float)p.wy;
-    fft_warp<float, false, 32, 32>(line, 2 * ny, LNY + 1, lane, true, tw, p.twlog, l, sz);
-  }
-}
-
-template <typename T> __host__ __device__ constexpr bool w2_ok(int ln) {
-  return sizeof(T) == 4 && ln == 9;
-}
-static size_t smem_b_w2(int nx) {
-  return sizeof(float2) * (4 * (size_t)padded_len(4 * nx) + 2 * (size_t)(2 * nx + 16));
-}
-static size_t smem_c_w2(int ny) { return sizeof(float2) * 4 * (size_t)padded_len(4 * ny); }
-
 // ------------------------------------------------------------------ combine
 // y = local part of (EJ1)/(uT1) + TBC rows, with the TBC sign that makes T
 // the exterior admittance z x curl E^s of (EGa2):
@@ -694,17 +448,19 @@ static size_t smem_c_w2(int ny) { return sizeof(float2) * 4 * (size_t)padded_len
 //  row 2: (-1+tau2)E2 + (n pi h/b + vs2)E3 + (h/c)(2k^2 U2 + 2(m pi/a) W)
 //  row 3: (m pi h/a)E1 + (n pi h/b)E2 + (-1+tau3)E3
 // One thread per mode pair (m, n), m < nx, n < ny, writing the rows of the
-// three components that exist for it; grid (ceil(nx ny / 256), ndir).
+// three components that exist for it; nyp: pitch of O's rows; grid
+// (ceil(nx ny / 256), ndir).
 template <typename T>
 __global__ void k_combine(const C<T>* __restrict__ x, const C<T>* __restrict__ O,
-                          const C<T>* __restrict__ top, C<T>* __restrict__ y, long long ys, TbcP p) {
+                          const C<T>* __restrict__ top, C<T>* __restrict__ y, long long ys, int nyp,
+                          TbcP p) {
   const int d = blockIdx.y;
   const int mn = blockIdx.x * blockDim.x + threadIdx.x;
   if (mn >= p.nx * p.ny) return;
   const int m = mn >> p.lny, n = mn & (p.ny - 1);
   const C<T>* xd = x + (size_t)d * p.nap;
   C<T>* yd = y + (size_t)d * ys;
-  const int N = p.N, nyp = p.ny + 1;
+  const int N = p.N;
   const size_t fs = (size_t)p.nx * nyp;
   const C<T>* Od = O + (size_t)d * 3 * fs;
   const T pa = (T)p.pia, pb = (T)p.pib, h = (T)p.h, ab = (T)p.ab;
@@ -830,8 +586,8 @@ cavity_status launch_mode_mask_t(cavity_ctx* ctx, int ndir, C<T>* y, long long y
 }
 
 template <typename T>
-cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
-                           long long ystride) {
+cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
+                                   long long ystride) {
   if (!ctx->g.fft_ok) {
     ctx->err = "the FFT operator needs the convolution period 4 on both axes";
     return CAVITY_EINVAL;
@@ -865,48 +621,21 @@ cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, vo
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     constexpr int L = pairs_per_cta<T>(4 << LN);
-    if constexpr (w2_ok<T>(LN)) {
-      if (ctx->opt[CAVITY_OPT_PASS_B_2048] == 0) {
-        static std::atomic<bool> done2{false};
-        CKS(smem_once(ctx, k_tbcB_w2<LN>, done2));
-        KScope ks_(ctx, kclass<T>(1));
-        k_tbcB_w2<LN><<<dim3(g.Py / 2, 3, ndir), T_, smem_b_w2(g.nx), st>>>(
-            (const float2*)R1, (float2*)R2, p, (const float2*)tw,
-            (const float2*)Tabs<T>::ex(ctx, 0), (const float2*)Tabs<T>::ex(ctx, 1),
-            (const float2*)Tabs<T>::kh(ctx));
-        return CAVITY_OK;
-      }
-    }
-    {
-      static std::atomic<bool> done{false};  // set once; host threads may race
-      CKS(smem_once(ctx, k_tbcB<T, LN>, done));
-      KScope ks_(ctx, kclass<T>(1));
-      k_tbcB<T, LN><<<dim3((g.Py + L - 1) / L, 3, ndir), T_, smem_b<T>(g.nx), st>>>(
-          R1, R2, p, tw, Tabs<T>::ex(ctx, 0), Tabs<T>::ex(ctx, 1), Tabs<T>::kh(ctx));
-      return CAVITY_OK;
-    }
+    static std::atomic<bool> done{false};  // set once; host threads may race
+    CKS(smem_once(ctx, k_tbcB<T, LN>, done));
+    KScope ks_(ctx, kclass<T>(1));
+    k_tbcB<T, LN><<<dim3((g.Py + L - 1) / L, 3, ndir), T_, smem_b<T>(g.nx), st>>>(
+        R1, R2, p, tw, Tabs<T>::ex(ctx, 0), Tabs<T>::ex(ctx, 1), Tabs<T>::kh(ctx));
+    return CAVITY_OK;
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     constexpr int L = lines_per_cta<T>(4 << LN);
-    if constexpr (w2_ok<T>(LN)) {
-      if (ctx->opt[CAVITY_OPT_PASS_C_2048] == 0) {
-        static std::atomic<bool> done2{false};
-        CKS(smem_once(ctx, k_tbcC_w2<LN>, done2));
-        KScope ks_(ctx, kclass<T>(2));
-        k_tbcC_w2<LN><<<dim3((g.nx + 1 + 3) / 4, 3, ndir), T_, smem_c_w2(g.ny), st>>>(
-            (const float2*)R2, (float2*)R1, p, (const float2*)tw);
-        return CAVITY_OK;
-      }
-    }
-    {
-      static std::atomic<bool> done{false};  // set once; host threads may race
-      CKS(smem_once(ctx, k_tbcC<T, LN>, done));
-      KScope ks_(ctx, kclass<T>(2));
-      k_tbcC<T, LN><<<dim3((g.nx + 1 + L - 1) / L, 3, ndir), T_, smem_c<T>(g.ny), st>>>(R2, R1, p,
-                                                                                       tw);
-      return CAVITY_OK;
-    }
+    static std::atomic<bool> done{false};  // set once; host threads may race
+    CKS(smem_once(ctx, k_tbcC<T, LN>, done));
+    KScope ks_(ctx, kclass<T>(2));
+    k_tbcC<T, LN><<<dim3((g.nx + 1 + L - 1) / L, 3, ndir), T_, smem_c<T>(g.ny), st>>>(R2, R1, p, tw);
+    return CAVITY_OK;
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
@@ -920,7 +649,7 @@ cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, vo
   {
     KScope ks_(ctx, kclass<T>(4));
     k_combine<T><<<dim3((g.nx * g.ny + 255) / 256, ndir), 256, 0, st>>>(x, R2, Tabs<T>::top(ctx), y,
-                                                                       ystride, p);
+                                                                       ystride, g.ny + 1, p);
   }
   CK(cudaGetLastError());
   // truncated expansion: the rows of the dropped modes (the operator then
@@ -929,3 +658,8 @@ cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, vo
   return CAVITY_OK;
 }
 
+template <typename T>
+cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
+                           long long ystride) {
+  return launch_apply_generic<T>(ctx, ndir, x, y, work, ystride);
+}
