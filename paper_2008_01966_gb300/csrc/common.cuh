@@ -260,6 +260,21 @@ inline int smem_optin() {
   return v > 0 ? v : 48 * 1024;
 }
 
+// SMs of the current device
+inline int sm_count() {
+  static const int n = [] {
+    int dev = 0, v = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev);
+    return v > 0 ? v : 1;
+  }();
+  return n;
+}
+
+// threads per block of an elementwise kernel over n items: 256, or 64 where
+// that would leave SMs idle
+inline int elem_block(long long n) { return n >= 512LL * sm_count() ? 256 : 64; }
+
 // allow `func` the device's opt-in dynamic shared memory (minus its static part)
 template <typename F> inline cudaError_t allow_max_smem(F func) {
   cudaFuncAttributes a;

@@ -226,6 +226,9 @@ __device__ __forceinline__ void fft_pass(C<T>* line, int n, int s, int t, int tp
   constexpr int R = 1 << LR;
   const int Ns = 1 << s;
   const int nb = n >> LR;
+  // slot addresses are recomputed in each pass: carried over from one pass to
+  // the next they cost FP64 and pair lines more registers than there are
+  asm volatile("" : "+r"(t));
   C<T> v[PER * R];
   if (active) {
 #pragma unroll

@@ -7,11 +7,21 @@
 //   U1 = <cs_mn, G*u1>,  U2 = <sc_mn, G*u2>,  W = <cc_mn, G*w>,
 // u1 = sum E1 cs, u2 = sum E2 sc, w = div_Gamma(z x E) = sum (k2 pi/b) E1 cc -
 // sum (k1 pi/a) E2 cc (Sec. 5.1 reduces every coefficient to I1, I2, I3).
-// Each one is four passes of batched line transforms in shared memory:
-//   A  (rows k1)   basis transform along x2: FFT convolution of the mirrored
-//                  coefficients with the 1-D kernel E(nu) of F(F)
-//   B  (cols j2)   basis transform along x1, times F(G)/(Lx Ly), inverse DFT
-//                  along x1 evaluated at the nodes p = 0..Nx
+// E1 is a sine series in x2 and E2 one in x1: each vanishes on the two edges
+// across which w differentiates it, so the transform of the truncated w is
+// exactly
+//   F(w)(xi) = 2 pi i (xi2 F(E1)(xi) - xi1 F(E2)(xi)),
+// and only E1 and E2 take the basis transform: pass A does 2/3 and pass B 3/4
+// of the operations of three.  Both FP64 (two lanes per SM) and pair arithmetic
+// (6 to 25 FP32 instructions per operation) are bound by operations; operator
+// on one GB300, before and after: FP64 256 x 256, 6 vectors 6.43 -> 5.00 ms,
+// 512 x 512, 4 vectors 18.5 -> 14.2 ms, 1024 x 1024, 2 vectors 41.9 -> 32.0 ms;
+// pair, the same, 2.97 -> 2.34, 6.33 -> 5.07, 21.2 -> 17.2 ms.
+// Four passes of batched line transforms in shared memory:
+//   A  (rows k1)   basis transform of E1, E2 along x2: FFT convolution of the
+//                  mirrored coefficients with the 1-D kernel E(nu) of F(F)
+//   B  (cols j2)   basis transform along x1, w from it, all three fields times
+//                  F(G)/(Lx Ly), inverse DFT along x1 at the nodes p = 0..Nx
 //   C  (rows p)    inverse DFT along x2 at q = 0..Ny, trapezoid projection
 //                  onto cos/sin(n pi q/Ny) (an extended FFT of length 2Ny)
 //   D  (cols n)    trapezoid projection along x1 (extended FFT of length 2Nx)
@@ -63,6 +73,21 @@ template <typename T> __host__ __device__ constexpr int lines_per_cta(int nlong)
 template <typename T> __host__ __device__ constexpr int pairs_per_cta(int n) {
   return 2 * fft_tpl<T>(n) >= LINES_THREADS ? 1 : LINES_THREADS / (2 * fft_tpl<T>(n));
 }
+// These are the most lines of a CTA; a launch whose grid would not give every
+// SM two CTAs takes fewer (halved until it does, with the threads to match):
+// an SM has two FP64 lanes, so a 32 x 32 grid in 16 CTAs of eight columns used
+// a tenth of the machine (operator on one FP64 vector at 32 x 32: 125 us,
+// 164 us with full CTAs).  lL: log2 of the lines (or pairs) of a CTA.
+struct CtaLines {
+  int lL, threads;
+  unsigned blocks(int lines) const { return (unsigned)((lines + (1 << lL) - 1) >> lL); }
+};
+inline CtaLines cta_lines(int lL_max, int per_line, int tpl, long long lines, long long batch) {
+  const long long want = 2 * sm_count();
+  int lL = lL_max;
+  while (lL > 0 && ((lines + (1 << lL) - 1) >> lL) * batch < want) --lL;
+  return CtaLines{lL, std::min(LINES_THREADS, std::max(32, (per_line << lL) * tpl))};
+}
 // registers: the pass kernels run two CTAs of LINES_THREADS per SM (the
 // pair-of-FP32 ones spill ~450 bytes per thread at this bound, but one CTA per
 // SM without spills was slower: pass B 10.6 ms against 7.6 ms)
@@ -77,8 +102,8 @@ template <typename T> __host__ __device__ constexpr int pairs_per_cta(int n) {
 // Py = 4 ny.
 
 // ------------------------------------------------------------------ pass A
-// grid (ceil(nx / L) row groups, 3 fields, ndir); field 0: cs (E1), 1: sc (E2),
-// 2: cc (w).  Per row k1: the mirrored coefficient sequence along x2 (period
+// grid (ceil(nx / L) row groups, 2 fields, ndir); field 0: cs (E1), 1: sc (E2).
+// Per row k1: the mirrored coefficient sequence along x2 (period
 // Py) is transformed, multiplied by the transforms of the two parity kernels
 // eps_r and transformed back: the linear convolutions give the basis
 // transform at j2 = 2t + r of the symmetric box.  Lines: [parity][row].
@@ -93,17 +118,13 @@ struct GatherA {
   const C<T>* E1;
   const C<T>* E2;
   int row0, nx, f;
-  T pib, pia;                     // pi / b, pi / a
   __device__ __forceinline__ C<T> coef(int k1, int k2) const {
     constexpr int ny = 1 << LNY, N = ny - 1;
     C<T> c = czero<T>();
     if (f == 0) {
       if (k2 >= 1) c = E1[k1 * N + (k2 - 1)];
-    } else if (f == 1) {
-      if (k1 >= 1) c = E2[(k1 - 1) * ny + k2];
     } else {
-      if (k2 >= 1) c = cscale<T>(E1[k1 * N + (k2 - 1)], (T)k2 * pib);
-      if (k1 >= 1) c = csub<T>(c, cscale<T>(E2[(k1 - 1) * ny + k2], (T)k1 * pia));
+      if (k1 >= 1) c = E2[(k1 - 1) * ny + k2];
     }
     return c;
   }
@@ -156,15 +177,15 @@ struct ScatterA : LineId<T> {
 template <typename T, int LNY>
 __global__ void TBC_BOUNDS_LN(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __restrict__ Vy, TbcP p,
                                   const C<T>* __restrict__ tw, const C<T>* __restrict__ eh_c,
-                                  const C<T>* __restrict__ eh_s) {
+                                  const C<T>* __restrict__ eh_s, int lL_) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   C<T>* buf = (C<T>*)sm_raw;
   constexpr int LPY = LNY + 2, Py = 1 << LPY, ls = padded_len(Py);
-  constexpr int L = pairs_per_cta<T>(Py);
+  const int lL = pairs_per_cta<T>(Py) == 1 ? 0 : lL_, L = 1 << lL;
   const int f = blockIdx.y, d = blockIdx.z;
   const int row0 = blockIdx.x * L;
   ScatterA<T, LNY> sc;
-  sc.Vy = Vy + (size_t)(d * 3 + f) * p.nx * Py;
+  sc.Vy = Vy + (size_t)(d * 2 + f) * p.nx * Py;
   sc.row0 = row0;
   sc.nx = p.nx;
   sc.L = L;
@@ -174,8 +195,6 @@ __global__ void TBC_BOUNDS_LN(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __re
   fwd.row0 = row0;
   fwd.nx = p.nx;
   fwd.f = f;
-  fwd.pib = (T)p.pib;
-  fwd.pia = (T)p.pia;
   fwd.eh = f != 0 ? eh_c : eh_s;
   fwd.P = Py;
   fwd.L = L;
@@ -186,11 +205,13 @@ __global__ void TBC_BOUNDS_LN(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __re
 }
 
 // ------------------------------------------------------------------ pass B
-// grid (Py / L column groups, 3 fields, ndir).  Per column j2: the basis
-// transform along x1 split by the parity of j1 = 2t + r (as in pass A), times
-// F(G)(|j1|, |j2|)/(Lx Ly), then the inverse torus transform along x1 at the
-// nodes p = 0..nx:  sum_j1 Y(j1) e^{2 pi i j1 p/Px} = Z_0(p) + e^{2 pi i p/Px} Z_1(p),
-// Z_r = inverse transform of length Px/2 of Y(2t + r) over t.
+// grid (Py / L column groups, ndir).  Per column j2 and field E1, E2: the
+// basis transform along x1 split by the parity of j1 = 2t + r (as in pass A),
+// times F(G)(|j1|, |j2|)/(Lx Ly), then the inverse torus transform along x1 at
+// the nodes p = 0..nx:  sum_j1 Y(j1) e^{2 pi i j1 p/Px} = Z_0(p) + e^{2 pi i p/Px} Z_1(p),
+// Z_r = inverse transform of length Px/2 of Y(2t + r) over t.  The products of
+// w are gathered on the way (j2 / Ly times those of E1 minus j1 / Lx times
+// those of E2) in two half-length lines, which take the same last transform.
 // Fused: the parity products (last write of the forward transform), the
 // kernel-table products with the move of t to slot t mod Px/2 (last write of
 // the first inverse transforms).  The column gather stays a cooperative pass:
@@ -198,13 +219,15 @@ __global__ void TBC_BOUNDS_LN(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __re
 
 // last write of the first inverse transforms of pass B: output t (k = t mod
 // Px) of line (r, l), |t| < Px/4, times the kernel table at (|2t + r|, |j2|),
-// written to slot t mod Px/2 (other outputs are not needed)
+// written to slot t mod Px/2 (other outputs are not needed), and into w
 // STAGED: kh holds the rows of the block's columns in shared memory,
 // [l][j1 < Px/2]; else kh is the whole quarter box in global memory, [j2][j1]
-template <typename T, int LNX, bool STAGED = true>
+template <typename T, int LNX, int F, bool STAGED>
 struct KhatB : LineId<T> {
   const C<T>* kh;
+  C<T>* wl;                       // w: half-length lines [r][l]
   int j0, Py, L;
+  T scale;                        // 2 pi / Ly (field 0), 2 pi / Lx (field 1)
   __device__ __forceinline__ void st(int lr, C<T>* line, int k, C<T> v) const {
     constexpr int Px = 4 << LNX, hp = Px / 2, qp = Px / 4;
     int t, u;
@@ -213,116 +236,236 @@ struct KhatB : LineId<T> {
     else return;
     const int r = lr >= L ? 1 : 0, l = lr - r * L;
     const int j = j0 + l;
-    const int j1 = 2 * t + r;
+    const int j1 = 2 * t + r, j2 = j < Py / 2 ? j : j - Py;
     C<T> o = czero<T>();
     if (j1 != -hp && j < Py && j != Py / 2) {
       const int j1a = j1 < 0 ? -j1 : j1;
       if constexpr (STAGED) {
         o = cmul<T>(v, kh[l * hp + j1a]);
       } else {
-        const int j2a = j < Py / 2 ? j : Py - j;
+        const int j2a = j2 < 0 ? -j2 : j2;
         o = cmul<T>(v, kh[(size_t)j2a * hp + j1a]);
       }
     }
     line[pidx(u)] = o;
+    C<T>* w = wl + (size_t)lr * padded_len(hp) + pidx(u);
+    if (F == 0) *w = cscale<T>(o, (T)j2 * scale);
+    else *w = csub<T>(*w, cscale<T>(o, (T)j1 * scale));
   }
 };
 
 // pass B stages the two parity kernels and the kernel-table rows of its
 // columns in shared memory when lines and tables together take at most
-// 100 KB (every FP32 grid; 16-byte types up to 256 points per side); else it
+// 100 KB (16-byte types up to 256 points per side); else it
 // reads them from global memory (they stay in L2), which leaves room for more
 // CTAs per SM: at 512 points per side the pair-of-FP32 pass B of the
 // four-layer 512^2 benchmark step went from 16.2 to 9.4 ms (one CTA per SM
-// with the 156 KB of staging, two without), and it is the only way at 1024
-template <typename T> __host__ __device__ constexpr size_t smem_b_lines(int nx) {
-  return sizeof(C<T>) * 2 * (size_t)pairs_per_cta<T>(4 * nx) * (size_t)padded_len(4 * nx);
+// with the staging, two without), and it is the only way at 1024
+template <typename T> __host__ __device__ constexpr size_t smem_b_lines(int nx, int lL) {
+  return sizeof(C<T>) * ((size_t)2 << lL) * (size_t)(padded_len(4 * nx) + padded_len(2 * nx));
 }
-template <typename T> __host__ __device__ constexpr size_t smem_b_tables(int nx) {
-  return sizeof(C<T>) * (2 * 4 * (size_t)nx + (size_t)pairs_per_cta<T>(4 * nx) * 2 * (size_t)nx);
+template <typename T> __host__ __device__ constexpr size_t smem_b_tables(int nx, int lL) {
+  return sizeof(C<T>) * (2 * 4 * (size_t)nx + ((size_t)2 << lL) * nx);
 }
 template <typename T> __host__ __device__ constexpr bool b_staged(int nx) {
-  return smem_b_lines<T>(nx) + smem_b_tables<T>(nx) <= 100 * 1024;
+  return smem_b_lines<T>(nx, clog2(pairs_per_cta<T>(4 * nx))) +
+             smem_b_tables<T>(nx, clog2(pairs_per_cta<T>(4 * nx))) <= 100 * 1024;
+}
+
+// shared memory of pass B: 2L lines, 2L half-length lines of w, then (STAGE)
+// the two parity kernels [2][Px] and the kernel-table rows |j2| of the L
+// columns [L][Px/2], so that the fused products read shared memory instead of
+// waiting on loads
+template <typename T, int LNX> struct BShape {
+  static constexpr int LPX = LNX + 2, Px = 1 << LPX, nx = 1 << LNX;
+  static constexpr int ls = padded_len(Px), lsh = padded_len(Px / 2);
+  static constexpr bool STAGE = b_staged<T>(nx);
+};
+
+// Z_0 + e^{2 pi i q / Px} Z_1 of the lines at z (stride zs), into W's rows;
+// w carries the factor i (TIMES_I)
+template <typename T, int LNX, bool TIMES_I>
+__device__ __forceinline__ void b_store(const C<T>* z, int zs, C<T>* __restrict__ dst, int j0,
+                                        int Py, const C<T>* __restrict__ tw, int sh, int lL) {
+  using S = BShape<T, LNX>;
+  const int L = 1 << lL;
+  for (int idx = threadIdx.x; idx < L * (S::nx + 1); idx += blockDim.x) {
+    const int q = idx >> lL, l = idx & (L - 1);
+    const int j = j0 + l;
+    if (j >= Py) continue;
+    const C<T> z0 = z[(size_t)l * zs + pidx(q)];
+    const C<T> z1 = z[(size_t)(L + l) * zs + pidx(q)];
+    const C<T> o = cadd<T>(z0, cmul<T>(z1, twid<T, true>(tw, q << sh)));
+    dst[(size_t)q * Py + j] = TIMES_I ? cmul_i<T>(o) : o;
+  }
+}
+
+// Field F of pass B.  The field is a template argument: with a loop over the
+// two fields the compiler spilled 2-4 KB per thread.
+template <typename T, int LNX, int F>
+__device__ __forceinline__ void b_field(const C<T>* __restrict__ src, C<T>* __restrict__ dst,
+                                     const C<T>* __restrict__ tw, const C<T>* __restrict__ eh,
+                                     const C<T>* __restrict__ kh, int j0, int Py,
+                                     int twlog, T scale, int lL) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  using S = BShape<T, LNX>;
+  constexpr int LPX = S::LPX, Px = S::Px, nx = S::nx, ls = S::ls;
+  const int L = 1 << lL;
+  C<T>* buf = (C<T>*)sm_raw;
+  C<T>* wl = buf + (size_t)2 * L * ls;
+  C<T>* eh_sm = wl + (size_t)2 * L * S::lsh;
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  constexpr bool xcos = F == 0;
+  if constexpr (S::STAGE) {
+    for (int t = tid; t < 2 * Px; t += nthr) eh_sm[t] = eh[t];
+  }
+  // cooperative, coalesced gather of the L columns (consecutive threads take
+  // consecutive columns of a row); the mirrored lines cover every slot but
+  // [nx, Px - nx], which is cleared
+#pragma unroll 4
+  for (int idx = tid; idx < L * nx; idx += nthr) {
+    const int k1 = idx >> lL, l = idx & (L - 1);
+    const int j = j0 + l;
+    const C<T> c = j < Py ? src[(size_t)k1 * Py + j] : czero<T>();
+    const C<T> c0 = k1 == 0 ? (xcos ? cscale<T>(c, (T)2) : czero<T>()) : c;
+    const C<T> cm = xcos ? c : mk<T>(-c.x, -c.y);
+    C<T>* line = buf + (size_t)l * ls;
+    line[pidx(k1)] = c0;
+    if (k1 > 0) line[pidx(Px - k1)] = cm;
+  }
+  for (int idx = tid; idx < L * (2 * nx + 1); idx += nthr) {
+    const int l = idx / (2 * nx + 1), k = nx + idx - l * (2 * nx + 1);
+    buf[(size_t)l * ls + pidx(k)] = czero<T>();
+  }
+  __syncthreads();
+  ParityProducts<T, LineId<T>> fwd;
+  fwd.eh = S::STAGE ? eh_sm : eh;
+  fwd.P = Px;
+  fwd.L = L;
+  fwd.ls = ls;
+  fwd.buf = buf;
+  fft_lines<T, false, LPX>(buf, ls, L, tw, twlog, fwd);
+  KhatB<T, LNX, F, S::STAGE> kb;
+  kb.kh = S::STAGE ? eh_sm + 2 * Px : kh;
+  kb.wl = wl;
+  kb.j0 = j0;
+  kb.Py = Py;
+  kb.L = L;
+  kb.scale = scale;
+  fft_lines<T, true, LPX>(buf, ls, 2 * L, tw, twlog, kb);
+  fft_lines<T, true, LPX - 1>(buf, ls, 2 * L, tw, twlog);
+  b_store<T, LNX, false>(buf, ls, dst, j0, Py, tw, twlog - LPX, lL);
+  __syncthreads();
 }
 
 template <typename T, int LNX>
 __global__ void TBC_BOUNDS_LN(LNX) k_tbcB(const C<T>* __restrict__ Vy, C<T>* __restrict__ W, TbcP p,
                                   const C<T>* __restrict__ tw, const C<T>* __restrict__ eh_c,
-                                  const C<T>* __restrict__ eh_s, const C<T>* __restrict__ kh) {
+                                  const C<T>* __restrict__ eh_s, const C<T>* __restrict__ kh,
+                                  T ax, T ay, int lL_) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
-  C<T>* buf = (C<T>*)sm_raw;
-  constexpr int LPX = LNX + 2, Px = 1 << LPX, nx = 1 << LNX, ls = padded_len(Px);
-  constexpr int L = pairs_per_cta<T>(Px), lL = clog2(L);
-  const int Py = p.Py;
-  const int f = blockIdx.y, d = blockIdx.z;
-  const int j0 = blockIdx.x * L;
-  const int tid = threadIdx.x, nthr = blockDim.x;
-  const bool xcos = (f != 1);
-  // shared memory: 2L lines, then the two parity kernels [2][Px], then the
-  // kernel-table rows |j2| of the L columns [L][Px/2] (staged once per block,
-  // so the fused products read shared memory instead of waiting on loads)
-  constexpr bool STAGE = b_staged<T>(nx);
-  C<T>* eh_sm = buf + (size_t)2 * L * ls;
-  C<T>* kh_sm = eh_sm + 2 * Px;
-  const C<T>* eh_use = xcos ? eh_c : eh_s;
-  if constexpr (STAGE) {
-    const C<T>* eh = xcos ? eh_c : eh_s;
-    for (int t = tid; t < 2 * Px; t += nthr) eh_sm[t] = eh[t];
-    for (int idx = tid; idx < L * (Px / 2); idx += nthr) {
+  using S = BShape<T, LNX>;
+  constexpr int LPX = S::LPX, Px = S::Px, nx = S::nx;
+  const int lL = pairs_per_cta<T>(Px) == 1 ? 0 : lL_, L = 1 << lL;
+  C<T>* wl = (C<T>*)sm_raw + (size_t)2 * L * S::ls;
+  const int Py = p.Py, d = blockIdx.y, j0 = blockIdx.x * L;
+  if constexpr (S::STAGE) {
+    C<T>* kh_sm = wl + (size_t)2 * L * S::lsh + 2 * Px;
+    for (int idx = threadIdx.x; idx < L * (Px / 2); idx += blockDim.x) {
       const int l = idx >> (LPX - 1), j1 = idx & (Px / 2 - 1);
       const int j = j0 + l;
       const int j2a = j < Py / 2 ? j : Py - j;
       kh_sm[idx] = (j < Py && j != Py / 2) ? kh[(size_t)j2a * (Px / 2) + j1] : czero<T>();
     }
-    eh_use = eh_sm;
   }
-  // cooperative, coalesced gather of the L columns (consecutive threads take
-  // consecutive columns of a row); the mirrored lines cover every slot but
-  // [nx, Px - nx], which is cleared
-  {
-    const C<T>* src = Vy + (size_t)(d * 3 + f) * nx * Py;
-#pragma unroll 4
-    for (int idx = tid; idx < L * nx; idx += nthr) {
-      const int k1 = idx >> lL, l = idx & (L - 1);
-      const int j = j0 + l;
-      const C<T> c = j < Py ? src[(size_t)k1 * Py + j] : czero<T>();
-      const C<T> c0 = k1 == 0 ? (xcos ? cscale<T>(c, (T)2) : czero<T>()) : c;
-      const C<T> cm = xcos ? c : mk<T>(-c.x, -c.y);
-      C<T>* line = buf + (size_t)l * ls;
-      line[pidx(k1)] = c0;
-      if (k1 > 0) line[pidx(Px - k1)] = cm;
-    }
-    for (int idx = tid; idx < L * (2 * nx + 1); idx += nthr) {
-      const int l = idx / (2 * nx + 1), k = nx + idx - l * (2 * nx + 1);
-      buf[(size_t)l * ls + pidx(k)] = czero<T>();
-    }
-    __syncthreads();
+  const C<T>* src = Vy + (size_t)d * 2 * nx * Py;
+  const size_t fs = (size_t)(nx + 1) * Py;
+  C<T>* dst = W + (size_t)d * 3 * fs;
+  b_field<T, LNX, 0>(src, dst, tw, eh_c, kh, j0, Py, p.twlog, ay, lL);
+  b_field<T, LNX, 1>(src + (size_t)nx * Py, dst + fs, tw, eh_s, kh, j0, Py, p.twlog, ax, lL);
+  fft_lines<T, true, LPX - 1>(wl, S::lsh, 2 * L, tw, p.twlog);
+  b_store<T, LNX, true>(wl, S::lsh, dst + 2 * fs, j0, Py, tw, p.twlog - LPX, lL);
+}
+
+// Pass B for small launches (fewer columns than keep the machine busy): one
+// column per CTA with both fields' lines, and those of w, side by side, so a
+// CTA goes through three transforms instead of seven.  Lines (stride ls):
+// (field f, parity r) at 2 f + r, w at 4 + r.  One FP64 vector at 32 x 32:
+// 62 us with k_tbcB, 28 us.
+template <typename T, int LNX>
+struct ProdsB1 : LineId<T> {     // parity products of both fields' spectra
+  const C<T>* eh_c;
+  const C<T>* eh_s;
+  __device__ __forceinline__ void st(int f, C<T>* line, int k, C<T> v) const {
+    constexpr int Px = 4 << LNX, ls = padded_len(Px);
+    const C<T>* eh = f == 0 ? eh_c : eh_s;
+    line[pidx(k)] = cmul<T>(v, eh[k]);
+    line[ls + pidx(k)] = cmul<T>(v, eh[Px + k]);
   }
-  KhatB<T, LNX, STAGE> kb;
-  kb.kh = STAGE ? kh_sm : kh;
-  kb.j0 = j0;
-  kb.Py = Py;
-  kb.L = L;
-  ParityProducts<T, LineId<T>> fwd;
-  fwd.eh = eh_use;
-  fwd.P = Px;
-  fwd.L = L;
-  fwd.ls = ls;
-  fwd.buf = buf;
-  fft_lines<T, false, LPX>(buf, ls, L, tw, p.twlog, fwd);
-  fft_lines<T, true, LPX>(buf, ls, 2 * L, tw, p.twlog, kb);
-  fft_lines<T, true, LPX - 1>(buf, ls, 2 * L, tw, p.twlog);
-  C<T>* dst = W + (size_t)(d * 3 + f) * (nx + 1) * Py;
-  const int sh = p.twlog - LPX;
-  for (int idx = tid; idx < L * (nx + 1); idx += nthr) {
-    const int q = idx >> lL, l = idx & (L - 1);
-    const int j = j0 + l;
-    if (j >= Py) continue;
-    const C<T> z0 = buf[(size_t)l * ls + pidx(q)];
-    const C<T> z1 = buf[(size_t)(L + l) * ls + pidx(q)];
-    dst[(size_t)q * Py + j] = cadd<T>(z0, cmul<T>(z1, twid<T, true>(tw, q << sh)));
+};
+template <typename T, int LNX>
+struct KhatB1 : LineId<T> {      // table products; the result stays in slot t mod Px/2
+  const C<T>* kh;                // row |j2|
+  bool dead;
+  __device__ __forceinline__ void st(int lr, C<T>* line, int k, C<T> v) const {
+    constexpr int Px = 4 << LNX, hp = Px / 2, qp = Px / 4;
+    int t, u;
+    if (k < qp) { t = k; u = k; }
+    else if (k >= Px - qp) { t = k - Px; u = k - hp; }
+    else return;
+    const int j1 = 2 * t + (lr & 1);
+    line[pidx(u)] = (j1 == -hp || dead) ? czero<T>() : cmul<T>(v, kh[j1 < 0 ? -j1 : j1]);
+  }
+};
+template <typename T, int LNX>
+__global__ void TBC_BOUNDS k_tbcB1(const C<T>* __restrict__ Vy, C<T>* __restrict__ W, TbcP p,
+                                   const C<T>* __restrict__ tw, const C<T>* __restrict__ eh_c,
+                                   const C<T>* __restrict__ eh_s, const C<T>* __restrict__ kh,
+                                   T ax, T ay) {
+  extern __shared__ __align__(16) unsigned char sm_raw[];
+  C<T>* buf = (C<T>*)sm_raw;
+  using S = BShape<T, LNX>;
+  constexpr int LPX = S::LPX, Px = S::Px, nx = S::nx, ls = S::ls;
+  const int Py = p.Py, d = blockIdx.y, j = blockIdx.x, tid = threadIdx.x, nthr = blockDim.x;
+  const int j2 = j < Py / 2 ? j : j - Py;
+  const bool dead = j == Py / 2;
+  for (int idx = tid; idx < 2 * Px; idx += nthr) {
+    const int f = idx / Px, k = idx % Px;
+    const int k1 = k < nx ? k : Px - k;     // mirrored
+    C<T> c = czero<T>();
+    if (k1 < nx && (f == 0 || k1 > 0)) c = Vy[((size_t)(d * 2 + f) * nx + k1) * Py + j];
+    if (k == 0) c = cscale<T>(c, (T)2);
+    if (f == 1 && k > nx) c = mk<T>(-c.x, -c.y);
+    buf[(size_t)(2 * f) * ls + pidx(k)] = c;
+  }
+  __syncthreads();
+  ProdsB1<T, LNX> fwd;
+  fwd.eh_c = eh_c;
+  fwd.eh_s = eh_s;
+  fft_lines<T, false, LPX>(buf, 2 * ls, 2, tw, p.twlog, fwd);
+  KhatB1<T, LNX> kb;
+  kb.kh = kh + (size_t)(dead ? 0 : (j2 < 0 ? -j2 : j2)) * (Px / 2);
+  kb.dead = dead;
+  fft_lines<T, true, LPX>(buf, ls, 4, tw, p.twlog, kb);
+  for (int idx = tid; idx < Px; idx += nthr) {
+    const int r = idx / (Px / 2), u = idx % (Px / 2);
+    const int j1 = 2 * (u < nx ? u : u - Px / 2) + r;
+    const C<T> g0 = buf[(size_t)r * ls + pidx(u)], g1 = buf[(size_t)(2 + r) * ls + pidx(u)];
+    buf[(size_t)(4 + r) * ls + pidx(u)] =
+        csub<T>(cscale<T>(g0, (T)j2 * ay), cscale<T>(g1, (T)j1 * ax));
+  }
+  __syncthreads();
+  fft_lines<T, true, LPX - 1>(buf, ls, 6, tw, p.twlog);
+  for (int idx = tid; idx < 3 * (nx + 1); idx += nthr) {
+    const int f = idx / (nx + 1), q = idx % (nx + 1);
+    const C<T> z0 = buf[(size_t)(2 * f) * ls + pidx(q)], z1 = buf[(size_t)(2 * f + 1) * ls + pidx(q)];
+    const C<T> o = cadd<T>(z0, cmul<T>(z1, twid<T, true>(tw, q << (p.twlog - LPX))));
+    W[((size_t)(d * 3 + f) * (nx + 1) + q) * Py + j] = f == 2 ? cmul_i<T>(o) : o;
   }
 }
+// sizes it is built for, and launches small enough for it
+template <typename T> __host__ __device__ constexpr bool b1_ok(int ln) { return sizeof(C<T>) == 16 && ln <= 7; }
+inline bool b1_use(int Py, int ndir) { return (long long)Py * ndir <= 4LL * sm_count(); }
 
 // ------------------------------------------------------------------ pass C
 // grid (ceil((nx+1)/L) row groups, 3 fields, ndir).  Per node row p: inverse
@@ -369,11 +512,11 @@ struct StoreZ : LineId<T> {
 
 template <typename T, int LNY>
 __global__ void TBC_BOUNDS_LN(LNY) k_tbcC(const C<T>* __restrict__ W, C<T>* __restrict__ Z, TbcP p,
-                                  const C<T>* __restrict__ tw) {
+                                  const C<T>* __restrict__ tw, int lL_) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   C<T>* buf = (C<T>*)sm_raw;
   constexpr int LPY = LNY + 2, Py = 1 << LPY, ny = 1 << LNY, ls = padded_len(Py);
-  constexpr int L = lines_per_cta<T>(Py);
+  const int L = lines_per_cta<T>(Py) == 1 ? 1 : 1 << lL_;
   const int f = blockIdx.y, d = blockIdx.z;
   const int r0 = blockIdx.x * L;
   const bool ycos = (f != 0);
@@ -425,11 +568,11 @@ struct ColD {
 
 template <typename T, int LNX>
 __global__ void TBC_BOUNDS_LN(LNX) k_tbcD(const C<T>* __restrict__ Z, C<T>* __restrict__ O, TbcP p,
-                                  const C<T>* __restrict__ tw) {
+                                  const C<T>* __restrict__ tw, int lL_) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
   C<T>* buf = (C<T>*)sm_raw;
   constexpr int nx = 1 << LNX, n2 = 2 * nx, ls = padded_len(n2);
-  constexpr int L = lines_per_cta<T>(n2);
+  const int L = lines_per_cta<T>(n2) == 1 ? 1 : 1 << lL_;
   const int f = blockIdx.y, d = blockIdx.z;
   ColD<T, LNX> cd;
   cd.src = Z + (size_t)(d * 3 + f) * (nx + 1) * (p.ny + 1);
@@ -496,14 +639,18 @@ __global__ void k_combine(const C<T>* __restrict__ x, const C<T>* __restrict__ O
 // Explicit instantiation (EXT empty) or its declaration (EXT = extern) of the
 // four pass kernels of type T at log2 size LN; lets a type's instantiations
 // be compiled in several translation units (in parallel) while one unit
-// launches them.
+// launches them (TBC_B1_KERNEL: sizes of b1_ok).
+#define TBC_B1_KERNEL(EXT, T, LN)                                                             \
+  EXT template __global__ void k_tbcB1<T, LN>(const C<T>*, C<T>*, TbcP, const C<T>*,          \
+                                              const C<T>*, const C<T>*, const C<T>*, T, T);
 #define TBC_PASS_KERNELS(EXT, T, LN)                                                          \
   EXT template __global__ void k_tbcA<T, LN>(const C<T>*, C<T>*, TbcP, const C<T>*,           \
-                                             const C<T>*, const C<T>*);                       \
+                                             const C<T>*, const C<T>*, int);                  \
   EXT template __global__ void k_tbcB<T, LN>(const C<T>*, C<T>*, TbcP, const C<T>*,           \
-                                             const C<T>*, const C<T>*, const C<T>*);          \
-  EXT template __global__ void k_tbcC<T, LN>(const C<T>*, C<T>*, TbcP, const C<T>*);          \
-  EXT template __global__ void k_tbcD<T, LN>(const C<T>*, C<T>*, TbcP, const C<T>*);
+                                             const C<T>*, const C<T>*, const C<T>*, T, T,     \
+                                             int);                                            \
+  EXT template __global__ void k_tbcC<T, LN>(const C<T>*, C<T>*, TbcP, const C<T>*, int);     \
+  EXT template __global__ void k_tbcD<T, LN>(const C<T>*, C<T>*, TbcP, const C<T>*, int);
 
 template <typename T> struct Tabs;
 template <> struct Tabs<double> {
@@ -521,13 +668,19 @@ template <> struct Tabs<float> {
   static const float2* top(cavity_ctx* c) { return c->top32; }
 };
 
-// shared memory of each pass (bytes) for the grid sizes of g
-template <typename T> static size_t smem_a(int ny) { return sizeof(C<T>) * 2 * pairs_per_cta<T>(4 * ny) * (size_t)padded_len(4 * ny); }
-template <typename T> static size_t smem_b(int nx) {
-  return smem_b_lines<T>(nx) + (b_staged<T>(nx) ? smem_b_tables<T>(nx) : 0);
+// shared memory of each pass (bytes) at 2^lL lines (or pairs) per CTA
+template <typename T> static size_t smem_a(int ny, int lL) {
+  return sizeof(C<T>) * ((size_t)2 << lL) * padded_len(4 * ny);
 }
-template <typename T> static size_t smem_c(int ny) { return sizeof(C<T>) * lines_per_cta<T>(4 * ny) * (size_t)padded_len(4 * ny); }
-template <typename T> static size_t smem_d(int nx) { return sizeof(C<T>) * lines_per_cta<T>(2 * nx) * (size_t)padded_len(2 * nx); }
+template <typename T> static size_t smem_b(int nx, int lL) {
+  return smem_b_lines<T>(nx, lL) + (b_staged<T>(nx) ? smem_b_tables<T>(nx, lL) : 0);
+}
+template <typename T> static size_t smem_c(int ny, int lL) {
+  return sizeof(C<T>) * ((size_t)1 << lL) * padded_len(4 * ny);
+}
+template <typename T> static size_t smem_d(int nx, int lL) {
+  return sizeof(C<T>) * ((size_t)1 << lL) * padded_len(2 * nx);
+}
 
 // opt every instantiation of kernel K into the device's shared-memory maximum
 // once per process
@@ -594,62 +747,84 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
   }
   if (ystride < 0) ystride = ctx->g.nap;
   const Geo& g = ctx->g;
-  const size_t need = std::max(std::max(smem_a<T>(g.ny), smem_b<T>(g.nx)),
-                               std::max(smem_c<T>(g.ny), smem_d<T>(g.nx)));
+  const int pl = clog2(pairs_per_cta<T>(4 * g.ny)), pb = clog2(pairs_per_cta<T>(4 * g.nx));
+  const size_t need = std::max(
+      std::max(smem_a<T>(g.ny, pl), smem_b<T>(g.nx, pb)),
+      std::max(smem_c<T>(g.ny, clog2(lines_per_cta<T>(4 * g.ny))),
+               smem_d<T>(g.nx, clog2(lines_per_cta<T>(2 * g.nx)))));
   if (need > (size_t)smem_optin()) {
     ctx->err = "grid too large for the shared-memory transforms";
     return CAVITY_EINVAL;
   }
   TbcP p = make_params(ctx);
-  size_t vy = (size_t)ndir * 3 * g.nx * g.Py;
+  size_t vy = (size_t)ndir * 2 * g.nx * g.Py;
   size_t z = (size_t)ndir * 3 * (g.nx + 1) * (g.ny + 1);
   C<T>* R1 = (C<T>*)work;                      // Vy, later Z
   C<T>* R2 = R1 + std::max(vy, z);             // W, later O
   cudaStream_t st = ctx->stream;
   const C<T>* tw = Tabs<T>::tw(ctx);
-  const int T_ = LINES_THREADS;
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    constexpr int L = pairs_per_cta<T>(4 << LN);
+    const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN), g.nx,
+                                  2LL * ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcA<T, LN>, done));
     KScope ks_(ctx, kclass<T>(0));
-    k_tbcA<T, LN><<<dim3((g.nx + L - 1) / L, 3, ndir), T_, smem_a<T>(g.ny), st>>>(
-        x, R1, p, tw, Tabs<T>::ey(ctx, 0), Tabs<T>::ey(ctx, 1));
+    k_tbcA<T, LN><<<dim3(cl.blocks(g.nx), 2, ndir), cl.threads, smem_a<T>(g.ny, cl.lL), st>>>(
+        x, R1, p, tw, Tabs<T>::ey(ctx, 0), Tabs<T>::ey(ctx, 1), cl.lL);
     return CAVITY_OK;
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    constexpr int L = pairs_per_cta<T>(4 << LN);
+    if constexpr (b1_ok<T>(LN)) {
+      if (b1_use(g.Py, ndir)) {
+        static std::atomic<bool> done1{false};
+        CKS(smem_once(ctx, k_tbcB1<T, LN>, done1));
+        KScope ks_(ctx, kclass<T>(1));
+        k_tbcB1<T, LN><<<dim3(g.Py, ndir), std::max(64, std::min(LINES_THREADS, 6 * fft_tpl<T>(4 << LN))),
+                         sizeof(C<T>) * 6 * (size_t)padded_len(4 << LN), st>>>(
+            R1, R2, p, tw, Tabs<T>::ex(ctx, 0), Tabs<T>::ex(ctx, 1), Tabs<T>::kh(ctx),
+            T(2.0 * M_PI / g.Lx), T(2.0 * M_PI / g.Ly));
+        return CAVITY_OK;
+      }
+    }
+    const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN), g.Py,
+                                  ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcB<T, LN>, done));
     KScope ks_(ctx, kclass<T>(1));
-    k_tbcB<T, LN><<<dim3((g.Py + L - 1) / L, 3, ndir), T_, smem_b<T>(g.nx), st>>>(
-        R1, R2, p, tw, Tabs<T>::ex(ctx, 0), Tabs<T>::ex(ctx, 1), Tabs<T>::kh(ctx));
+    k_tbcB<T, LN><<<dim3(cl.blocks(g.Py), ndir), cl.threads, smem_b<T>(g.nx, cl.lL), st>>>(
+        R1, R2, p, tw, Tabs<T>::ex(ctx, 0), Tabs<T>::ex(ctx, 1), Tabs<T>::kh(ctx),
+        T(2.0 * M_PI / g.Lx), T(2.0 * M_PI / g.Ly), cl.lL);
     return CAVITY_OK;
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    constexpr int L = lines_per_cta<T>(4 << LN);
+    const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(4 << LN)), 1, fft_tpl<T>(4 << LN), g.nx + 1,
+                                  3LL * ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcC<T, LN>, done));
     KScope ks_(ctx, kclass<T>(2));
-    k_tbcC<T, LN><<<dim3((g.nx + 1 + L - 1) / L, 3, ndir), T_, smem_c<T>(g.ny), st>>>(R2, R1, p, tw);
+    k_tbcC<T, LN><<<dim3(cl.blocks(g.nx + 1), 3, ndir), cl.threads, smem_c<T>(g.ny, cl.lL), st>>>(
+        R2, R1, p, tw, cl.lL);
     return CAVITY_OK;
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    constexpr int L = lines_per_cta<T>(2 << LN);
+    const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(2 << LN)), 1, fft_tpl<T>(2 << LN), g.ny + 1,
+                                  3LL * ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcD<T, LN>, done));
     KScope ks_(ctx, kclass<T>(3));
-    k_tbcD<T, LN><<<dim3((g.ny + 1 + L - 1) / L, 3, ndir), T_, smem_d<T>(g.nx), st>>>(R1, R2, p, tw);
+    k_tbcD<T, LN><<<dim3(cl.blocks(g.ny + 1), 3, ndir), cl.threads, smem_d<T>(g.nx, cl.lL), st>>>(
+        R1, R2, p, tw, cl.lL);
     return CAVITY_OK;
   }));
   {
     KScope ks_(ctx, kclass<T>(4));
-    k_combine<T><<<dim3((g.nx * g.ny + 255) / 256, ndir), 256, 0, st>>>(x, R2, Tabs<T>::top(ctx), y,
-                                                                       ystride, g.ny + 1, p);
+    const int eb = elem_block((long long)g.nx * g.ny * ndir);
+    k_combine<T><<<dim3((g.nx * g.ny + eb - 1) / eb, ndir), eb, 0, st>>>(x, R2, Tabs<T>::top(ctx), y,
+                                                                         ystride, g.ny + 1, p);
   }
   CK(cudaGetLastError());
   // truncated expansion: the rows of the dropped modes (the operator then

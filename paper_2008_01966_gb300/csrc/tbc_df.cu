@@ -16,11 +16,17 @@ template <> struct Tabs<df> {
 // the pass kernels of the pair type are compiled in tbc_df_k*.cu (in
 // parallel: one unit with all sizes took three minutes)
 TBC_PASS_KERNELS(extern, df, 2)
+TBC_B1_KERNEL(extern, df, 2)
 TBC_PASS_KERNELS(extern, df, 3)
+TBC_B1_KERNEL(extern, df, 3)
 TBC_PASS_KERNELS(extern, df, 4)
+TBC_B1_KERNEL(extern, df, 4)
 TBC_PASS_KERNELS(extern, df, 5)
+TBC_B1_KERNEL(extern, df, 5)
 TBC_PASS_KERNELS(extern, df, 6)
+TBC_B1_KERNEL(extern, df, 6)
 TBC_PASS_KERNELS(extern, df, 7)
+TBC_B1_KERNEL(extern, df, 7)
 TBC_PASS_KERNELS(extern, df, 8)
 TBC_PASS_KERNELS(extern, df, 9)
 TBC_PASS_KERNELS(extern, df, 10)

@@ -4,5 +4,8 @@
 #include "tbc_apply.cuh"
 
 TBC_PASS_KERNELS(, df, 2)
+TBC_B1_KERNEL(, df, 2)
 TBC_PASS_KERNELS(, df, 3)
+TBC_B1_KERNEL(, df, 3)
 TBC_PASS_KERNELS(, df, 4)
+TBC_B1_KERNEL(, df, 4)

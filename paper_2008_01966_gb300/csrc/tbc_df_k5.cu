@@ -4,4 +4,6 @@
 #include "tbc_apply.cuh"
 
 TBC_PASS_KERNELS(, df, 5)
+TBC_B1_KERNEL(, df, 5)
 TBC_PASS_KERNELS(, df, 6)
+TBC_B1_KERNEL(, df, 6)

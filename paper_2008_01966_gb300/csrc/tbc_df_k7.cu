@@ -4,4 +4,5 @@
 #include "tbc_apply.cuh"
 
 TBC_PASS_KERNELS(, df, 7)
+TBC_B1_KERNEL(, df, 7)
 TBC_PASS_KERNELS(, df, 8)
