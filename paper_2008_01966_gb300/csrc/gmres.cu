@@ -65,49 +65,60 @@ __global__ void __launch_bounds__(256) k_dots(const C<T>* __restrict__ V, long l
 
 // Multi-dot V^H w in two fixed-order stages: each block keeps one chunk of w
 // in shared memory and forms the partial dots of that chunk with all cnt basis
-// vectors; a second kernel adds the chunk partials in chunk order.
+// vectors (blockIdx.z takes MDOT_VECS of them); a second kernel adds the chunk
+// partials in chunk order.  The chunk depends on n_ap alone (mdot_chunk), so a
+// direction's sums do not depend on the batch.  FP64 work is scarce per SM (two
+// lanes), so a short vector is cut into pieces for as many SMs as it can feed:
+// up to 24 vectors of 3,007 entries took 40 us in two blocks, now 6.4 us in 24
+// to 72.
 #define MDOT_CHUNK 2048
+#define MDOT_VECS 8
 template <typename T>
 __global__ void __launch_bounds__(256) k_mdot_partial(const C<T>* __restrict__ V, long long vs,
                                                       const C<T>* __restrict__ w, long long ws,
                                                       double2* __restrict__ part, int cnt, int nap,
-                                                      int nchunk, const int* __restrict__ flag) {
+                                                      int chunk, int nchunk,
+                                                      const int* __restrict__ flag) {
   __shared__ C<T> sw[MDOT_CHUNK];
   __shared__ double rr[8], ri[8];
   const int c = blockIdx.x, d = blockIdx.y, tid = threadIdx.x;
+  const int ib = blockIdx.z * MDOT_VECS, ie = min(cnt, ib + MDOT_VECS);
   if (flag && !flag[d]) {
     // pass skipped for this direction: zero partials
-    for (int i = tid; i < cnt; i += blockDim.x)
+    for (int i = ib + tid; i < ie; i += blockDim.x)
       part[((size_t)d * nchunk + c) * cnt + i] = make_double2(0.0, 0.0);
     return;
   }
-  const int e0 = c * MDOT_CHUNK;
-  const int ne = min(nap - e0, MDOT_CHUNK);
+  const int e0 = c * chunk;
+  const int ne = min(nap - e0, chunk);
   const C<T>* wd = w + (size_t)d * ws + e0;
   for (int e = tid; e < ne; e += 256) sw[e] = wd[e];
   __syncthreads();
   const int warp = tid >> 5, lane = tid & 31;
   const int nsub = cnt >= 8 ? 1 : 8 / cnt;  // warps per basis vector
   const int ng = 8 / nsub;                  // basis vectors per round
-  for (int i0 = 0; i0 < cnt; i0 += ng) {
+  for (int i0 = ib; i0 < ie; i0 += ng) {
     const int i = i0 + warp / nsub, sub = warp - (warp / nsub) * nsub;
     double sr = 0, si = 0;
-    if (i < cnt) {
+    if (i < ie) {
       // per-lane partial sums (at most 64 terms) and the sum across the warp
       // in the vector precision; FP64 across warps and chunks.  (FP64
       // instructions are scarce on this GPU: an FP64 shuffle tree per warp
       // would cost more than the FP32 products themselves.)
       const C<T>* v = V + (size_t)d * vs + (size_t)i * nap + e0;
       T ar = 0, ai = 0;
-      if (nsub == 1 && ne == MDOT_CHUNK) {
+      if (nsub == 1 && ne == chunk) {
         // full chunk, one warp per vector: 8 loads in flight, 4 partial sums
         T pr[4] = {0, 0, 0, 0}, pi[4] = {0, 0, 0, 0};
-#pragma unroll 8
-        for (int k = 0; k < MDOT_CHUNK / 32; ++k) {
-          const int e = lane + 32 * k;
-          const C<T> a = v[e], b = sw[e];
-          pr[k & 3] += a.x * b.x + a.y * b.y;
-          pi[k & 3] += a.x * b.y - a.y * b.x;
+#pragma unroll 2
+        for (int k0 = 0; k0 < chunk / 32; k0 += 4) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int e = lane + 32 * (k0 + k);
+            const C<T> a = v[e], b = sw[e];
+            pr[k] += a.x * b.x + a.y * b.y;
+            pi[k] += a.x * b.y - a.y * b.x;
+          }
         }
         ar = (pr[0] + pr[1]) + (pr[2] + pr[3]);
         ai = (pi[0] + pi[1]) + (pi[2] + pi[3]);
@@ -127,7 +138,7 @@ __global__ void __launch_bounds__(256) k_mdot_partial(const C<T>* __restrict__ V
     }
     if (lane == 0) { rr[warp] = sr; ri[warp] = si; }
     __syncthreads();
-    if (tid < ng && i0 + tid < cnt) {
+    if (tid < ng && i0 + tid < ie) {
       double a = 0, b = 0;
       for (int q = 0; q < nsub; ++q) { a += rr[tid * nsub + q]; b += ri[tid * nsub + q]; }
       part[((size_t)d * nchunk + c) * cnt + i0 + tid] = make_double2(a, b);
@@ -285,7 +296,14 @@ template <typename T> struct GW {
   void* apw;    // operator workspace
 };
 
-static inline int mdot_chunks(int nap) { return (nap + MDOT_CHUNK - 1) / MDOT_CHUNK; }
+// entries per chunk: a power of two, 128 .. MDOT_CHUNK, about 300 chunks where
+// the vector allows
+static inline int mdot_chunk(int nap) {
+  int c = 128;
+  while (c < MDOT_CHUNK && (long long)c * 300 < nap) c *= 2;
+  return c;
+}
+static inline int mdot_chunks(int nap) { return (nap + mdot_chunk(nap) - 1) / mdot_chunk(nap); }
 
 template <typename T>
 static size_t gw_bytes(const Geo& g, int ndir, int m) {
@@ -327,8 +345,8 @@ static void mdot(cavity_ctx* ctx, const C<T>* V, long long vs, const C<T>* w, lo
   const int nap = ctx->g.nap, nchunk = mdot_chunks(nap);
   {
     KScope ks_(ctx, KC_KRYLOV);
-    k_mdot_partial<T><<<dim3(nchunk, ndir), 256, 0, ctx->stream>>>(V, vs, w, ws, part, cnt, nap,
-                                                                   nchunk, flag);
+    k_mdot_partial<T><<<dim3(nchunk, ndir, (cnt + MDOT_VECS - 1) / MDOT_VECS), 256, 0,
+                        ctx->stream>>>(V, vs, w, ws, part, cnt, nap, mdot_chunk(nap), nchunk, flag);
   }
   {
     KScope ks_(ctx, KC_KRYLOV);
@@ -363,6 +381,7 @@ static cavity_status gmres_core(cavity_ctx* ctx, int ndir, const C<T>* b, C<T>* 
   const long long nv = (long long)ndir * nap;
   const long long vs = (long long)(m + 1) * nap;
   cudaStream_t st = ctx->stream;
+  const int eb = elem_block(nv);
   std::vector<double> bnorm, rn;
   CKS(norms<T>(ctx, b, ndir, W.h, m + 1, bnorm, W.part));
   rn = bnorm;
@@ -409,7 +428,7 @@ static cavity_status gmres_core(cavity_ctx* ctx, int ndir, const C<T>* b, C<T>* 
       mdot<T>(ctx, W.V, vs, Vn, vs, k + 2, W.h, m + 1, W.part, ndir);
       {
         KScope ks_(ctx, KC_KRYLOV);
-        k_basis_axpy<T><<<dim3(nblk(nap, 256), ndir), 256, 0, st>>>(W.V, vs, W.h, m + 1, k + 1, Vn, nap,
+        k_basis_axpy<T><<<dim3(nblk(nap, eb), ndir), eb, 0, st>>>(W.V, vs, W.h, m + 1, k + 1, Vn, nap,
                                                                     (T)-1, nullptr, vs);
       }
       {
@@ -420,7 +439,7 @@ static cavity_status gmres_core(cavity_ctx* ctx, int ndir, const C<T>* b, C<T>* 
       mdot<T>(ctx, W.V, vs, Vn, vs, k + 1, W.h2, m + 1, W.part, ndir, W.flag);
       {
         KScope ks_(ctx, KC_KRYLOV);
-        k_basis_axpy<T><<<dim3(nblk(nap, 256), ndir), 256, 0, st>>>(W.V, vs, W.h2, m + 1, k + 1, Vn, nap,
+        k_basis_axpy<T><<<dim3(nblk(nap, eb), ndir), eb, 0, st>>>(W.V, vs, W.h2, m + 1, k + 1, Vn, nap,
                                                                     (T)-1, W.flag, vs);
       }
       mdot<T>(ctx, Vn, vs, Vn, vs, 1, W.y, m + 1, W.part, ndir);
@@ -509,7 +528,7 @@ static cavity_status gmres_core(cavity_ctx* ctx, int ndir, const C<T>* b, C<T>* 
     CK(cudaMemsetAsync(W.w, 0, sizeof(C<T>) * nv, st));
     {
       KScope ks_(ctx, KC_KRYLOV);
-      k_basis_axpy<T><<<dim3(nblk(nap, 256), ndir), 256, 0, st>>>(W.V, vs, W.y, m + 1, kmax, W.w, nap,
+      k_basis_axpy<T><<<dim3(nblk(nap, eb), ndir), eb, 0, st>>>(W.V, vs, W.y, m + 1, kmax, W.w, nap,
                                                                   (T)1);
     }
     CKS(launch_precond_apply<T>(ctx, ndir, W.w, W.z));

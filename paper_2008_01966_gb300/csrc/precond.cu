@@ -244,7 +244,8 @@ cavity_status launch_precond_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
   long long tot = (long long)g.nx * g.ny * ndir;
   {
     KScope ks_(ctx, KC_PRECOND);
-    k_pc_apply<T><<<(unsigned)((tot + 255) / 256), 256, 0, ctx->stream>>>(x, xs, y, ys, pinv, g.nx,
+    const int eb = elem_block(tot);
+    k_pc_apply<T><<<(unsigned)((tot + eb - 1) / eb), eb, 0, ctx->stream>>>(x, xs, y, ys, pinv, g.nx,
         g.ny, g.n1, g.n2, g.nap, ndir);
   }
   CK(cudaGetLastError());
