@@ -66,11 +66,11 @@ __global__ void __launch_bounds__(256) k_dots(const C<T>* __restrict__ V, long l
 // Multi-dot V^H w in two fixed-order stages: each block keeps one chunk of w
 // in shared memory and forms the partial dots of that chunk with all cnt basis
 // vectors (blockIdx.z takes MDOT_VECS of them); a second kernel adds the chunk
-// partials in chunk order.  The chunk depends on n_ap alone (mdot_chunk), so a
-// direction's sums do not depend on the batch.  FP64 work is scarce per SM (two
-// lanes), so a short vector is cut into pieces for as many SMs as it can feed:
-// up to 24 vectors of 3,007 entries took 40 us in two blocks, now 6.4 us in 24
-// to 72.
+// partials in chunk order.  The chunk depends on n_ap and cnt alone
+// (mdot_chunk), so a direction's sums do not depend on the batch.  FP64 work is
+// scarce per SM (two lanes), so a short vector is cut into pieces for as many
+// SMs as it can feed: up to 24 vectors of 3,007 entries took 40 us in two
+// blocks, now 6.4 us in 24 to 72.
 #define MDOT_CHUNK 2048
 #define MDOT_VECS 8
 template <typename T>
@@ -296,14 +296,17 @@ template <typename T> struct GW {
   void* apw;    // operator workspace
 };
 
-// entries per chunk: a power of two, 128 .. MDOT_CHUNK, about 300 chunks where
-// the vector allows
-static inline int mdot_chunk(int nap) {
+// entries per chunk: a power of two, 128 .. MDOT_CHUNK, for about 300 chunks
+// where the vector allows; about 32 for few products, where a chunk is little
+// work (norms of 16 vectors of 48,641 entries: 19 us, 40 us with 300)
+static inline int mdot_chunk(int nap, int cnt) {
   int c = 128;
-  while (c < MDOT_CHUNK && (long long)c * 300 < nap) c *= 2;
+  while (c < MDOT_CHUNK && (long long)c * (cnt >= MDOT_VECS ? 300 : 32) < nap) c *= 2;
   return c;
 }
-static inline int mdot_chunks(int nap) { return (nap + mdot_chunk(nap) - 1) / mdot_chunk(nap); }
+static inline int mdot_chunks(int nap, int cnt = MDOT_VECS) {
+  return (nap + mdot_chunk(nap, cnt) - 1) / mdot_chunk(nap, cnt);
+}
 
 template <typename T>
 static size_t gw_bytes(const Geo& g, int ndir, int m) {
@@ -342,11 +345,12 @@ static GW<T> gw_carve(void* base, const Geo& g, int ndir, int m) {
 template <typename T>
 static void mdot(cavity_ctx* ctx, const C<T>* V, long long vs, const C<T>* w, long long ws, int cnt,
                  double2* out, int ostride, double2* part, int ndir, const int* flag = nullptr) {
-  const int nap = ctx->g.nap, nchunk = mdot_chunks(nap);
+  const int nap = ctx->g.nap, nchunk = mdot_chunks(nap, cnt);
   {
     KScope ks_(ctx, KC_KRYLOV);
     k_mdot_partial<T><<<dim3(nchunk, ndir, (cnt + MDOT_VECS - 1) / MDOT_VECS), 256, 0,
-                        ctx->stream>>>(V, vs, w, ws, part, cnt, nap, mdot_chunk(nap), nchunk, flag);
+                        ctx->stream>>>(V, vs, w, ws, part, cnt, nap, mdot_chunk(nap, cnt), nchunk,
+                                       flag);
   }
   {
     KScope ks_(ctx, KC_KRYLOV);
