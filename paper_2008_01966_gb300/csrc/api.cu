@@ -506,7 +506,10 @@ extern "C" cavity_status cavity_set_option(cavity_ctx* ctx, int option, int valu
   switch (option) {
     case CAVITY_OPT_PASS_B_2048:
     case CAVITY_OPT_PASS_C_2048: ok = value == 0 || value == 1; break;
-    case CAVITY_OPT_GROUP_WIDTH: ok = value >= 1 && value <= 16; break;
+    case CAVITY_OPT_GROUP_WIDTH:
+      ok = value >= 1 && value <= 16;
+      if (ok) ctx->gw_set = true;
+      break;
     case CAVITY_OPT_FIELD_FUSED:
       ok = value >= 0 && value <= 2;
       // the FP32 profiles are laid out for one kernel or the other

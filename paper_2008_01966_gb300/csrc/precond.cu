@@ -225,30 +225,24 @@ cavity_status launch_precond(cavity_ctx* ctx) {
   return CAVITY_OK;
 }
 
-// y = (block diagonal)^{-1} x for ndir vectors
+// y = (block diagonal)^{-1} x at mode pair mn; pm: order of x
 template <typename T>
-__global__ void k_pc_apply(const C<T>* __restrict__ x, long long xs, C<T>* __restrict__ y,
-                           long long ys, const C<T>* __restrict__ pinv, int nx, int ny, int n1,
-                           int n2, int nap, int ndir) {
-  long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  const long long per = (long long)nx * ny;
-  if (gid >= per * ndir) return;
-  const int d = (int)(gid / per);
-  const int mn = (int)(gid - (long long)d * per);
+__device__ __forceinline__ void pc_mode(const C<T>* __restrict__ xd, C<T>* __restrict__ yd, int mn,
+                                        const C<T>* __restrict__ pinv, int ny, int n1, int n2,
+                                        const ParityMap& pm) {
   const int lny = __ffs(ny) - 1;                 // ny is a power of two
   const int m = mn >> lny, n = mn & (ny - 1);
   const int N = ny - 1;
   const bool has1 = n >= 1, has2 = m >= 1, has3 = m >= 1 && n >= 1;
   const int i1 = m * N + (n - 1), i2 = n1 + (m - 1) * (N + 1) + n;
   const int i3 = n1 + n2 + (m - 1) * N + (n - 1);
-  const C<T>* xd = x + (size_t)d * xs;
-  C<T>* yd = y + (size_t)d * ys;
   C<T> v[3] = {mk<T>(0, 0), mk<T>(0, 0), mk<T>(0, 0)};
-  if (has1) v[0] = xd[i1];
-  if (has2) v[1] = xd[i2];
-  if (has3) v[2] = xd[i3];
+  if (has1) v[0] = xd[pm.on ? pm.e1(m, n) : i1];
+  if (has2) v[1] = xd[pm.on ? pm.e2(m, n) : i2];
+  if (has3) v[2] = xd[pm.on ? pm.e3(m, n) : i3];
   const C<T>* B = pinv + (size_t)mn * 9;
   C<T> r[3];
+#pragma unroll
   for (int a = 0; a < 3; ++a) {
     r[a] = cmul<T>(B[a * 3 + 0], v[0]);
     r[a] = cadd<T>(r[a], cmul<T>(B[a * 3 + 1], v[1]));
@@ -259,9 +253,32 @@ __global__ void k_pc_apply(const C<T>* __restrict__ x, long long xs, C<T>* __res
   if (has3) yd[i3] = r[2];
 }
 
+// y = (block diagonal)^{-1} x for ndir vectors
+template <typename T>
+__global__ void k_pc_apply(const C<T>* __restrict__ x, long long xs, C<T>* __restrict__ y,
+                           long long ys, const C<T>* __restrict__ pinv, int nx, int ny, int n1,
+                           int n2, int nap, int ndir, ParityMap pm) {
+  long long gid = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+  const long long per = (long long)nx * ny;
+  if (gid >= per * ndir) return;
+  const int d = (int)(gid / per);
+  pc_mode<T>(x + (size_t)d * xs, y + (size_t)d * ys, (int)(gid - (long long)d * per), pinv, ny, n1,
+             n2, pm);
+}
+// the same for the columns of several groups; grid (ceil(nx ny / 256), ncol)
+__global__ void k_pc_groups(PcCols cols, float2* __restrict__ y, const float2* __restrict__ pinv,
+                            int nmode, int ny, int n1, int n2, int nap, ParityMap pm) {
+  const int c = blockIdx.y, mn = blockIdx.x * blockDim.x + threadIdx.x;
+  if (mn >= nmode) return;
+  int g = 0;
+  while (g + 1 < cols.n && cols.first[g + 1] <= c) ++g;
+  pc_mode<float>(cols.src[g] + (size_t)(c - cols.first[g]) * nap, y + (size_t)c * nap, mn, pinv, ny,
+                 n1, n2, pm);
+}
+
 template <typename T>
 cavity_status launch_precond_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y,
-                                   long long xs, long long ys) {
+                                   long long xs, long long ys, const ParityMap& pm) {
   if (xs < 0) xs = ctx->g.nap;
   if (ys < 0) ys = ctx->g.nap;
   const Geo& g = ctx->g;
@@ -273,7 +290,7 @@ cavity_status launch_precond_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
     KScope ks_(ctx, KC_PRECOND);
     const int eb = elem_block(tot);
     k_pc_apply<T><<<(unsigned)((tot + eb - 1) / eb), eb, 0, ctx->stream>>>(x, xs, y, ys, pinv, g.nx,
-        g.ny, g.n1, g.n2, g.nap, ndir);
+        g.ny, g.n1, g.n2, g.nap, ndir, pm);
   }
   CK(cudaGetLastError());
   // two-level variant (FP32 inner solves of the mixed path): the coarse
@@ -283,6 +300,24 @@ cavity_status launch_precond_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
 }
 
 template cavity_status launch_precond_apply<double>(cavity_ctx*, int, const double2*, double2*,
-                                                    long long, long long);
+                                                    long long, long long, const ParityMap&);
 template cavity_status launch_precond_apply<float>(cavity_ctx*, int, const float2*, float2*,
-                                                   long long, long long);
+                                                   long long, long long, const ParityMap&);
+
+cavity_status launch_precond_groups(cavity_ctx* ctx, int ncol, const PcCols& cols, float2* y,
+                                    const ParityMap& pm) {
+  const Geo& g = ctx->g;
+  if (ctx->opt[CAVITY_OPT_COARSE_MODES] > 0) {   // the coarse level works group by group
+    for (int q = 0; q < cols.n; ++q) {
+      const int n = (q + 1 < cols.n ? cols.first[q + 1] : ncol) - cols.first[q];
+      CKS(launch_precond_apply<float>(ctx, n, cols.src[q], y + (size_t)cols.first[q] * g.nap, g.nap,
+                                      g.nap, pm));
+    }
+    return CAVITY_OK;
+  }
+  KScope ks_(ctx, KC_PRECOND);
+  k_pc_groups<<<dim3((g.nx * g.ny + 255) / 256, ncol), 256, 0, ctx->stream>>>(
+      cols, y, ctx->pinv32, g.nx * g.ny, g.ny, g.n1, g.n2, g.nap, pm);
+  CK(cudaGetLastError());
+  return CAVITY_OK;
+}

@@ -108,7 +108,7 @@ size_t apply_work_bytes(const Geo& g, int ndir, int eb) {
 }
 
 template cavity_status launch_apply<double>(cavity_ctx*, int, const double2*, double2*, void*,
-                                           long long);
+                                           long long, const ParityMap&);
 
 
 // ------------------------------------------------------------------ no-alloc
@@ -164,6 +164,39 @@ extern "C" cavity_status cavity_apply_noalloc(cavity_ctx* ctx, int ndir, int pre
   return CAVITY_OK;
 }
 
-cavity_status launch_mode_mask(cavity_ctx* ctx, int ndir, double2* v) {
-  return launch_mode_mask_t<double>(ctx, ndir, v, ctx->g.nap, KC_RHS);
+// Truncated aperture expansion (Sec. 7, Table 2: the paper's runs keep the
+// modes m <= ~2a/lambda): y_i = 0 for unknowns i of a mode (m, n) with
+// m > mm or n > nn.  Unknown order (Appendix A): E1 over m = 0..M, n = 1..N;
+// E2 over m = 1..M, n = 0..N; E3 over m = 1..M, n = 1..N.
+// grid (ceil(nap / 256), ndir)
+__global__ void k_mode_mask(double2* __restrict__ y, int nap, int N, int n1, int n2,
+                            int mm, int nn) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= nap) return;
+  int m, n;
+  if (i < n1) {
+    m = i / N;
+    n = i - m * N + 1;
+  } else if (i < n1 + n2) {
+    const int j = i - n1;
+    m = j / (N + 1) + 1;
+    n = j - (m - 1) * (N + 1);
+  } else {
+    const int j = i - n1 - n2;
+    m = j / N + 1;
+    n = j - (m - 1) * N + 1;
+  }
+  if (m > mm || n > nn) y[(size_t)blockIdx.y * nap + i] = make_double2(0.0, 0.0);
+}
+
+cavity_status launch_mode_mask(cavity_ctx* ctx, int ndir, double2* y) {
+  const cavity_desc& d = ctx->desc;
+  if (d.modes_m <= 0 && d.modes_n <= 0) return CAVITY_OK;
+  const Geo& g = ctx->g;
+  const int mm = d.modes_m > 0 ? d.modes_m : g.M, nn = d.modes_n > 0 ? d.modes_n : g.N;
+  KScope ks_(ctx, KC_RHS);
+  k_mode_mask<<<dim3((g.nap + 255) / 256, ndir), 256, 0, ctx->stream>>>(y, g.nap, g.N, g.n1,
+                                                                          g.n2, mm, nn);
+  CK(cudaGetLastError());
+  return CAVITY_OK;
 }

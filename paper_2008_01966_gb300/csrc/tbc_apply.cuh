@@ -591,12 +591,14 @@ __global__ void TBC_BOUNDS_LN(LNX) k_tbcD(const C<T>* __restrict__ Z, C<T>* __re
 //  row 2: (-1+tau2)E2 + (n pi h/b + vs2)E3 + (h/c)(2k^2 U2 + 2(m pi/a) W)
 //  row 3: (m pi h/a)E1 + (n pi h/b)E2 + (-1+tau3)E3
 // One thread per mode pair (m, n), m < nx, n < ny, writing the rows of the
-// three components that exist for it; nyp: pitch of O's rows; grid
-// (ceil(nx ny / 256), ndir).
+// three components that exist for it, 0 for the modes beyond (mm, nn) of a
+// truncated expansion (the operator then maps the kept subspace to itself, as
+// does the mode-wise preconditioner); nyp: pitch of O's rows; pm: order of y;
+// grid (ceil(nx ny / blockDim), ndir).
 template <typename T>
 __global__ void k_combine(const C<T>* __restrict__ x, const C<T>* __restrict__ O,
                           const C<T>* __restrict__ top, C<T>* __restrict__ y, long long ys, int nyp,
-                          TbcP p) {
+                          TbcP p, int mm, int nn, ParityMap pm) {
   const int d = blockIdx.y;
   const int mn = blockIdx.x * blockDim.x + threadIdx.x;
   if (mn >= p.nx * p.ny) return;
@@ -611,6 +613,7 @@ __global__ void k_combine(const C<T>* __restrict__ x, const C<T>* __restrict__ O
   const int i1 = m * N + (n - 1), i2 = p.n1 + (m - 1) * (N + 1) + n;
   const int i3 = p.n1 + p.n2 + (m - 1) * N + (n - 1);
   const bool has1 = n >= 1, has2 = m >= 1, has3 = m >= 1 && n >= 1;
+  const bool kept = m <= mm && n <= nn;
   const C<T> e1 = has1 ? xd[i1] : mk<T>(0, 0);
   const C<T> e2 = has2 ? xd[i2] : mk<T>(0, 0);
   const C<T> e3 = has3 ? xd[i3] : mk<T>(0, 0);
@@ -620,19 +623,20 @@ __global__ void k_combine(const C<T>* __restrict__ x, const C<T>* __restrict__ O
     if (has3) r = cadd<T>(r, cmul<T>(cadd<T>(mk<T>(m * pa * h, 0), top[p.nap + i1]), e3));
     const T s = h / (m == 0 ? ab / 2 : ab / 4);
     const C<T> t = csub<T>(cscale<T>(Od[o], k2), cscale<T>(Od[2 * fs + o], 2 * n * pb));
-    yd[i1] = cadd<T>(r, cscale<T>(t, s));
+    yd[pm.on ? pm.e1(m, n) : i1] = kept ? cadd<T>(r, cscale<T>(t, s)) : czero<T>();
   }
   if (has2) {
     C<T> r = cmul<T>(cadd<T>(mk<T>(-1, 0), top[i2]), e2);
     if (has3) r = cadd<T>(r, cmul<T>(cadd<T>(mk<T>(n * pb * h, 0), top[p.nap + i2]), e3));
     const T s = h / (n == 0 ? ab / 2 : ab / 4);
     const C<T> t = cadd<T>(cscale<T>(Od[fs + o], k2), cscale<T>(Od[2 * fs + o], 2 * m * pa));
-    yd[i2] = cadd<T>(r, cscale<T>(t, s));
+    yd[pm.on ? pm.e2(m, n) : i2] = kept ? cadd<T>(r, cscale<T>(t, s)) : czero<T>();
   }
   if (has3) {
     C<T> r = cscale<T>(e1, m * pa * h);
     r = cadd<T>(r, cscale<T>(e2, n * pb * h));
-    yd[i3] = cadd<T>(r, cmul<T>(cadd<T>(mk<T>(-1, 0), top[i3]), e3));
+    r = cadd<T>(r, cmul<T>(cadd<T>(mk<T>(-1, 0), top[i3]), e3));
+    yd[pm.on ? pm.e3(m, n) : i3] = kept ? r : czero<T>();
   }
 }
 
@@ -682,6 +686,10 @@ template <typename T> static size_t smem_d(int nx, int lL) {
   return sizeof(C<T>) * ((size_t)1 << lL) * padded_len(2 * nx);
 }
 
+// the last kept mode of each axis
+static int last_m(const cavity_ctx* ctx) { return ctx->desc.modes_m > 0 ? ctx->desc.modes_m : ctx->g.M; }
+static int last_n(const cavity_ctx* ctx) { return ctx->desc.modes_n > 0 ? ctx->desc.modes_n : ctx->g.N; }
+
 // opt every instantiation of kernel K into the device's shared-memory maximum
 // once per process
 template <typename K> static cavity_status smem_once(cavity_ctx* ctx, K kern, std::atomic<bool>& done) {
@@ -699,48 +707,9 @@ template <typename T> static int kclass(int k) {
   return KC_TBC_AP + k;
 }
 
-// Truncated aperture expansion (Sec. 7, Table 2: the paper's runs keep the
-// modes m <= ~2a/lambda): y_i = 0 for unknowns i of a mode (m, n) with
-// m > mm or n > nn.  Unknown order (Appendix A): E1 over m = 0..M, n = 1..N;
-// E2 over m = 1..M, n = 0..N; E3 over m = 1..M, n = 1..N.
-// grid (ceil(nap / 256), ndir)
-template <typename T>
-__global__ void k_mode_mask(C<T>* __restrict__ y, long long ystride, int nap, int N, int n1, int n2,
-                            int mm, int nn) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nap) return;
-  int m, n;
-  if (i < n1) {
-    m = i / N;
-    n = i - m * N + 1;
-  } else if (i < n1 + n2) {
-    const int j = i - n1;
-    m = j / (N + 1) + 1;
-    n = j - (m - 1) * (N + 1);
-  } else {
-    const int j = i - n1 - n2;
-    m = j / N + 1;
-    n = j - (m - 1) * N + 1;
-  }
-  if (m > mm || n > nn) y[(size_t)blockIdx.y * ystride + i] = czero<T>();
-}
-
-template <typename T>
-cavity_status launch_mode_mask_t(cavity_ctx* ctx, int ndir, C<T>* y, long long ystride, int cls) {
-  const cavity_desc& d = ctx->desc;
-  if (d.modes_m <= 0 && d.modes_n <= 0) return CAVITY_OK;
-  const Geo& g = ctx->g;
-  const int mm = d.modes_m > 0 ? d.modes_m : g.M, nn = d.modes_n > 0 ? d.modes_n : g.N;
-  KScope ks_(ctx, cls);
-  k_mode_mask<T><<<dim3((g.nap + 255) / 256, ndir), 256, 0, ctx->stream>>>(y, ystride, g.nap, g.N, g.n1,
-                                                                          g.n2, mm, nn);
-  CK(cudaGetLastError());
-  return CAVITY_OK;
-}
-
 template <typename T>
 cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
-                                   long long ystride) {
+                                   long long ystride, const ParityMap& pm) {
   if (!ctx->g.fft_ok) {
     ctx->err = "the FFT operator needs the convolution period 4 on both axes";
     return CAVITY_EINVAL;
@@ -824,17 +793,15 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
     KScope ks_(ctx, kclass<T>(4));
     const int eb = elem_block((long long)g.nx * g.ny * ndir);
     k_combine<T><<<dim3((g.nx * g.ny + eb - 1) / eb, ndir), eb, 0, st>>>(x, R2, Tabs<T>::top(ctx), y,
-                                                                         ystride, g.ny + 1, p);
+                                                                         ystride, g.ny + 1, p,
+                                                                         last_m(ctx), last_n(ctx), pm);
   }
   CK(cudaGetLastError());
-  // truncated expansion: the rows of the dropped modes (the operator then
-  // maps the kept subspace to itself, as does the mode-wise preconditioner)
-  CKS(launch_mode_mask_t<T>(ctx, ndir, y, ystride, kclass<T>(4)));
   return CAVITY_OK;
 }
 
 template <typename T>
 cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
-                           long long ystride) {
-  return launch_apply_generic<T>(ctx, ndir, x, y, work, ystride);
+                           long long ystride, const ParityMap& pm) {
+  return launch_apply_generic<T>(ctx, ndir, x, y, work, ystride, pm);
 }

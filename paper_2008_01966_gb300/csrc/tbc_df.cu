@@ -31,7 +31,8 @@ TBC_PASS_KERNELS(extern, df, 8)
 TBC_PASS_KERNELS(extern, df, 9)
 TBC_PASS_KERNELS(extern, df, 10)
 
-template cavity_status launch_apply<df>(cavity_ctx*, int, const cdf*, cdf*, void*, long long);
+template cavity_status launch_apply<df>(cavity_ctx*, int, const cdf*, cdf*, void*, long long,
+                                        const ParityMap&);
 
 __global__ void k_to_pair(const double2* __restrict__ a, cdf* __restrict__ b, long long n) {
   const long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x;

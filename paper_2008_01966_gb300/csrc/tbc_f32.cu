@@ -433,7 +433,7 @@ cavity_status launch_khat_split(cavity_ctx* ctx) {
 }
 
 static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x, float2* y,
-                                      void* work, long long ystride) {
+                                      void* work, long long ystride, const ParityMap& pm) {
   const Geo& g = ctx->g;
   TbcP p = make_params(ctx);
   cudaStream_t st = ctx->stream;
@@ -486,10 +486,10 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
   {
     KScope ks_(ctx, KC_COMB32);
     k_combine<float><<<dim3((g.nx * g.ny + 255) / 256, ndir), 256, 0, st>>>(
-        x, R2, ctx->top32, y, ystride, g.ny, p);
+        x, R2, ctx->top32, y, ystride, g.ny, p, last_m(ctx), last_n(ctx), pm);
   }
   CK(cudaGetLastError());
-  return launch_mode_mask_t<float>(ctx, ndir, y, ystride, KC_COMB32);
+  return CAVITY_OK;
 }
 
 // Sides of 4 or 8 intervals (a line has fewer points than the smallest group
@@ -497,12 +497,12 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
 // transform, take the generic passes of tbc_apply.cuh.
 template <>
 cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, float2* y,
-                                  void* work, long long ystride) {
+                                  void* work, long long ystride, const ParityMap& pm) {
   const Geo& g = ctx->g;
   if (ystride < 0) ystride = g.nap;
   const bool block = (g.lnx == 9 && ctx->opt[CAVITY_OPT_PASS_B_2048]) ||
                      (g.lny == 9 && ctx->opt[CAVITY_OPT_PASS_C_2048]);
   if (g.fft_ok && f32_fast_size(g.lnx) && f32_fast_size(g.lny) && !block)
-    return launch_apply_f32(ctx, ndir, x, y, work, ystride);
-  return launch_apply_generic<float>(ctx, ndir, x, y, work, ystride);
+    return launch_apply_f32(ctx, ndir, x, y, work, ystride, pm);
+  return launch_apply_generic<float>(ctx, ndir, x, y, work, ystride, pm);
 }
