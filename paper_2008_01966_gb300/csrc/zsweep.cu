@@ -104,7 +104,11 @@ __global__ void k_zsweep(ZP p, LayerTab L, double2* __restrict__ prof, double2* 
     const double n2 = piv.x * piv.x + piv.y * piv.y;
     worst = fmin(worst, n2 * isc);
     const double inv = 1.0 / n2;
-    rho = make_double2(piv.x * inv, -piv.y * inv);
+    // quotients by one correction of the products with the reciprocal
+    double qx = piv.x * inv, qy = -piv.y * inv;
+    qx = fma(fma(-qx, n2, piv.x), inv, qx);
+    qy = fma(fma(-qy, n2, -piv.y), inv, qy);
+    rho = make_double2(qx, qy);
     if (src) eta = cmul<double>(rho, eta);
     prof[(size_t)(j - 1) * p.nap + i] = rho;
     if (src) profq[(size_t)(j - 1) * nqs + i] = eta;
