@@ -316,7 +316,8 @@ cavity_status cavity_lu_solve(cavity_ctx* ctx, const void* lu, int n, int lda, c
  *      of a group of lanes (default), 1 = the generic passes with the block
  *      (Stockham) transform.
  *  CAVITY_OPT_GROUP_WIDTH: directions per group of the mixed solve's block
- *      Krylov iterations (one basis per group), 1..16; default 16.
+ *      Krylov iterations (one basis per group), 1..16; default 16, taken as 8
+ *      on grids of fewer than 30,000 aperture unknowns unless it is set.
  *  CAVITY_OPT_COARSE_MODES: two-level preconditioner of the mixed solve's
  *      inner FP32 iterations (Krylov solver): 0 (default) = the 3 x 3 block
  *      diagonal of each mode alone; mc > 0 = in addition the kept block of
@@ -325,13 +326,10 @@ cavity_status cavity_lu_solve(cavity_ctx* ctx, const void* lu, int n, int lda, c
  *      at the first mixed solve after cavity_prepare or a change of mc; its
  *      3 mc^2 + 2 mc unknowns must not exceed CAVITY_DENSE_MAX_N.  Changes
  *      the iteration count, not the result beyond the solver tolerance.
- *  CAVITY_OPT_FIELD_FUSED: the complex64 field synthesis of square grids of
- *      32..512 points per side: 0 (default) = the fused persistent kernel at
- *      512 points per side (faster there), the two-pass kernels elsewhere;
- *      1 = the fused kernel on every square grid it supports; 2 = always the
- *      two-pass kernels.  The fields agree to FP32 rounding.  The FP32
- *      profiles are stored in the chosen kernel's layout at cavity_prepare,
- *      so a change takes effect at the next prepare (a solve re-prepares).
+ *  CAVITY_OPT_FIELD_FUSED: accepts 0, 1 and 2, as before; the complex64 field
+ *      has one path (two passes), which is faster than the fused kernel these
+ *      values used to choose.  A change still takes effect at the next prepare
+ *      (a solve re-prepares).
  * CAVITY_EINVAL for an unknown option or a value out of range. */
 enum { CAVITY_OPT_PASS_B_2048 = 0, CAVITY_OPT_PASS_C_2048 = 1, CAVITY_OPT_GROUP_WIDTH = 2,
        CAVITY_OPT_COARSE_MODES = 3, CAVITY_OPT_FIELD_FUSED = 4, CAVITY_NUM_OPT = 5 };

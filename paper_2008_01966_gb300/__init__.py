@@ -361,8 +361,7 @@ class Cavity:
         (1..16 directions per block Krylov group), "coarse_modes" (0, or
         mc > 0: the mixed solve's two-level preconditioner with the exact
         solve of the modes m, n <= mc as its coarse level) or "field_fused"
-        (complex64 field synthesis: 0 the default per grid, 1 the fused
-        kernel where the grid allows it, 2 the two passes)."""
+        (0, 1 or 2: accepted, the complex64 field has one path)."""
         self._check(self.lib.cavity_set_option(self.h, _lib.OPTIONS[name], int(value)))
 
     def get_option(self, name):

@@ -16,7 +16,7 @@ OUT = os.path.join(HERE, "libcavity.so")
 BUILD = os.path.join(HERE, "_build")
 SOURCES = ["api.cu", "tbc.cu", "tbc_f32.cu", "tbc_df.cu", "tbc_df_k2.cu", "tbc_df_k5.cu",
            "tbc_df_k7.cu", "tbc_df_k9.cu", "tbc_df_k10.cu", "zsweep.cu", "khat.cu", "rhs.cu",
-           "precond.cu", "gmres.cu", "bgmres.cu", "dense.cu", "field.cu", "field_fused.cu"]
+           "precond.cu", "gmres.cu", "bgmres.cu", "dense.cu", "field.cu", "field_f32.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fcx-limited-range",
          "-Xptxas", "-O3"]

@@ -92,7 +92,7 @@ extern "C" cavity_status cavity_setup(const cavity_desc* desc, void* cuda_stream
   ctx->TW = 2 * std::max(g.Px, g.Py);
   cavity_status s = launch_twiddles(ctx);
   if (s == CAVITY_OK && g.fft_ok) s = launch_ehat(ctx);
-  if (s == CAVITY_OK && g.fft_ok) s = launch_lane_tables(ctx);
+  if (s == CAVITY_OK) s = launch_lane_tables(ctx);
   if (s == CAVITY_OK) {
     cudaError_t e = cudaStreamSynchronize(ctx->stream);
     if (e != cudaSuccess) {
@@ -116,8 +116,9 @@ extern "C" void cavity_destroy(cavity_ctx* ctx) {
                   ctx->ehat_y32[1], ctx->khat64, ctx->khat32, ctx->khat_raw, ctx->prof, ctx->profq,
                   ctx->top64, ctx->top32, ctx->pinv64, ctx->pinv32, ctx->prof32, ctx->profq32,
                   ctx->minpiv, ctx->ws, ctx->ws2, ctx->stage, ctx->tw_p, ctx->ehat_xp[0],
-                  ctx->ehat_xp[1], ctx->ehat_yp[0], ctx->ehat_yp[1], ctx->khat_p, ctx->top_p, ctx->prof_rec,
-                  ctx->dn_scr, ctx->khat32s, ctx->lane_tab[0], ctx->lane_tab[1]};
+                  ctx->ehat_xp[1], ctx->ehat_yp[0], ctx->ehat_yp[1], ctx->khat_p, ctx->top_p,
+                  ctx->dn_scr, ctx->khat32s, ctx->lane_tab[0], ctx->lane_tab[1],
+                  ctx->lane_tab_f[0], ctx->lane_tab_f[1]};
   for (void* p : ptrs)
     if (p) cudaFree(p);
   dense_free(ctx->dn);
@@ -512,7 +513,7 @@ extern "C" cavity_status cavity_set_option(cavity_ctx* ctx, int option, int valu
       break;
     case CAVITY_OPT_FIELD_FUSED:
       ok = value >= 0 && value <= 2;
-      // the FP32 profiles are laid out for one kernel or the other
+      // a change takes effect at the next prepare
       if (ok && value != ctx->opt[option]) ctx->prepared = false;
       break;
     case CAVITY_OPT_COARSE_MODES: {

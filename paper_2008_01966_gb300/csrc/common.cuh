@@ -183,6 +183,7 @@ struct cavity_ctx {
   float2* khat32 = nullptr;
   float2* khat32s = nullptr;   // khat32 by parity of j1 for the FP32 passes (tbc_f32.cu)
   float2* lane_tab[2] = {nullptr, nullptr};  // their twiddle tables per axis (gfft.cuh)
+  float2* lane_tab_f[2] = {nullptr, nullptr};  // the same for the field's lines (field_f32.cu)
   double2* khat_raw = nullptr; // unscaled copy [j1][j2] for export
   double2* prof = nullptr;     // (nz-1) x nap profiles P, level-major
   double2* profq = nullptr;    // (nz-1) x (n1+n2) profiles Q (layered only)
@@ -194,12 +195,6 @@ struct cavity_ctx {
   float2* pinv32 = nullptr;
   float2* prof32 = nullptr;    // FP32 copies of the profiles for the mixed field path
   float2* profq32 = nullptr;
-  // FP32 profiles of the fused field kernel as one record per (level, m, n)
-  // on the full nx x ny mode grid: {P1, P2}, {P3, Q1}, {Q2, 0} (layered, 3
-  // float4) or {P1, P2}, {P3, 0} (homogeneous, 2 float4); entries outside a
-  // component's index set are 0 (field_fused.cu)
-  float4* prof_rec = nullptr;
-  int prof_rec_w = 0;
   double* minpiv = nullptr;    // device scalar: min |pivot| / scale
 
   // ---- workspaces (grown on demand)
@@ -421,14 +416,11 @@ cavity_status launch_mode_mask(cavity_ctx* ctx, int ndir, double2* v);
 template <typename T>
 cavity_status launch_field(cavity_ctx* ctx, int ndir, const double2* ap, C<T>* out,
                            void* host_out = nullptr);
-// the fused field kernel (field_fused.cu): the grids it covers, and the
-// per-(level, m, n) FP32 profile records it reads, built from the FP64
-// profiles at prepare
-bool field_fused_supported(const Geo& g);
-// whether this context's complex64 field takes the fused kernel
-// (CAVITY_OPT_FIELD_FUSED; fixed at prepare, with the profile layout)
-bool field_fused_use(const cavity_ctx* ctx);
-cavity_status launch_prof_records(cavity_ctx* ctx);
+// the two-pass complex64 field of field_f32.cu (grids of 16 and more per side)
+bool field_f32_supported(const Geo& g);
+size_t field_f32_slab_bytes(const Geo& g);
+cavity_status launch_field_f32(cavity_ctx* ctx, int ndir, const float2* ap, float2* out, float2* T1,
+                               int j0, int nlev);
 // the copy stream and at least n events for it (created once per context)
 inline cavity_status ensure_copy_stream(cavity_ctx* ctx, size_t n) {
   if (!ctx->copy_stream) {

@@ -72,6 +72,12 @@ cavity_status launch_lane_tables(cavity_ctx* ctx) {
       CK(cudaMalloc(&ctx->lane_tab[ax], sizeof(float2) * sz));
       KScope ks_(ctx, KC_SETUP);
       k_lane_tab<<<(sz + 255) / 256, 256, 0, ctx->stream>>>(ctx->lane_tab[ax], n, S::LG, S::RV);
+      // the field's lines, of 2 << ln points
+      using SF = GShape<decltype(c)::value + 1>;
+      const int szf = lane_tab_size(n / 2, SF::LG);
+      CK(cudaMalloc(&ctx->lane_tab_f[ax], sizeof(float2) * szf));
+      k_lane_tab<<<(szf + 255) / 256, 256, 0, ctx->stream>>>(ctx->lane_tab_f[ax], n / 2, SF::LG,
+                                                            SF::RV);
       return CAVITY_OK;
     }));
   }

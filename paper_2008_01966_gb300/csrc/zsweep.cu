@@ -189,11 +189,8 @@ cavity_status launch_zsweep(cavity_ctx* ctx, double kappa0) {
   }
   size_t nprof = (size_t)(g.nz - 1) * g.nap;
   size_t nq = (size_t)(g.nz - 1) * (g.n1 + g.n2);
-  // FP32 copies of the profiles for the complex64 field of mixed contexts:
-  // records for the fused kernel where it runs, else plain copies
-  const bool mixed = ctx->desc.precision == CAVITY_MIXED;
-  const bool recs = mixed && field_fused_use(ctx);
-  const bool plain32 = mixed && !recs;
+  // FP32 copies of the profiles for the complex64 field of mixed contexts
+  const bool plain32 = ctx->desc.precision == CAVITY_MIXED;
   if (!ctx->prof) CK(cudaMalloc(&ctx->prof, sizeof(double2) * nprof));
   if (plain32 && !ctx->prof32) CK(cudaMalloc(&ctx->prof32, sizeof(float2) * nprof));
   if (!ctx->top64) CK(cudaMalloc(&ctx->top64, sizeof(double2) * (g.nap + g.n1 + g.n2)));
@@ -229,7 +226,6 @@ cavity_status launch_zsweep(cavity_ctx* ctx, double kappa0) {
     k_f32_copy<<<(unsigned)((nprof + 255) / 256), 256, 0, ctx->stream>>>(ctx->prof, ctx->prof32,
                                                                        (long long)nprof);
   }
-  if (recs) CKS(launch_prof_records(ctx));
   long long ntop = g.nap + g.n1 + g.n2;
   {
     KScope ks_(ctx, KC_SETUP);
