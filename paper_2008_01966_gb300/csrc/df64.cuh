@@ -13,7 +13,7 @@
 // Every step uses the _rn intrinsics, which the compiler never contracts into
 // fused multiply-adds or reassociates, so the transformations stay exact.
 #pragma once
-#include "common.cuh"
+#include "fft.cuh"
 
 struct __align__(8) df {
   float hi, lo;
@@ -31,6 +31,18 @@ struct __align__(16) cdf {
   df x, y;
 };
 template <> struct cplx_t<df> { typedef cdf type; };
+// Four points a thread, radix 4 (fft.cuh): 64 registers, so 32 warps per SM, where
+// radix 8 takes 128 and 16 warps left the kernels waiting (issue slots 40-55 %
+// busy).  A line has 256 threads at most, so that two CTAs share an SM; at 4096
+// points, where shared memory holds one CTA, 512.  Operator on a GB300, with
+// radix 8 and spills of 0.3-2 KB a thread, and now (128 threads a line of 1024
+// points and 256 of 2048 then): 256 x 256, 6 vectors 2.35 -> 1.74 ms; 512 x 512,
+// 8 vectors 10.0 -> 8.6 ms (10.4 with 512 threads a line and one CTA per SM);
+// 1024 x 1024, 3 vectors 25.7 -> 14.8 ms; 32 x 32, one vector 96 -> 75 us.
+template <> struct FftE<df> {
+  static constexpr int E = 4, LRMAX = 2, THREADS = 512;
+  __host__ __device__ static constexpr int max_tpl(int n) { return n < 4096 ? 256 : 512; }
+};
 
 __device__ __forceinline__ df df_two_sum(float a, float b) {
   const float s = __fadd_rn(a, b);

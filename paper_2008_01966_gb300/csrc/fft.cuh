@@ -33,11 +33,14 @@ __host__ __device__ constexpr int pidx(int i) { return i + (i >> 4); }
 // line length in shared memory: room for the padded layout and for the
 // transposed tile of the warp transform (n + n/8 for n >= 64)
 __host__ __device__ constexpr int padded_len(int n) { return n + (n >> 3) + 2; }
-// block transform: elements per thread (radix up to 8), and at most
-// FFT_MAX_TPL threads per line: lines longer than 8 FFT_MAX_TPL points give
-// each thread several butterflies per pass (16 points per thread at 4096)
-template <typename T> struct FftE { static constexpr int E = 8, LRMAX = 3; };
-#define FFT_MAX_TPL 256
+// block transform: elements per thread (radix up to E = 2^LRMAX), threads of a
+// CTA, most threads of a line of n points: longer lines than E max_tpl points
+// give each thread several butterflies per pass (16 points per thread at
+// 4096).  The pair type has its own (df64.cuh).
+template <typename T> struct FftE {
+  static constexpr int E = 8, LRMAX = 3, THREADS = 256;
+  __host__ __device__ static constexpr int max_tpl(int) { return THREADS; }
+};
 // warp transform (FP32, 64 <= n <= 1024): n = LW * RV lanes x values per lane
 __host__ __device__ constexpr bool warp_fft_ok(int n, int elem_bytes) {
   return elem_bytes == 8 && n >= 64 && n <= 1024;
@@ -50,7 +53,8 @@ __host__ __device__ constexpr int warp_lanes(int n) {
 // threads cooperating on one line (same as LineShape<T, log2 n>::TPL)
 template <typename T> __host__ __device__ constexpr int fft_tpl(int n) {
   if (warp_fft_ok(n, (int)sizeof(C<T>))) return warp_lanes(n);
-  return n >= FftE<T>::E ? (n / FftE<T>::E < FFT_MAX_TPL ? n / FftE<T>::E : FFT_MAX_TPL) : 1;
+  return n >= FftE<T>::E
+             ? (n / FftE<T>::E < FftE<T>::max_tpl(n) ? n / FftE<T>::E : FftE<T>::max_tpl(n)) : 1;
 }
 
 // twiddle constants (forward sign); the inverse uses the conjugates
@@ -415,32 +419,27 @@ template <typename T, int LOGN> struct LineShape {
   static constexpr bool WARP = sizeof(T) == 4 && LOGN >= 6 && LOGN <= 10;
   static constexpr int LW = 1 << (LOGN / 2);
   static constexpr int RV = (1 << LOGN) / LW;
-  static constexpr int TPL =
-      WARP ? LW : (LOGN >= 3 ? ((1 << LOGN) / 8 < FFT_MAX_TPL ? (1 << LOGN) / 8 : FFT_MAX_TPL) : 1);
+  static constexpr int TPL = WARP ? LW : fft_tpl<T>(1 << LOGN);
 };
 
-// radix (log2) of pass P of the balanced schedule for a length 2^LOGN
-template <int LOGN, int P> struct BlockRadix {
-  static constexpr int K = (LOGN + 2) / 3;
+// radix (log2, at most LM) of pass P of the balanced schedule for a length 2^LOGN
+template <int LOGN, int LM, int P> struct BlockRadix {
+  static constexpr int K = (LOGN + LM - 1) / LM;
   static constexpr int LR = LOGN / K + (P < LOGN % K ? 1 : 0);
-  static constexpr int S = P == 0 ? 0 : BlockRadix<LOGN, (P > 0 ? P - 1 : 0)>::S + BlockRadix<LOGN, (P > 0 ? P - 1 : 0)>::LR;
-};
-template <int LOGN> struct BlockRadix<LOGN, 0> {
-  static constexpr int K = (LOGN + 2) / 3;
-  static constexpr int LR = LOGN / K + (0 < LOGN % K ? 1 : 0);
-  static constexpr int S = 0;
+  static constexpr int S = P * (LOGN / K) + (P < LOGN % K ? P : LOGN % K);   // bits done before it
 };
 
 template <typename T, bool INV, int LOGN, int P, typename Op>
 __device__ __forceinline__ void block_passes(C<T>* line, int t, int tpl, const C<T>* __restrict__ tw,
                                              int twlog, bool active, int lidx, const Op& op) {
-  constexpr int K = BlockRadix<LOGN, 0>::K;
+  using BR = BlockRadix<LOGN, FftE<T>::LRMAX, P>;
+  constexpr int K = BR::K;
   if constexpr (P < K) {
-    constexpr int LR = BlockRadix<LOGN, P>::LR;
-    constexpr int EPT = (1 << LOGN) / LineShape<T, LOGN>::TPL;   // 8, or 16 at 4096
+    constexpr int LR = BR::LR;
+    constexpr int EPT = (1 << LOGN) / LineShape<T, LOGN>::TPL;   // E, or more at 4096
     constexpr int PER = EPT >> LR;
-    fft_pass<T, INV, LR, PER, P == 0, P == K - 1, Op>(line, 1 << LOGN, BlockRadix<LOGN, P>::S, t,
-                                                      tpl, tw, twlog, active, lidx, op);
+    fft_pass<T, INV, LR, PER, P == 0, P == K - 1, Op>(line, 1 << LOGN, BR::S, t, tpl, tw, twlog,
+                                                      active, lidx, op);
     block_passes<T, INV, LOGN, P + 1, Op>(line, t, tpl, tw, twlog, active, lidx, op);
   }
 }
@@ -449,28 +448,38 @@ __device__ __forceinline__ void block_passes(C<T>* line, int t, int tpl, const C
 // In-place FFT of `nlines` padded lines (stride lstride) of the compile-time
 // length 2^LOGN: the warp transform where it applies, else the block
 // transform.  Called by all threads of the CTA; ends with a CTA barrier.
-template <typename T, bool INV, int LOGN, typename Op = LineId<T>>
+// ML > 0: there are at most ML lines, and the CTA has threads for all of them or
+// CT threads.  The loop over groups of lines is then unrolled
+// (one turn in most cases): inside a loop the compiler hoists addresses and
+// spills (pair-of-FP32 passes: 0.3-0.7 KB per thread with it, none without).
+template <typename T, bool INV, int LOGN, int ML = 0, int CT = FftE<T>::THREADS,
+          typename Op = LineId<T>>
 __device__ __forceinline__ void fft_lines(C<T>* base, int lstride, int nlines,
                                           const C<T>* __restrict__ tw, int twlog,
                                           const Op& op = Op()) {
   using S = LineShape<T, LOGN>;
   constexpr int n = 1 << LOGN, tpl = S::TPL;
   const int tid = threadIdx.x + threadIdx.y * blockDim.x;
-  const int nthr = blockDim.x * blockDim.y;
-  const int lpg = nthr >= tpl ? nthr / tpl : 1;
   const int lg = tid / tpl, t = tid - lg * tpl;
-  for (int l0 = 0; l0 < nlines; l0 += lpg) {
-    const int l = l0 + lg;
-    const bool active = lg < lpg && l < nlines;
+  auto group = [&](int l, bool active) {
     C<T>* line = base + (size_t)(active ? l : 0) * lstride;
     if constexpr (S::WARP) {
       fft_warp<T, INV, S::LW, S::RV, Op>(line, n, LOGN, t, active, tw, twlog, l, op);
-    } else if constexpr (LOGN <= 3) {
+    } else if constexpr (LOGN <= FftE<T>::LRMAX) {
       if constexpr (LOGN >= 1)
         fft_pass<T, INV, LOGN, 1, true, true, Op>(line, n, 0, t, tpl, tw, twlog, active, l, op);
     } else {
       block_passes<T, INV, LOGN, 0, Op>(line, t, tpl, tw, twlog, active, l, op);
     }
+  };
+  if constexpr (ML > 0) {
+    constexpr int NG = (ML * tpl + CT - 1) / CT, LPG = CT / tpl;
+#pragma unroll
+    for (int q = 0; q < NG; ++q) group(q * LPG + lg, q * LPG + lg < nlines);
+  } else {
+    const int nthr = blockDim.x * blockDim.y;
+    const int lpg = nthr >= tpl ? nthr / tpl : 1;
+    for (int l0 = 0; l0 < nlines; l0 += lpg) group(l0 + lg, lg < lpg && l0 + lg < nlines);
   }
   __syncthreads();
 }

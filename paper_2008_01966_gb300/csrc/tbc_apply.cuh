@@ -16,7 +16,8 @@
 // (6 to 25 FP32 instructions per operation) are bound by operations; operator
 // on one GB300, before and after: FP64 256 x 256, 6 vectors 6.43 -> 5.00 ms,
 // 512 x 512, 4 vectors 18.5 -> 14.2 ms, 1024 x 1024, 2 vectors 41.9 -> 32.0 ms;
-// pair, the same, 2.97 -> 2.34, 6.33 -> 5.07, 21.2 -> 17.2 ms.
+// pair, the same, 2.97 -> 2.34, 6.33 -> 5.07, 21.2 -> 17.2 ms (before the pair
+// type's own line shape, df64.cuh).
 // Four passes of batched line transforms in shared memory:
 //   A  (rows k1)   basis transform of E1, E2 along x2: FFT convolution of the
 //                  mirrored coefficients with the 1-D kernel E(nu) of F(F)
@@ -64,14 +65,18 @@ static TbcP make_params(const cavity_ctx* ctx) {
 template <typename T> __device__ __forceinline__ C<T> czero() { return mk<T>(0, 0); }
 
 // Lines per CTA: enough lines that a pass of the longest transform in the
-// kernel occupies LINES_THREADS threads (nlong = that length).
-#define LINES_THREADS 256
+// kernel occupies the CTA's threads (nlong = that length).
 template <typename T> __host__ __device__ constexpr int lines_per_cta(int nlong) {
-  return fft_tpl<T>(nlong) >= LINES_THREADS ? 1 : LINES_THREADS / fft_tpl<T>(nlong);
+  return fft_tpl<T>(nlong) >= FftE<T>::THREADS ? 1 : FftE<T>::THREADS / fft_tpl<T>(nlong);
+}
+// threads of a CTA of passes A and B: at 4096 points, where shared memory holds
+// one CTA per SM, both lines of a pair side by side
+template <typename T> __host__ __device__ constexpr int pair_threads(int n) {
+  return n < 4096 ? FftE<T>::THREADS : 2 * FftE<T>::THREADS;
 }
 // passes A and B hold two lines (parities r = 0, 1) per row / column
 template <typename T> __host__ __device__ constexpr int pairs_per_cta(int n) {
-  return 2 * fft_tpl<T>(n) >= LINES_THREADS ? 1 : LINES_THREADS / (2 * fft_tpl<T>(n));
+  return 2 * fft_tpl<T>(n) >= FftE<T>::THREADS ? 1 : FftE<T>::THREADS / (2 * fft_tpl<T>(n));
 }
 // These are the most lines of a CTA; a launch whose grid would not give every
 // SM two CTAs takes fewer (halved until it does, with the threads to match):
@@ -82,20 +87,18 @@ struct CtaLines {
   int lL, threads;
   unsigned blocks(int lines) const { return (unsigned)((lines + (1 << lL) - 1) >> lL); }
 };
-inline CtaLines cta_lines(int lL_max, int per_line, int tpl, long long lines, long long batch) {
+inline CtaLines cta_lines(int lL_max, int per_line, int tpl, int most, long long lines,
+                          long long batch) {
   const long long want = 2 * sm_count();
   int lL = lL_max;
   while (lL > 0 && ((lines + (1 << lL) - 1) >> lL) * batch < want) --lL;
-  return CtaLines{lL, std::min(LINES_THREADS, std::max(32, (per_line << lL) * tpl))};
+  return CtaLines{lL, std::min(most, std::max(32, (per_line << lL) * tpl))};
 }
-// registers: the pass kernels run two CTAs of LINES_THREADS per SM (the
-// pair-of-FP32 ones spill ~450 bytes per thread at this bound, but one CTA per
-// SM without spills was slower: pass B 10.6 ms against 7.6 ms)
-#define TBC_BOUNDS __launch_bounds__(LINES_THREADS, 2)
-// the same per grid size: with 4096-point lines (1024-point sides) a CTA's
-// lines take most of the shared memory, so one CTA per SM, with the whole
-// register file for the 16 points per thread of the block transform
-#define TBC_BOUNDS_LN(LN) __launch_bounds__(LINES_THREADS, (LN) >= 10 ? 1 : 2)
+// registers: the pass kernels run two CTAs per SM, but with 4096-point lines
+// (1024-point sides) a CTA's lines take most of the shared memory
+#define TBC_BOUNDS __launch_bounds__(FftE<T>::THREADS, 2)
+#define TBC_BOUNDS_LN(LN) __launch_bounds__(FftE<T>::THREADS, (LN) >= 10 ? 1 : 2)
+#define TBC_PAIR_BOUNDS(LN) __launch_bounds__(pair_threads<T>(4 << (LN)), (LN) >= 10 ? 1 : 2)
 
 // The pass kernels are instantiated per grid size: LNY = log2 ny (passes A,
 // C), LNX = log2 nx (passes B, D).  With the period pad = 4: Px = 4 nx,
@@ -175,7 +178,7 @@ struct ScatterA : LineId<T> {
 };
 
 template <typename T, int LNY>
-__global__ void TBC_BOUNDS_LN(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __restrict__ Vy, TbcP p,
+__global__ void TBC_PAIR_BOUNDS(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __restrict__ Vy, TbcP p,
                                   const C<T>* __restrict__ tw, const C<T>* __restrict__ eh_c,
                                   const C<T>* __restrict__ eh_s, int lL_) {
   extern __shared__ __align__(16) unsigned char sm_raw[];
@@ -200,8 +203,8 @@ __global__ void TBC_BOUNDS_LN(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __re
   fwd.L = L;
   fwd.ls = ls;
   fwd.buf = buf;
-  fft_lines<T, false, LPY>(buf, ls, L, tw, p.twlog, fwd);
-  fft_lines<T, true, LPY>(buf, ls, 2 * L, tw, p.twlog, sc);
+  fft_lines<T, false, LPY, pairs_per_cta<T>(Py), pair_threads<T>(Py)>(buf, ls, L, tw, p.twlog, fwd);
+  fft_lines<T, true, LPY, 2 * pairs_per_cta<T>(Py), pair_threads<T>(Py)>(buf, ls, 2 * L, tw, p.twlog, sc);
 }
 
 // ------------------------------------------------------------------ pass B
@@ -316,6 +319,7 @@ __device__ __forceinline__ void b_field(const C<T>* __restrict__ src, C<T>* __re
   C<T>* eh_sm = wl + (size_t)2 * L * S::lsh;
   const int tid = threadIdx.x, nthr = blockDim.x;
   constexpr bool xcos = F == 0;
+  constexpr int ML = 2 * pairs_per_cta<T>(Px), CT = pair_threads<T>(Px);
   if constexpr (S::STAGE) {
     for (int t = tid; t < 2 * Px; t += nthr) eh_sm[t] = eh[t];
   }
@@ -344,7 +348,7 @@ __device__ __forceinline__ void b_field(const C<T>* __restrict__ src, C<T>* __re
   fwd.L = L;
   fwd.ls = ls;
   fwd.buf = buf;
-  fft_lines<T, false, LPX>(buf, ls, L, tw, twlog, fwd);
+  fft_lines<T, false, LPX, pairs_per_cta<T>(Px), pair_threads<T>(Px)>(buf, ls, L, tw, twlog, fwd);
   KhatB<T, LNX, F, S::STAGE> kb;
   kb.kh = S::STAGE ? eh_sm + 2 * Px : kh;
   kb.wl = wl;
@@ -352,14 +356,14 @@ __device__ __forceinline__ void b_field(const C<T>* __restrict__ src, C<T>* __re
   kb.Py = Py;
   kb.L = L;
   kb.scale = scale;
-  fft_lines<T, true, LPX>(buf, ls, 2 * L, tw, twlog, kb);
-  fft_lines<T, true, LPX - 1>(buf, ls, 2 * L, tw, twlog);
+  fft_lines<T, true, LPX, ML, CT>(buf, ls, 2 * L, tw, twlog, kb);
+  fft_lines<T, true, LPX - 1, ML, CT>(buf, ls, 2 * L, tw, twlog);
   b_store<T, LNX, false>(buf, ls, dst, j0, Py, tw, twlog - LPX, lL);
   __syncthreads();
 }
 
 template <typename T, int LNX>
-__global__ void TBC_BOUNDS_LN(LNX) k_tbcB(const C<T>* __restrict__ Vy, C<T>* __restrict__ W, TbcP p,
+__global__ void TBC_PAIR_BOUNDS(LNX) k_tbcB(const C<T>* __restrict__ Vy, C<T>* __restrict__ W, TbcP p,
                                   const C<T>* __restrict__ tw, const C<T>* __restrict__ eh_c,
                                   const C<T>* __restrict__ eh_s, const C<T>* __restrict__ kh,
                                   T ax, T ay, int lL_) {
@@ -383,7 +387,7 @@ __global__ void TBC_BOUNDS_LN(LNX) k_tbcB(const C<T>* __restrict__ Vy, C<T>* __r
   C<T>* dst = W + (size_t)d * 3 * fs;
   b_field<T, LNX, 0>(src, dst, tw, eh_c, kh, j0, Py, p.twlog, ay, lL);
   b_field<T, LNX, 1>(src + (size_t)nx * Py, dst + fs, tw, eh_s, kh, j0, Py, p.twlog, ax, lL);
-  fft_lines<T, true, LPX - 1>(wl, S::lsh, 2 * L, tw, p.twlog);
+  fft_lines<T, true, LPX - 1, 2 * pairs_per_cta<T>(Px), pair_threads<T>(Px)>(wl, S::lsh, 2 * L, tw, p.twlog);
   b_store<T, LNX, true>(wl, S::lsh, dst + 2 * fs, j0, Py, tw, p.twlog - LPX, lL);
 }
 
@@ -442,11 +446,11 @@ __global__ void TBC_BOUNDS k_tbcB1(const C<T>* __restrict__ Vy, C<T>* __restrict
   ProdsB1<T, LNX> fwd;
   fwd.eh_c = eh_c;
   fwd.eh_s = eh_s;
-  fft_lines<T, false, LPX>(buf, 2 * ls, 2, tw, p.twlog, fwd);
+  fft_lines<T, false, LPX, 2>(buf, 2 * ls, 2, tw, p.twlog, fwd);
   KhatB1<T, LNX> kb;
   kb.kh = kh + (size_t)(dead ? 0 : (j2 < 0 ? -j2 : j2)) * (Px / 2);
   kb.dead = dead;
-  fft_lines<T, true, LPX>(buf, ls, 4, tw, p.twlog, kb);
+  fft_lines<T, true, LPX, 4>(buf, ls, 4, tw, p.twlog, kb);
   for (int idx = tid; idx < Px; idx += nthr) {
     const int r = idx / (Px / 2), u = idx % (Px / 2);
     const int j1 = 2 * (u < nx ? u : u - Px / 2) + r;
@@ -455,7 +459,7 @@ __global__ void TBC_BOUNDS k_tbcB1(const C<T>* __restrict__ Vy, C<T>* __restrict
         csub<T>(cscale<T>(g0, (T)j2 * ay), cscale<T>(g1, (T)j1 * ax));
   }
   __syncthreads();
-  fft_lines<T, true, LPX - 1>(buf, ls, 6, tw, p.twlog);
+  fft_lines<T, true, LPX - 1, 6>(buf, ls, 6, tw, p.twlog);
   for (int idx = tid; idx < 3 * (nx + 1); idx += nthr) {
     const int f = idx / (nx + 1), q = idx % (nx + 1);
     const C<T> z0 = buf[(size_t)(2 * f) * ls + pidx(q)], z1 = buf[(size_t)(2 * f + 1) * ls + pidx(q)];
@@ -525,14 +529,14 @@ __global__ void TBC_BOUNDS_LN(LNY) k_tbcC(const C<T>* __restrict__ W, C<T>* __re
   rc.r0 = r0;
   rc.nx = p.nx;
   rc.ycos = ycos;
-  fft_lines<T, true, LPY>(buf, ls, L, tw, p.twlog, rc);
+  fft_lines<T, true, LPY, lines_per_cta<T>(Py)>(buf, ls, L, tw, p.twlog, rc);
   StoreZ<T, LNY> sz;
   sz.Z = Z + (size_t)(d * 3 + f) * (p.nx + 1) * (ny + 1);
   sz.r0 = r0;
   sz.nx = p.nx;
   sz.ycos = ycos;
   sz.w = (T)p.wy;
-  fft_lines<T, false, LNY + 1>(buf, ls, L, tw, p.twlog, sz);
+  fft_lines<T, false, LNY + 1, lines_per_cta<T>(Py)>(buf, ls, L, tw, p.twlog, sz);
 }
 
 // ------------------------------------------------------------------ pass D
@@ -581,7 +585,7 @@ __global__ void TBC_BOUNDS_LN(LNX) k_tbcD(const C<T>* __restrict__ Z, C<T>* __re
   cd.ny = p.ny;
   cd.xcos = (f != 1);
   cd.w = (T)p.wx;
-  fft_lines<T, false, LNX + 1>(buf, ls, L, tw, p.twlog, cd);
+  fft_lines<T, false, LNX + 1, lines_per_cta<T>(n2)>(buf, ls, L, tw, p.twlog, cd);
 }
 
 // ------------------------------------------------------------------ combine
@@ -734,7 +738,8 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
   const C<T>* tw = Tabs<T>::tw(ctx);
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN), g.nx,
+    const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN),
+                                  pair_threads<T>(4 << LN), g.nx,
                                   2LL * ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcA<T, LN>, done));
@@ -750,14 +755,15 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
         static std::atomic<bool> done1{false};
         CKS(smem_once(ctx, k_tbcB1<T, LN>, done1));
         KScope ks_(ctx, kclass<T>(1));
-        k_tbcB1<T, LN><<<dim3(g.Py, ndir), std::max(64, std::min(LINES_THREADS, 6 * fft_tpl<T>(4 << LN))),
+        k_tbcB1<T, LN><<<dim3(g.Py, ndir), std::max(64, std::min(FftE<T>::THREADS, 6 * fft_tpl<T>(4 << LN))),
                          sizeof(C<T>) * 6 * (size_t)padded_len(4 << LN), st>>>(
             R1, R2, p, tw, Tabs<T>::ex(ctx, 0), Tabs<T>::ex(ctx, 1), Tabs<T>::kh(ctx),
             T(2.0 * M_PI / g.Lx), T(2.0 * M_PI / g.Ly));
         return CAVITY_OK;
       }
     }
-    const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN), g.Py,
+    const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN),
+                                  pair_threads<T>(4 << LN), g.Py,
                                   ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcB<T, LN>, done));
@@ -769,7 +775,8 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(4 << LN)), 1, fft_tpl<T>(4 << LN), g.nx + 1,
+    const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(4 << LN)), 1, fft_tpl<T>(4 << LN),
+                                  FftE<T>::THREADS, g.nx + 1,
                                   3LL * ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcC<T, LN>, done));
@@ -780,7 +787,8 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(2 << LN)), 1, fft_tpl<T>(2 << LN), g.ny + 1,
+    const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(2 << LN)), 1, fft_tpl<T>(2 << LN),
+                                  FftE<T>::THREADS, g.ny + 1,
                                   3LL * ndir);
     static std::atomic<bool> done{false};  // set once; host threads may race
     CKS(smem_once(ctx, k_tbcD<T, LN>, done));
