@@ -302,9 +302,12 @@ __device__ __forceinline__ void mma_tf32(float (&d)[4], const unsigned (&a)[4], 
 // buffers (row pitch 40 words: the fragment loads of a warp hit distinct
 // banks); warp w takes rows 16 w .. 16 w + 15 of each tile, and the four
 // warps' sums are added in warp order at the end.
+// NT: n8 tiles of W computed, 4 columns each: 2 where no group has more than 8
+// columns (512 x 512, 8 directions: 4.16 -> 3.84 ms a solve), else 4.
 #define TP_ROWS 64
 #define TP_LD 40
 #define TP_SMEM (sizeof(float) * 2 * 2 * TP_ROWS * TP_LD)
+template <int NT>
 __global__ void __launch_bounds__(128, 4) k_bproj_tc(BGSet set, double2* __restrict__ part, int nap,
                                                   int rs, int nct, int kcap) {
   extern __shared__ __align__(16) float tsm[];  // [buf][V | W][row][TP_LD]
@@ -327,16 +330,21 @@ __global__ void __launch_bounds__(128, 4) k_bproj_tc(BGSet set, double2* __restr
       const bool in = e < e1;
       const float2* src = i < Kv ? gd.V + (size_t)i * nap : gd.W + (size_t)(i - Kv) * nap;
       cp_async8((float2*)(vs + el * TP_LD + 2 * c), (in && i < K) ? src + e : gd.W, in && i < K);
-      cp_async8((float2*)(ws + el * TP_LD + 2 * c), (in && c < r) ? gd.W + (size_t)c * nap + e : gd.W,
-                in && c < r);
+    }
+#pragma unroll
+    for (int u = 0; u < 2 * NT; ++u) {   // 4 NT columns of W, row bits 2-5 from the top bits of q
+      const int q = tid + 128 * u, c = (q >> 2) & (4 * NT - 1), el = (q & 3) | ((q / (16 * NT)) << 2);
+      const int e = eb + el;
+      const bool in = e < e1 && c < r;
+      cp_async8((float2*)(ws + el * TP_LD + 2 * c), in ? gd.W + (size_t)c * nap + e : gd.W, in);
     }
     cp_async_commit();
   };
-  float acc[2][4][4];
+  float acc[2][NT][4];
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
       for (int q = 0; q < 4; ++q) acc[mt][nt][q] = 0.f;
   const int ntile = (e1 - e0 + TP_ROWS - 1) / TP_ROWS;
@@ -362,7 +370,7 @@ __global__ void __launch_bounds__(128, 4) k_bproj_tc(BGSet set, double2* __restr
         tf32_split(vs[eb * TP_LD + w0 + 8], ahi[mt][3], alo[mt][3]);
       }
 #pragma unroll
-      for (int nt = 0; nt < 4; ++nt) {
+      for (int nt = 0; nt < NT; ++nt) {
         unsigned bh0, bl0, bh1, bl1;
         tf32_split(ws[ea * TP_LD + 8 * nt + g], bh0, bl0);
         tf32_split(ws[eb * TP_LD + 8 * nt + g], bh1, bl1);
@@ -384,7 +392,7 @@ __global__ void __launch_bounds__(128, 4) k_bproj_tc(BGSet set, double2* __restr
 #pragma unroll
   for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt) {
+    for (int nt = 0; nt < NT; ++nt) {
       const int m = 16 * mt + g, n = 8 * nt + 2 * t;
       float* rw = red + warp * 32 * 33;
       rw[m * 33 + n] = acc[mt][nt][0];
@@ -406,6 +414,156 @@ __global__ void __launch_bounds__(128, 4) k_bproj_tc(BGSet set, double2* __restr
       pi += (double)rw[(2 * li) * 33 + 2 * lj + 1] - (double)rw[(2 * li + 1) * 33 + 2 * lj];
     }
     part[((size_t)(blockIdx.z * nct + blockIdx.x) * kcap + ib + li) * BG_MAX + lj] = make_double2(pr, pi);
+  }
+}
+
+// ------------------------------------------------------------ narrow blocks
+// Blocks of few columns (few directions in a call: one plane wave is one
+// column).  The tensor-core tiles are 16 columns wide, so these would multiply
+// mostly zeros and split every basis value into TF32 parts for them; per basis
+// value there are only 8 r FP32 operations, which the FP32 lanes do while the
+// basis streams through at the rate of memory.  Same set, partial sums and
+// results as the kernels above.  Up to BG_NARROW columns for the projection (its
+// sums of 8 basis columns fill the registers beyond that), up to BG_NARROW_UPD
+// for the update (at 16 the FP32 lanes would take as long as the tensor-core
+// kernel, 6.6 ms of operations against its 7.6 at 256 x 256, 64 directions).
+// Measured in a solve to 1e-10 on a GB300, tensor-core kernels and these:
+//   1024 x 1024, 3 directions: projections 11.1 -> 4.0 ms, updates 10.9 -> 3.6
+//   512 x 512, 8 directions:   updates 4.25 -> 2.93 ms
+//   whole solve, 512 x 512, 1 direction 11.5 -> 7.5 ms; 256 x 256, 1 direction
+//   5.0 -> 3.7 ms (pair operator 0.2 and 0.1 ms of it)
+#define BG_NARROW 4
+#define BG_NARROW_UPD 8
+
+// update: one thread per two rows, the group's coefficients in shared memory
+template <int RN>
+__global__ void __launch_bounds__(256) k_bnn_narrow(BGSet set, const double2* __restrict__ cmat,
+                                                    int nap, float beta, float sgn) {
+  extern __shared__ float2 ncs[];   // [Kv][RN]
+  const BGrp& gd = set.g[blockIdx.z];
+  const int Kv = gd.Kv, r = gd.r, n = gd.n, tid = threadIdx.x;
+  const int row0 = blockIdx.x * 512;
+  if (row0 >= n) return;  // uniform over the block
+  const double2* Cm = cmat + gd.coff;
+  for (int i = tid; i < Kv * RN; i += 256) {
+    const int q = i / RN, j = i % RN;
+    const double2 c = j < r ? Cm[(size_t)q * BG_MAX + j] : make_double2(0.0, 0.0);
+    ncs[i] = make_float2((float)(sgn * c.x), (float)(sgn * c.y));
+  }
+  __syncthreads();
+  const int e0 = row0 + tid, e1 = e0 + 256;
+  const float2* v0 = gd.V + min(e0, n - 1);
+  const float2* v1 = gd.V + min(e1, n - 1);
+  float2 a0[RN], a1[RN];
+#pragma unroll
+  for (int j = 0; j < RN; ++j) a0[j] = a1[j] = make_float2(0.f, 0.f);
+  auto add = [&](float2 x, float2 y, const float2* c) {
+#pragma unroll
+    for (int j = 0; j < RN; ++j) {
+      const float2 w = c[j];
+      a0[j].x = fmaf(x.x, w.x, fmaf(-x.y, w.y, a0[j].x));
+      a0[j].y = fmaf(x.x, w.y, fmaf(x.y, w.x, a0[j].y));
+      a1[j].x = fmaf(y.x, w.x, fmaf(-y.y, w.y, a1[j].x));
+      a1[j].y = fmaf(y.x, w.y, fmaf(y.y, w.x, a1[j].y));
+    }
+  };
+  int i = 0;
+  for (; i + 8 <= Kv; i += 8) {
+    float2 x[8], y[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      x[u] = v0[(size_t)(i + u) * nap];
+      y[u] = v1[(size_t)(i + u) * nap];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u) add(x[u], y[u], ncs + (i + u) * RN);
+  }
+  for (; i < Kv; ++i) add(v0[(size_t)i * nap], v1[(size_t)i * nap], ncs + i * RN);
+#pragma unroll
+  for (int j = 0; j < RN; ++j) {
+    if (j >= r) break;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int e = h ? e1 : e0;
+      if (e >= n) break;
+      const float2 s = h ? a1[j] : a0[j];
+      const float2 o = beta != 0.f ? gd.W[(size_t)j * nap + e] : make_float2(0.f, 0.f);
+      gd.O[(size_t)j * nap + e] = make_float2(fmaf(beta, o.x, s.x), fmaf(beta, o.y, s.y));
+    }
+  }
+}
+
+// projection: a block takes NP_KC basis columns against all block columns over
+// its slab, each thread its rows in FP32; the threads' sums are added by a
+// halving exchange within the warp, the warps' in FP64
+#define NP_KC 8
+template <int RN>
+__global__ void __launch_bounds__(128, 4) k_bproj_narrow(BGSet set, double2* __restrict__ part,
+                                                         int nap, int rs, int nct, int kcap) {
+  constexpr int NV = NP_KC * RN * 2;
+  __shared__ float red[4][NV];
+  const BGrp& gd = set.g[blockIdx.z];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int ib = blockIdx.y * NP_KC, K = gd.K, Kv = gd.Kv, r = gd.r;
+  if (ib >= K) return;  // uniform over the block
+  const int e0 = blockIdx.x * rs, e1 = min(gd.n, e0 + rs);
+  const float2* src[NP_KC];
+#pragma unroll
+  for (int u = 0; u < NP_KC; ++u) {
+    const int i = min(ib + u, K - 1);
+    src[u] = i < Kv ? gd.V + (size_t)i * nap : gd.W + (size_t)(i - Kv) * nap;
+  }
+  float acc[NV];   // [u][j][re, im]
+#pragma unroll
+  for (int q = 0; q < NV; ++q) acc[q] = 0.f;
+  for (int e = e0 + tid; e < e1; e += 128) {
+    float2 x[NP_KC], w[RN];
+#pragma unroll
+    for (int u = 0; u < NP_KC; ++u) x[u] = __ldg(src[u] + e);
+#pragma unroll
+    for (int j = 0; j < RN; ++j) w[j] = __ldg(gd.W + (size_t)min(j, r - 1) * nap + e);
+#pragma unroll
+    for (int u = 0; u < NP_KC; ++u)
+#pragma unroll
+      for (int j = 0; j < RN; ++j) {   // conj(x) w
+        float* a = acc + (u * RN + j) * 2;
+        a[0] = fmaf(x[u].x, w[j].x, fmaf(x[u].y, w[j].y, a[0]));
+        a[1] = fmaf(x[u].x, w[j].y, fmaf(-x[u].y, w[j].x, a[1]));
+      }
+  }
+  // lane exchange: while the count is even, a lane keeps one half of the sums
+  int base = 0;
+  auto step = [&](auto cnt, int o) {
+    constexpr int H = decltype(cnt)::value / 2;
+    const bool up = lane & o;
+#pragma unroll
+    for (int k = 0; k < H; ++k) {
+      const float keep = up ? acc[k + H] : acc[k], send = up ? acc[k] : acc[k + H];
+      acc[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
+    base += up ? H : 0;
+  };
+  step(std::integral_constant<int, NV>{}, 16);
+  step(std::integral_constant<int, NV / 2>{}, 8);
+  step(std::integral_constant<int, NV / 4>{}, 4);
+  step(std::integral_constant<int, NV / 8>{}, 2);
+  constexpr int L = NV / 16;   // RN sums are left
+#pragma unroll
+  for (int k = 0; k < L; ++k) {
+    acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], 1);
+    if (!(lane & 1)) red[warp][base + k] = acc[k];
+  }
+  __syncthreads();
+  for (int q = tid; q < NP_KC * RN; q += 128) {
+    const int u = q / RN, j = q % RN;
+    if (ib + u >= K || j >= r) continue;
+    double pr = 0, pi = 0;
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      pr += (double)red[w][2 * q];
+      pi += (double)red[w][2 * q + 1];
+    }
+    part[((size_t)(blockIdx.z * nct + blockIdx.x) * kcap + ib + u) * BG_MAX + j] = make_double2(pr, pi);
   }
 }
 
@@ -531,11 +689,30 @@ static int max_rows(const BGSet& set, int ng) {
   return n;
 }
 
+static int max_r(const BGSet& set, int ng) {
+  int r = 0;
+  for (int t = 0; t < ng; ++t) r = std::max(r, set.g[t].r);
+  return r;
+}
+// f(RN) with RN >= r a compile-time constant, 1 <= r <= MOST (4 or 8)
+template <int MOST, typename F> static void narrow_dispatch(int r, F f) {
+  if (r == 1) f(std::integral_constant<int, 1>{});
+  else if (r == 2) f(std::integral_constant<int, 2>{});
+  else if (r == 3) f(std::integral_constant<int, 3>{});
+  else if (MOST == 4 || r == 4) f(std::integral_constant<int, 4>{});
+  else if constexpr (MOST == 8) {
+    if (r <= 6) f(std::integral_constant<int, 6>{});
+    else f(std::integral_constant<int, 8>{});
+  }
+}
+
 // V^H W for every system of `set` (ng of them, K and r each) into
 // hb + slot * emax * kcap * BG_MAX, laid out [z][i][j].
 static void bproj(cavity_ctx* ctx, const BGSet& set, int ng, int kmax, const BWork& w, int slot) {
   const int nap = ctx->g.nap, nrow = max_rows(set, ng);
-  const int ytiles = (kmax + 15) / 16;
+  const int rm = max_r(set, ng);
+  const bool narrow = rm <= BG_NARROW;
+  const int ytiles = narrow ? (kmax + NP_KC - 1) / NP_KC : (kmax + 15) / 16;
   // slabs of rows such that slabs x column tiles x groups fill one wave of
   // resident blocks (four per SM, BG_PART_CTAS in all): no tail wave, and a
   // short projection (the Gram matrix, K = 16) still spreads over every SM
@@ -547,13 +724,24 @@ static void bproj(cavity_ctx* ctx, const BGSet& set, int ng, int kmax, const BWo
   double2* h = w.hb + (size_t)slot * w.emax * w.kcap * BG_MAX;
   static std::atomic<bool> done{false};  // set once; host threads may race
   if (!done) {
-    cudaFuncSetAttribute(k_bproj_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TP_SMEM);
+    cudaFuncSetAttribute(k_bproj_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TP_SMEM);
+    cudaFuncSetAttribute(k_bproj_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TP_SMEM);
     done = true;
   }
-  {
+  if (narrow) {
     KScope ks_(ctx, KC_KRYLOV);
-    k_bproj_tc<<<dim3(nct, ytiles, ng), 128, TP_SMEM, ctx->stream>>>(set, w.part, nap, rs, nct,
-                                                                     w.kcap);
+    narrow_dispatch<BG_NARROW>(rm, [&](auto c) {
+      k_bproj_narrow<decltype(c)::value><<<dim3(nct, ytiles, ng), 128, 0, ctx->stream>>>(
+          set, w.part, nap, rs, nct, w.kcap);
+    });
+  } else {
+    KScope ks_(ctx, KC_KRYLOV);
+    if (rm <= 8)
+      k_bproj_tc<2><<<dim3(nct, ytiles, ng), 128, TP_SMEM, ctx->stream>>>(set, w.part, nap, rs, nct,
+                                                                          w.kcap);
+    else
+      k_bproj_tc<4><<<dim3(nct, ytiles, ng), 128, TP_SMEM, ctx->stream>>>(set, w.part, nap, rs, nct,
+                                                                          w.kcap);
   }
   {
     KScope ks_(ctx, KC_KRYLOV);
@@ -565,6 +753,17 @@ static cavity_status bnn(cavity_ctx* ctx, const BGSet& set, int ng, const double
                          float sgn) {
   const int nap = ctx->g.nap;
   KScope ks_(ctx, KC_KRYLOV);
+  const int rm = max_r(set, ng);
+  if (rm <= BG_NARROW_UPD) {
+    int kv = 0;
+    for (int t = 0; t < ng; ++t) kv = std::max(kv, set.g[t].Kv);
+    narrow_dispatch<BG_NARROW_UPD>(rm, [&](auto c) {
+      constexpr int RN = decltype(c)::value;
+      k_bnn_narrow<RN><<<dim3(bg_blocks(max_rows(set, ng), 512), 1, ng), 256,
+                         sizeof(float2) * RN * kv, ctx->stream>>>(set, cmat, nap, beta, sgn);
+    });
+    return CAVITY_OK;
+  }
   k_bnn_tc5<<<dim3(bg_blocks(max_rows(set, ng), 128), 1, ng), 128, 2 * sizeof(T5Buf), ctx->stream>>>(
       set, cmat, nap, beta, sgn);
   return CAVITY_OK;
