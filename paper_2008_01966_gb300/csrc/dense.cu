@@ -742,6 +742,210 @@ __global__ void __launch_bounds__(LU_THREADS) k_lu_panel(float2* __restrict__ A,
   }
 }
 
+// The same panel by one cluster of CL CTAs, for panels of at most CL * 192
+// rows.  A column of k_lu_panel costs a grid-wide barrier and three trips
+// through L2, 3.4 us whatever the rows, and a pass over the rows in shared
+// memory.  Here a column waits for one hardware cluster barrier (0.35 us), and
+// the rows live in registers: thread (k, g) holds column k of rows g, g + 8, ...,
+// so that the elimination reads only the multipliers and the pivot row.
+//   (1) every warp finds the CTA's best key from column j in shared memory;
+//   (2) the threads that hold them leave the candidate row and (one CTA) the
+//       diagonal row in shared memory, and the key and those rows' entries of
+//       column j go to all CTAs; cluster barrier;
+//   (3) every warp finds the winner among the CL keys; the pivot row (and,
+//       where row p lives, the old row kj) is fetched from its CTA while the
+//       multipliers are formed; the rows are exchanged, the rows below
+//       eliminated, and column j + 1 goes to shared memory.
+// What a column leaves for other CTAs is written again two columns later, by
+// when they have passed the barrier in between.  The same pivots and the same
+// operations on every entry as k_lu_panel.
+// Measured on a GB300, us per column of a panel, k_lu_panel and this one: 3.4 and
+// 2.6 at 1024-2048 rows, 2.0 at 512-1024, 1.5 below; 2,080 unknowns in all 6.9 and
+// 4.6 ms.  With the rows in shared memory the elimination alone took 0.9 us of
+// a column at 2,080 rows.
+#define LUC_THREADS 512
+__device__ __forceinline__ uint32_t luc_addr(const void* p, int rank) {
+  uint32_t r;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;"
+      : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+// two entries from the shared memory of a CTA of the cluster
+__device__ __forceinline__ void luc_get(float2* d, uint32_t a) {
+  float4 x;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w) : "r"(a) : "memory");
+  *(float4*)d = x;
+}
+__device__ __forceinline__ void luc_bar() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// largest key of a warp: the high words, then the low words beside the largest
+__device__ __forceinline__ unsigned long long luc_max(unsigned long long key) {
+  const unsigned hi = (unsigned)(key >> 32), m = __reduce_max_sync(0xffffffffu, hi);
+  const unsigned lo = __reduce_max_sync(0xffffffffu, hi == m ? (unsigned)key : 0u);
+  return ((unsigned long long)m << 32) | lo;
+}
+template <int RQ> __device__ __forceinline__ float2 luc_pick(const float2 (&v)[RQ], int q) {
+  float2 x = v[0];
+#pragma unroll
+  for (int u = 1; u < RQ; ++u)
+    if (u == q) x = v[u];
+  return x;
+}
+template <int RQ> __device__ __forceinline__ void luc_put(float2 (&v)[RQ], int q, float2 x) {
+#pragma unroll
+  for (int u = 0; u < RQ; ++u)
+    if (u == q) v[u] = x;
+}
+// R <= 8 RQ rows per CTA
+template <int CL, int RQ>
+__global__ void __launch_bounds__(LUC_THREADS)
+    k_lu_panel_cluster(float2* __restrict__ A, int lda, int n, int k0, int nb, int R,
+                       int* __restrict__ ipiv, int* __restrict__ err) {
+  __shared__ __align__(16) float2 cand[2][LU_NB], drow[2][LU_NB];   // read by the other CTAs
+  __shared__ __align__(16) ulonglong2 keys[2][CL];   // written by them: key, candidate's column j
+  __shared__ float2 diag_j[2];                       // and the diagonal row's
+  __shared__ __align__(16) float2 prow[LU_NB], dr[LU_NB];   // pivot row, old row kj
+  __shared__ float2 col[2][8 * RQ];                  // column j, then its multipliers
+  const int c = blockIdx.x, t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int k = t & (LU_NB - 1), g = t / LU_NB;
+  const int r0 = k0 + c * R, r1 = min(r0 + R, n), nr = max(r1 - r0, 0);
+  float2 v[RQ];
+#pragma unroll
+  for (int q = 0; q < RQ; ++q) {
+    const int i = g + 8 * q;
+    v[q] = i < nr && k < nb ? A[(size_t)(r0 + i) * lda + k0 + k] : make_float2(0.f, 0.f);
+    if (k == 0) col[0][i] = v[q];
+  }
+  luc_bar();   // every CTA of the cluster runs, and column 0 is complete
+  for (int j = 0; j < nb; ++j) {
+    const int kj = k0 + j, par = j & 1;
+    const bool diag = kj >= r0 && kj < r1;   // the diagonal row is here
+    unsigned long long own = 0;
+    for (int i = max(kj - r0, 0) + lane; i < nr; i += 32) {
+      const float2 x = col[par][i];
+      const unsigned long long kk = lu_key(x.x * x.x + x.y * x.y, r0 + i);
+      own = kk > own ? kk : own;
+    }
+    own = luc_max(own);
+    const int br = own ? (int)(~(unsigned int)(own & 0xffffffffu)) - r0 : -1, bd = kj - r0;
+    if (br >= 0 && g == (br & 7)) cand[par][k] = luc_pick<RQ>(v, br >> 3);
+    if (diag && g == (bd & 7)) drow[par][k] = luc_pick<RQ>(v, bd >> 3);
+    if (t < CL) {
+      const float2 x = col[par][max(br, 0)];
+      asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};"
+                   :: "r"(luc_addr(&keys[par][c], t)), "r"((unsigned)own), "r"((unsigned)(own >> 32)),
+                      "r"(__float_as_uint(x.x)), "r"(__float_as_uint(x.y)) : "memory");
+      if (diag) {
+        const float2 y = col[par][bd];
+        asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};"
+                     :: "r"(luc_addr(&diag_j[par], t)), "f"(y.x), "f"(y.y) : "memory");
+      }
+    }
+    luc_bar();
+    const unsigned long long best = luc_max(lane < CL ? keys[par][lane].x : 0ull);
+    const int p = (int)(~(unsigned int)(best & 0xffffffffu)), w = (p - k0) / R;
+    const bool here = p >= r0 && p < r1;
+    // the two rows on their way; meanwhile the multipliers, for which the pivot
+    // and the diagonal row's entry are here already
+    if (warp == 0) luc_get(prow + 2 * lane, luc_addr(&cand[par][2 * lane], w));
+    if (warp == 1 && here) luc_get(dr + 2 * lane, luc_addr(&drow[par][2 * lane], j / R));
+    const int i0 = max(bd + 1, 0);
+    {
+      const unsigned long long z = keys[par][w].y;
+      const float2 pv = make_float2(__uint_as_float((unsigned)z), __uint_as_float((unsigned)(z >> 32)));
+      float2 pinv = make_float2(0.f, 0.f);
+      if (pv.x != 0.f || pv.y != 0.f) pinv = cdiv<float>(make_float2(1.f, 0.f), pv);
+      for (int i = i0 + t; i < nr; i += LUC_THREADS)
+        col[par][i] = cmul<float>(r0 + i == p ? diag_j[par] : col[par][i], pinv);
+      if (c == 0 && t == 0) {
+        if (pv.x == 0.f && pv.y == 0.f) atomicMin(&err[1], kj);
+        ipiv[kj] = p;
+      }
+    }
+    __syncthreads();
+    // row kj takes the pivot row, row p the old row kj
+    if (diag && g == (bd & 7)) luc_put<RQ>(v, bd >> 3, prow[k]);
+    if (here && p != kj && g == ((p - r0) & 7)) luc_put<RQ>(v, (p - r0) >> 3, dr[k]);
+    // elimination below the pivot (a warp whose columns are all done has none);
+    // selects instead of branches keep the reads of the multipliers in flight
+    if (k >= j) {
+      const float2 pk = prow[k];
+#pragma unroll
+      for (int q = 0; q < RQ; ++q) {
+        const int i = g + 8 * q;
+        const float2 l = col[par][i], x = csub<float>(v[q], cmul<float>(l, pk));
+        const float2 y = k == j ? l : x;
+        v[q].x = i >= i0 ? y.x : v[q].x;
+        v[q].y = i >= i0 ? y.y : v[q].y;
+      }
+      if (k == j + 1) {
+#pragma unroll
+        for (int q = 0; q < RQ; ++q) col[par ^ 1][g + 8 * q] = v[q];
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int q = 0; q < RQ; ++q) {
+    const int i = g + 8 * q;
+    if (i < nr && k < nb) A[(size_t)(r0 + i) * lda + k0 + k] = v[q];
+  }
+  luc_bar();   // the others have read this CTA's rows
+}
+template <int CL, int RQ>
+static cudaError_t luc_launch(cudaStream_t st, int R, float2* a, int lda, int n, int k0, int nb,
+                              int* ipiv, int* err, int* active) {
+  cudaLaunchConfig_t c = {};
+  cudaLaunchAttribute at;
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = CL;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  c.gridDim = dim3(CL);
+  c.blockDim = dim3(LUC_THREADS);
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  auto kern = k_lu_panel_cluster<CL, RQ>;
+  if (active) {   // how many such clusters the device holds
+    if (CL > 8) {
+      const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
+    return cudaOccupancyMaxActiveClusters(active, kern, &c);
+  }
+  return cudaLaunchKernelEx(&c, kern, a, lda, n, k0, nb, R, ipiv, err);
+}
+// rows per thread by the rows per CTA
+template <int CL>
+static cudaError_t luc_dispatch(cudaStream_t st, int R, float2* a, int lda, int n, int k0, int nb,
+                                int* ipiv, int* err, int* active) {
+  if (R <= 32) return luc_launch<CL, 4>(st, R, a, lda, n, k0, nb, ipiv, err, active);
+  if (R <= 64) return luc_launch<CL, 8>(st, R, a, lda, n, k0, nb, ipiv, err, active);
+  if (R <= 128) return luc_launch<CL, 16>(st, R, a, lda, n, k0, nb, ipiv, err, active);
+  return luc_launch<CL, 24>(st, R, a, lda, n, k0, nb, ipiv, err, active);
+}
+#define LUC_RMAX 192   // 24 rows a thread; 32 spill
+// cluster size of the panels: 16 (a non-portable size) where the device runs it,
+// else 8, else 0 (none); asked once per process
+static int luc_cluster() {
+  static std::atomic<int> known{-1};
+  if (known >= 0) return known;
+  auto runs = [](auto dispatch) {
+    for (int R : {32, 64, 128, LUC_RMAX}) {
+      int m = 0;
+      if (dispatch(nullptr, R, nullptr, 0, 0, 0, 0, nullptr, nullptr, &m) != cudaSuccess || m < 1)
+        return false;
+    }
+    return true;
+  };
+  const int k = runs(luc_dispatch<16>) ? 16 : runs(luc_dispatch<8>) ? 8 : 0;
+  cudaGetLastError();   // a refused attribute is an answer, not an error
+  known = k;
+  return k;
+}
+
 // the panel's row exchanges on every column outside it
 __global__ void k_lu_swap(float2* __restrict__ A, int lda, int n, int k0, int nb,
                           const int* __restrict__ ipiv) {
@@ -844,9 +1048,13 @@ cavity_status dense_lu(cavity_ctx* ctx, float2* a, int n, int lda, int* ipiv, in
   }
   for (int p = 0; p < npanel; ++p) {
     const int k0 = p * LU_NB, nb = std::min(LU_NB, n - k0), H = n - k0;
-    const int G = nblk(H, LU_RMAX), R = nblk(H, G);
-    unsigned int* bar = s.bar + p;
-    {
+    const int cl = luc_cluster(), RC = cl ? nblk(H, cl) : 0;
+    if (cl && RC <= LUC_RMAX) {
+      KScope ks_(ctx, KC_DENSE_LU);
+      CK((cl == 16 ? luc_dispatch<16> : luc_dispatch<8>)(st, RC, a, lda, n, k0, nb, ipiv, s.err, nullptr));
+    } else {
+      const int G = nblk(H, LU_RMAX), R = nblk(H, G);
+      unsigned int* bar = s.bar + p;
       KScope ks_(ctx, KC_DENSE_LU);
       void* args[] = {&a, &lda, &n, (void*)&k0, (void*)&nb, (void*)&R, &ipiv, &s, &bar};
       CK(cudaLaunchCooperativeKernel((const void*)k_lu_panel, dim3(G), dim3(LU_THREADS), args,
