@@ -66,10 +66,7 @@ REF_ITERS = {"layered4": 31, "dirs16": 37}
 # capture, per launch of the benchmark (scaled by directions where the
 # capture had fewer; traffic is proportional to the directions).  Only valid
 # for the kernel as captured: emptied whenever the kernel changes.
-NCU_TRAFFIC = {("dirs16", "tbc_B_fp32"): 2 * (52.550656e6 + 21.679616e6),
-               # one 8-direction launch of the 512^2 pass B (16-level case of
-               # the same kernel; the pass does not depend on the depth)
-               ("layered4", "tbc_B_fp32"): 210.693376e6 + 169.210624e6}
+NCU_TRAFFIC = {}
 # FP64 FMA throughput measured on a GB300 with a throughput kernel (16
 # independent FMA chains per thread, 8 blocks of 256 threads per SM, CUDA
 # events, best of 5): 1.254 TFLOP/s (FP32 by the same kernel: 78.4 TFLOP/s).
@@ -142,7 +139,8 @@ class ClockSampler:
 def alg_flops_per_launch(cls, w, ndir):
     """Algorithmic FP flops per launch of a TBC pass (5 n log2 n per complex
     FFT of length n, 6 per complex multiply), for the batch of ndir
-    directions and the three convolution fields."""
+    directions, with every one of the three convolution fields taken through
+    the basis transforms (executed_share: what the passes run of it)."""
     nx, ny = w['nx'], w['ny']
     Px, Py = 4 * nx, 4 * ny
     lg = np.log2
@@ -164,6 +162,21 @@ def alg_flops_per_launch(cls, w, ndir):
     return None
 
 
+def executed_share(cls, w):
+    """Share of alg_flops_per_launch that passes A and B run: the third field's
+    basis transform follows pointwise from those of the other two, so two of
+    three fields take the transforms and products before the kernel table's,
+    and all three the last half-length ones."""
+    if cls.startswith("tbc_A"):
+        return 2.0 / 3.0
+    if cls.startswith("tbc_B"):
+        nx, Px = w['nx'], 4 * w['nx']
+        basis = 3 * 5.0 * Px * np.log2(Px) + 18 * Px
+        last = 2 * 5.0 * (Px // 2) * np.log2(Px // 2) + 8 * (nx + 1)
+        return (2 * basis + 3 * last) / (3 * (basis + last))
+    return 1.0
+
+
 def fp_peak_tflops(cls, sm_mhz):
     """ALU peaks: FP64 from the measured FMA throughput (the nominal GB300
     figure 1.25 TFLOP/s until measured); FP32 derived as 152 SMs x 128 FP32
@@ -182,6 +195,7 @@ def class_roofline(cls, cms, ccnt, w, ndir, sm_mhz, workload):
     flops = alg_flops_per_launch(cls, w, ndir)
     if flops is None or ccnt <= 0 or cms <= 0:
         return None
+    flops *= executed_share(cls, w)
     per_launch_s = cms / ccnt / 1e3
     ach = flops / per_launch_s / 1e12
     pk, pk_kind = fp_peak_tflops(cls, sm_mhz)
