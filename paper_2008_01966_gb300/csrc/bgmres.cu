@@ -12,7 +12,8 @@
 //
 // Orthogonalisation of the new block W against the basis V: one classical
 // Gram-Schmidt pass as two GEMM-shaped tensor-core kernels, TF32 operands
-// split into three products for FP32 accuracy.  W -= V H (k_bnn_tc5) runs on
+// split into three products for FP32 accuracy.  (Blocks of few columns
+// take kernels on the FP32 lanes, further down.)  W -= V H (k_bnn_tc5) runs on
 // the fifth-generation tensor cores (tcgen05.mma kind::tf32, accumulators in
 // tensor memory; tc05.cuh).  V^H W is a split reduction over the rows
 // (k_bproj_tc, then k_bproj_final in a fixed order) on warp-level mma.sync: a
