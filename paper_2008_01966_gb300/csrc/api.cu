@@ -201,12 +201,13 @@ extern "C" cavity_status cavity_prepare(cavity_ctx* ctx, double kappa0, int nlay
   ctx->prepared = false;
   ctx->dn.ready = false;
   ctx->cs.ready = false;
-  bool kappa_same = ctx->khat64 && ctx->kappa0 == kappa0;
   ctx->kappa0 = kappa0;
   ctx->layers = L;
-  if (!kappa_same) {
+  if (ctx->khat_kappa != kappa0) {
+    ctx->khat_kappa = 0;   // a call that fails here leaves no table that counts as made
     CKS(launch_khat(ctx, kappa0));
     if (ctx->g.fft_ok) CKS(launch_khat_split(ctx));
+    ctx->khat_kappa = kappa0;
   }
   CKS(launch_zsweep(ctx, kappa0));
   if (ctx->g.fft_ok) {   // the Krylov path's preconditioner and operator tables

@@ -172,6 +172,7 @@ struct cavity_ctx {
   float2 *ehat_x32[2] = {nullptr, nullptr}, *ehat_y32[2] = {nullptr, nullptr};
   // the same tables in pair-of-FP32 form (struct cdf, 16 bytes per entry) for
   // the residual operator of the mixed solve
+  bool pair_ready = false;     // all of these are made
   void* tw_p = nullptr;
   void *ehat_xp[2] = {nullptr, nullptr}, *ehat_yp[2] = {nullptr, nullptr};
 
@@ -179,6 +180,7 @@ struct cavity_ctx {
   bool prepared = false;
   double kappa0 = 0;
   std::vector<LayerDev> layers;
+  double khat_kappa = 0;       // wavenumber of the kernel tables, 0 until all of them are made
   double2* khat64 = nullptr;   // quarter box [j2][j1] (Py/2 x Px/2), scaled by 1/(Lx Ly)
   float2* khat32 = nullptr;
   float2* khat32s = nullptr;   // khat32 by parity of j1 for the FP32 passes (tbc_f32.cu)
@@ -264,10 +266,13 @@ struct KScope {
 };
 
 // ------------------------------------------------------------ errors
+// (the runtime remembers a failed call until it is asked; without asking here,
+// the check after the next launches would report it once more)
 #define CK(call)                                                                 \
   do {                                                                           \
     cudaError_t e_ = (call);                                                     \
     if (e_ != cudaSuccess) {                                                     \
+      cudaGetLastError();                                                        \
       ctx->err = std::string(#call) + ": " + cudaGetErrorString(e_);             \
       return CAVITY_ECUDA;                                                       \
     }                                                                            \
@@ -325,6 +330,7 @@ inline cavity_status ensure_pin(cavity_ctx* ctx, size_t bytes) {
   ctx->pin_bytes = 0;
   cudaError_t e = cudaMallocHost(&ctx->pin, bytes);
   if (e != cudaSuccess) {
+    cudaGetLastError();
     ctx->pin = nullptr;
     ctx->err = "pinned staging allocation of " + std::to_string(bytes) + " bytes failed: " +
                cudaGetErrorString(e);
@@ -342,6 +348,7 @@ inline cavity_status ensure_ws(cavity_ctx* ctx, void** p, size_t* have, size_t b
   *have = 0;
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
+    cudaGetLastError();
     *p = nullptr;
     ctx->err = "workspace allocation of " + std::to_string(bytes) + " bytes failed: " +
                cudaGetErrorString(e);
@@ -349,6 +356,13 @@ inline cavity_status ensure_ws(cavity_ctx* ctx, void** p, size_t* have, size_t b
   }
   *have = bytes;
   return CAVITY_OK;
+}
+
+// device memory of a table that lives with the context, allocated the first
+// time it is needed.  Each pointer stands for itself: a call that fails in the
+// middle of several leaves the rest to the next call.
+template <typename T> inline cudaError_t table_alloc(T** p, size_t n) {
+  return *p ? cudaSuccess : cudaMalloc(p, sizeof(T) * n);
 }
 
 // ------------------------------------------------------------ step launchers

@@ -401,11 +401,9 @@ cavity_status launch_khat(cavity_ctx* ctx, double kappa0) {
   lock.unlock();
   const int hx = g.Px / 2, hy = g.Py / 2;
   size_t n = (size_t)hx * hy;
-  if (!ctx->khat64) {
-    CK(cudaMalloc(&ctx->khat64, sizeof(double2) * n));
-    CK(cudaMalloc(&ctx->khat32, sizeof(float2) * n));
-    CK(cudaMalloc(&ctx->khat_raw, sizeof(double2) * n));
-  }
+  CK(table_alloc(&ctx->khat64, n));
+  CK(table_alloc(&ctx->khat32, n));
+  CK(table_alloc(&ctx->khat_raw, n));
   const long long threads = (long long)n * 32;
   {
     KScope ks_(ctx, KC_SETUP);

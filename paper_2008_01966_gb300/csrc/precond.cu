@@ -188,10 +188,8 @@ cavity_status launch_precond(cavity_ctx* ctx) {
   double2* dd = T + nT;
   double* ax = (double*)(dd + nd);
   double* ay = ax + nax;
-  if (!ctx->pinv64) {
-    CK(cudaMalloc(&ctx->pinv64, sizeof(double2) * 9 * (size_t)g.nx * g.ny));
-    CK(cudaMalloc(&ctx->pinv32, sizeof(float2) * 9 * (size_t)g.nx * g.ny));
-  }
+  CK(table_alloc(&ctx->pinv64, 9 * (size_t)g.nx * g.ny));
+  CK(table_alloc(&ctx->pinv32, 9 * (size_t)g.nx * g.ny));
   cudaStream_t st = ctx->stream;
   {
     KScope ks_(ctx, KC_SETUP);

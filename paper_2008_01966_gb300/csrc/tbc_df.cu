@@ -55,12 +55,13 @@ static cavity_status to_pair(cavity_ctx* ctx, const double2* a, void** dst, long
 // of the kernel table and top relations (every prepare)
 cavity_status launch_pair_tables(cavity_ctx* ctx) {
   const Geo& g = ctx->g;
-  if (!ctx->tw_p) {
+  if (!ctx->pair_ready) {
     CKS(to_pair(ctx, ctx->tw64, &ctx->tw_p, ctx->TW));
     for (int k = 0; k < 2; ++k) {
       CKS(to_pair(ctx, ctx->ehat_x64[k], &ctx->ehat_xp[k], 2LL * g.Px));
       CKS(to_pair(ctx, ctx->ehat_y64[k], &ctx->ehat_yp[k], 2LL * g.Py));
     }
+    ctx->pair_ready = true;
   }
   CKS(to_pair(ctx, ctx->khat64, &ctx->khat_p, (long long)(g.Px / 2) * (g.Py / 2)));
   CKS(to_pair(ctx, ctx->top64, &ctx->top_p, (long long)g.nap + g.n1 + g.n2));

@@ -430,7 +430,7 @@ cavity_status launch_khat_split(cavity_ctx* ctx) {
   const Geo& g = ctx->g;
   if (!f32_fast_size(g.lnx) || !f32_fast_size(g.lny)) return CAVITY_OK;
   const size_t n = (size_t)(g.Px / 2) * (g.Py / 2);
-  if (!ctx->khat32s) CK(cudaMalloc(&ctx->khat32s, sizeof(float2) * n));
+  CK(table_alloc(&ctx->khat32s, n));
   KScope ks_(ctx, KC_SETUP);
   k_khat_split<<<(unsigned)((n + 255) / 256), 256, 0, ctx->stream>>>(ctx->khat32, ctx->khat32s,
                                                                     g.Px / 2, g.Py / 2);

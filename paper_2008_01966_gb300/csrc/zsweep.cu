@@ -191,14 +191,14 @@ cavity_status launch_zsweep(cavity_ctx* ctx, double kappa0) {
   size_t nq = (size_t)(g.nz - 1) * (g.n1 + g.n2);
   // FP32 copies of the profiles for the complex64 field of mixed contexts
   const bool plain32 = ctx->desc.precision == CAVITY_MIXED;
-  if (!ctx->prof) CK(cudaMalloc(&ctx->prof, sizeof(double2) * nprof));
-  if (plain32 && !ctx->prof32) CK(cudaMalloc(&ctx->prof32, sizeof(float2) * nprof));
-  if (!ctx->top64) CK(cudaMalloc(&ctx->top64, sizeof(double2) * (g.nap + g.n1 + g.n2)));
-  if (!ctx->top32) CK(cudaMalloc(&ctx->top32, sizeof(float2) * (g.nap + g.n1 + g.n2)));
-  if (!ctx->minpiv) CK(cudaMalloc(&ctx->minpiv, sizeof(double)));
+  CK(table_alloc(&ctx->prof, nprof));
+  if (plain32) CK(table_alloc(&ctx->prof32, nprof));
+  CK(table_alloc(&ctx->top64, (size_t)g.nap + g.n1 + g.n2));
+  CK(table_alloc(&ctx->top32, (size_t)g.nap + g.n1 + g.n2));
+  CK(table_alloc(&ctx->minpiv, 1));
   const bool layered = L.nl > 1;
-  if (layered && !ctx->profq) CK(cudaMalloc(&ctx->profq, sizeof(double2) * nq));
-  if (plain32 && layered && !ctx->profq32) CK(cudaMalloc(&ctx->profq32, sizeof(float2) * nq));
+  if (layered) CK(table_alloc(&ctx->profq, nq));
+  if (plain32 && layered) CK(table_alloc(&ctx->profq32, nq));
   double big = 1e300;
   CK(cudaMemcpyAsync(ctx->minpiv, &big, sizeof(double), cudaMemcpyHostToDevice, ctx->stream));
   CK(cudaMemsetAsync(ctx->top64, 0, sizeof(double2) * (g.nap + g.n1 + g.n2), ctx->stream));
