@@ -166,11 +166,12 @@ struct ObsPar {
 // m of E1, then of E2: nx + nx - 1), RCS_ROWS rows a block, and a last block
 // per direction adds the blocks' parts in order.  (All modes of a direction in
 // one block used as many SMs as there are directions: 0.12 ms for 16
-// directions at 128 x 128, 0.035 ms now.)
+// directions at 128 x 128, 0.035 ms now.)  Directions along the first axis of
+// the grids, the only one that takes more than 65,535.
 #define RCS_ROWS 16
 __global__ void k_rcs_factors(const ObsPar* __restrict__ op, double2* __restrict__ fac, int nx,
                               int ny, double a, double b) {
-  const int d = blockIdx.y, i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int d = blockIdx.x, i = blockIdx.y * blockDim.x + threadIdx.x;
   if (i >= nx + ny) return;
   const bool xd = i < nx;
   const int m = xd ? i : i - nx;
@@ -188,18 +189,18 @@ __global__ void k_rcs_factors(const ObsPar* __restrict__ op, double2* __restrict
   }
 }
 
-// grid (ceil((2 nx - 1) / RCS_ROWS), ndir), 256 threads; part[d][block]: the
+// grid (ndir, ceil((2 nx - 1) / RCS_ROWS)), 256 threads; part[d][block]: the
 // block's parts of int E1 and int E2
 __global__ void __launch_bounds__(256) k_rcs_rows(const double2* __restrict__ ap,
                                                   const double2* __restrict__ fac,
                                                   double2* __restrict__ part, int nx, int ny,
                                                   int n1, int nap) {
   __shared__ double2 red[2][8];
-  const int d = blockIdx.y, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, N = ny - 1;
+  const int d = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, N = ny - 1;
   const double2* E = ap + (size_t)d * nap;
   const double2* f = fac + (size_t)d * 2 * (nx + ny);
   double2 L[2] = {make_double2(0, 0), make_double2(0, 0)};
-  for (int r = blockIdx.x * RCS_ROWS + warp; r < min((blockIdx.x + 1) * RCS_ROWS, 2 * nx - 1); r += 8) {
+  for (int r = blockIdx.y * RCS_ROWS + warp; r < min((blockIdx.y + 1) * RCS_ROWS, 2 * nx - 1); r += 8) {
     const bool first = r < nx;
     const int m = first ? r : r - nx + 1;
     const double2* row = first ? E + (size_t)m * N - 1 : E + n1 + (size_t)(m - 1) * ny;
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(256) k_rcs_rows(const double2* __restrict__ ap
   if (threadIdx.x < 2) {
     double2 s = make_double2(0, 0);
     for (int w = 0; w < 8; ++w) s = cadd<double>(s, red[threadIdx.x][w]);
-    part[((size_t)d * gridDim.x + blockIdx.x) * 2 + threadIdx.x] = s;
+    part[((size_t)d * gridDim.y + blockIdx.y) * 2 + threadIdx.x] = s;
   }
 }
 
@@ -281,12 +282,12 @@ cavity_status launch_rcs(cavity_ctx* ctx, int ndir, const double2* ap, const dou
   CK(cudaMemcpyAsync(op, hp.data(), sizeof(ObsPar) * ndir, cudaMemcpyHostToDevice, ctx->stream));
   {
     KScope ks_(ctx, KC_RHS);
-    k_rcs_factors<<<dim3((g.nx + g.ny + 127) / 128, ndir), 128, 0, ctx->stream>>>(op, fac, g.nx, g.ny,
+    k_rcs_factors<<<dim3(ndir, (g.nx + g.ny + 127) / 128), 128, 0, ctx->stream>>>(op, fac, g.nx, g.ny,
                                                                                g.a, g.b);
   }
   {
     KScope ks_(ctx, KC_RHS);
-    k_rcs_rows<<<dim3(nb, ndir), 256, 0, ctx->stream>>>(ap, fac, part, g.nx, g.ny, g.n1, g.nap);
+    k_rcs_rows<<<dim3(ndir, nb), 256, 0, ctx->stream>>>(ap, fac, part, g.nx, g.ny, g.n1, g.nap);
   }
   {
     KScope ks_(ctx, KC_RHS);

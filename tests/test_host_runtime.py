@@ -61,3 +61,11 @@ def test_prepare_at_a_second_wavenumber_after_a_failure(fake):
     assert any("k_khat(" in e for e in fake.log(n0))
     assert use(ctx)
     ctx.close()
+
+
+def test_cross_section_of_many_directions(fake):
+    """More directions than the second axis of a grid takes (65,535)."""
+    ctx = fake.context(nx=16, ny=16)
+    assert ctx.prepare() == 0
+    assert ctx.rcs(65535) == 0 and ctx.rcs(70000) == 0
+    ctx.close()
