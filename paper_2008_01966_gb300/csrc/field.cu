@@ -254,7 +254,9 @@ cavity_status launch_field(cavity_ctx* ctx, int ndir, const double2* ap, C<T>* o
   const bool regs = sizeof(T) == 4 && field_f32_supported(g);   // field_f32.cu
   const size_t slab = regs ? field_f32_slab_bytes(g) : (size_t)3 * g.nx * (g.ny + 1) * sizeof(C<T>);
   int lc = (int)std::max<size_t>(1, ((size_t)512 << 20) / (slab * ndir));
-  lc = std::min(lc, g.nz);
+  // slabs are the third axis of the grids, which takes 65,535 (small grids with
+  // many directions)
+  lc = std::min({lc, g.nz, std::max(1, 65535 / ndir)});
   const size_t t1 = slab * ndir * lc;
   const size_t apb = sizeof(C<T>) == 8 ? ((sizeof(float2) * (size_t)ndir * g.nap + 255) / 256) * 256 : 0;
   CKS(ensure_ws(ctx, &ctx->ws2, &ctx->ws2_bytes, t1 + apb));

@@ -69,3 +69,13 @@ def test_cross_section_of_many_directions(fake):
     assert ctx.prepare() == 0
     assert ctx.rcs(65535) == 0 and ctx.rcs(70000) == 0
     ctx.close()
+
+
+def test_field_of_many_slabs(fake):
+    """Small grids with many directions and levels: more slabs than the third
+    axis of a grid takes (65,535) go in several chunks."""
+    ctx = fake.context(nx=16, ny=16, nz=8)
+    assert ctx.prepare() == 0
+    for ndir in (8192, 21000, 27500, 42000, 65535):
+        assert ctx.field(ndir) == 0, ndir
+    ctx.close()
