@@ -612,7 +612,8 @@ struct BWork {
   double2 *part, *hb, *cb;
   int* map;
   void* apw;
-  int kcap, emax;
+  int vcap;         // basis columns of a group
+  int kcap, emax;   // rows of a system's coefficients, systems
 };
 
 static size_t al256(size_t x) { return (x + 255) / 256 * 256; }
@@ -642,12 +643,14 @@ static int num_classes(const cavity_ctx* ctx) {
 // groups at a time), V .. cb per group and class
 struct BSizes {
   int nd, gm, em;   // directions, groups, systems
+  size_t vcap;      // basis columns of a group: as wide as its block may be
   size_t kcap, col;
   BSizes(const cavity_ctx* ctx, int ndir, int mb) {
     const int gw = group_width(ctx);
     nd = std::min(ndir, BG_GROUPS * gw);
     gm = (nd + gw - 1) / gw;
     em = gm * num_classes(ctx);
+    vcap = (size_t)(mb + 1) * gw;
     kcap = (size_t)(mb + 1) * BG_MAX;
     col = sizeof(float2) * (size_t)ctx->g.nap;
   }
@@ -655,7 +658,7 @@ struct BSizes {
 size_t block_inner_work_bytes(const cavity_ctx* ctx, int ndir, int mb) {
   const BSizes z(ctx, ndir, mb);
   size_t b = 0;
-  b += al256(z.col * z.gm * z.kcap);                              // V
+  b += al256(z.col * z.gm * z.vcap);                              // V
   b += 4 * al256(z.col * z.nd);                                   // Rc, Z, Wb, Tt
   b += al256(sizeof(double2) * BG_PART_CTAS * z.kcap * BG_MAX);   // part
   b += al256(sizeof(double2) * 3 * z.em * z.kcap * BG_MAX);       // hb
@@ -669,7 +672,7 @@ static BWork bwork_carve(void* base, const cavity_ctx* ctx, int ndir, int mb) {
   const BSizes z(ctx, ndir, mb);
   char* p = (char*)base;
   BWork w;
-  w.V = (float2*)p; p += al256(z.col * z.gm * z.kcap);
+  w.V = (float2*)p; p += al256(z.col * z.gm * z.vcap);
   w.Rc = (float2*)p; p += al256(z.col * z.nd);
   w.Z = (float2*)p; p += al256(z.col * z.nd);
   w.Wb = (float2*)p; p += al256(z.col * z.nd);
@@ -679,6 +682,7 @@ static BWork bwork_carve(void* base, const cavity_ctx* ctx, int ndir, int mb) {
   w.cb = (double2*)p; p += al256(sizeof(double2) * z.em * z.kcap * BG_MAX);
   w.map = (int*)p; p += al256(sizeof(int) * z.nd);
   w.apw = p;
+  w.vcap = (int)z.vcap;
   w.kcap = (int)z.kcap;
   w.emax = z.em;
   return w;
@@ -825,7 +829,7 @@ cavity_status run_block_inner(cavity_ctx* ctx, int ndir, const float2* r, float2
     }
     std::vector<char> gdone(ng, 0);
     int used = 0;
-    auto Vg = [&](int z) { return w.V + (size_t)z * w.kcap * nap; };
+    auto Vg = [&](int z) { return w.V + (size_t)z * w.vcap * nap; };
     // column col of system e's basis, at its class' rows
     auto Ve = [&](int e, int col) { return Vg(e / NC) + (size_t)col * nap + crow(e % NC); };
     auto hptr = [&](int slot, int e) {

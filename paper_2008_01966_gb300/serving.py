@@ -130,15 +130,20 @@ def footprint_bytes(geom, ndir, precision, layered, want_field):
     by = (nz - 1) * nap * (16 + (8 if mixed else 0))
     if layered:
         by += (nz - 1) * n12 * (16 + (8 if mixed else 0))
-    by += (Px // 2) * (Py // 2) * 48 + 64 * nap
+    by += (Px // 2) * (Py // 2) * 64 + 160 * nap
     el = 8 if mixed else 16
     scratch = 2 * ndir * 3 * (nx + 1) * Py * el
     by += scratch
     vec = ndir * nap
     if mixed:
-        groups = -(-ndir // 16)
-        by += groups * 31 * 16 * nap * 8 + 4 * vec * 8 + 6 * vec * 16 + 2 * scratch
-        by += 608 * 31 * 16 * 16 * 16
+        # block bases of up to 32 groups, each of 31 blocks as wide as the
+        # library's groups, and their coefficients; the operator in FP32 (twice)
+        # and in pair-of-FP32 arithmetic
+        width = 8 if nap < 30000 else 16
+        nd = min(ndir, 32 * width)
+        groups = -(-nd // width)
+        by += groups * 31 * width * nap * 8 + 8 * vec * 8 + 6 * vec * 16 + 3 * scratch
+        by += (608 + 4 * groups * (1 if nap < 300000 else 4)) * 31 * 16 * 16 * 16
     else:
         by += vec * 41 * 16 + 4 * vec * 16
     if want_field:

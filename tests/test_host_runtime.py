@@ -79,3 +79,44 @@ def test_field_of_many_slabs(fake):
     for ndir in (8192, 21000, 27500, 42000, 65535):
         assert ctx.field(ndir) == 0, ndir
     ctx.close()
+
+
+@pytest.mark.parametrize("nx, ny, ndirs", [(16, 16, (1, 64, 300)), (32, 32, (8, 100, 256)),
+                                           (64, 64, (1, 9, 64, 200, 600)), (64, 128, (17, 100)),
+                                           (128, 128, (16, 64, 200)), (256, 256, (5, 16, 64)),
+                                           (512, 512, (1, 8, 16))])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_footprint_is_an_upper_estimate(fake, nx, ny, ndirs, precision):
+    """Serving admits contexts by footprint_bytes: what a context, its calls
+    and their outputs allocate stays below it."""
+    from paper_2008_01966_gb300.serving import footprint_bytes
+    for ndir in ndirs:
+        for nlayers in (1, 3):
+            for field in (False, True):
+                fake.lib.fake_reset()
+                base = fake.lib.fake_live()
+                ctx = fake.context(nx=nx, ny=ny, nz=12, precision=precision)
+                assert ctx.solve(ndir, field=field, nlayers=nlayers) == 0 and ctx.rcs(ndir) == 0
+                used = fake.lib.fake_peak() - base + ndir * ctx.n_ap * 16
+                used += ndir * ctx.field_per_dir * ctx.el if field else 0
+                ctx.close()
+                assert used <= footprint_bytes((1.0, 1.0, 0.5, nx, ny, 12), ndir, precision,
+                                               nlayers > 1, field), (ndir, nlayers, field)
+
+
+def test_basis_of_a_group_is_as_wide_as_the_group(fake):
+    """The block basis takes (steps + 1) x width columns per group."""
+    def peak(width):
+        fake.lib.fake_reset()
+        base = fake.lib.fake_live()
+        ctx = fake.context(nx=128, ny=128)
+        assert fake.lib.cavity_set_option(ctx.h, 2, width) == 0
+        assert ctx.solve(32, field=False) == 0
+        used = fake.lib.fake_peak() - base
+        n_ap = ctx.n_ap
+        ctx.close()
+        return used, n_ap
+
+    (a, n_ap), (b, _) = peak(16), peak(4)
+    # the same columns in all; what differs are the coefficients of more systems
+    assert b - a < 0.05 * 31 * 32 * n_ap * 8
