@@ -33,11 +33,10 @@
  *    cavity_last_error() describes it; outputs are then unspecified except where
  *    stated.
  *  - a context is not thread safe: one host thread at a time per context.
- *  - one device per process: the library raises the shared-memory limits of
- *    its kernels once per process, on the device current at that first use,
- *    so every context of a process must be set up on that device (on another
- *    device, a launch that needs the raised limit returns a CUDA error
- *    status, without a fault).  Use one process per GPU.
+ *  - a context belongs to the device that was current at cavity_setup, which
+ *    must be current in every call on it.  What a device needs once (kernel
+ *    attributes, constant tables) is set up on each device at its first use.
+ *    Tested on one device per process only; use one process per GPU.
  */
 #ifndef CAVITY_H
 #define CAVITY_H

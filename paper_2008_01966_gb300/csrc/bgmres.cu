@@ -37,7 +37,6 @@
 // batch; unlike per-direction GMRES it depends (within the tolerance) on which
 // directions share a group.
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <complex>
 #include <vector>
@@ -727,11 +726,11 @@ static void bproj(cavity_ctx* ctx, const BGSet& set, int ng, int kmax, const BWo
   rs = (rs + BP_ROWS - 1) / BP_ROWS * BP_ROWS;
   nct = (nrow + rs - 1) / rs;
   double2* h = w.hb + (size_t)slot * w.emax * w.kcap * BG_MAX;
-  static std::atomic<bool> done{false};  // set once; host threads may race
+  static DeviceFlag done;
   if (!done) {
     cudaFuncSetAttribute(k_bproj_tc<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TP_SMEM);
     cudaFuncSetAttribute(k_bproj_tc<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TP_SMEM);
-    done = true;
+    done.set();
   }
   if (narrow) {
     KScope ks_(ctx, KC_KRYLOV);

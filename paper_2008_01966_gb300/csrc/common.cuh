@@ -6,6 +6,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdint.h>
+#include <atomic>
 #include <string>
 #include <type_traits>
 #include <utility>
@@ -290,6 +291,21 @@ inline int ilog2(int n) {
   return l;
 }
 
+// Whether something that belongs to a device (a kernel's attributes, a constant
+// table) has been set up on the current one: a flag per device of the process.
+// Host threads may race; the setting is then made twice.  Devices from the 65th
+// on are set up at every call.
+struct DeviceFlag {
+  std::atomic<uint64_t> seen{0};
+  static uint64_t bit() {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return dev >= 0 && dev < 64 ? 1ull << dev : 0;
+  }
+  operator bool() const { return (seen.load(std::memory_order_acquire) & bit()) != 0; }
+  void set() { seen.fetch_or(bit(), std::memory_order_release); }
+};
+
 // opt-in shared memory limit of the current device (bytes)
 inline int smem_optin() {
   int dev = 0, v = 0;
@@ -298,7 +314,7 @@ inline int smem_optin() {
   return v > 0 ? v : 48 * 1024;
 }
 
-// SMs of the current device
+// SMs of the device first asked for (launch shapes only)
 inline int sm_count() {
   static const int n = [] {
     int dev = 0, v = 0;

@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(128) k_cgemm_tc(GemmArgs g) {
   if (warp == 0) tc_dealloc(tmem, 128);
 }
 
-static std::atomic<bool> g_gt_smem{false};
+static DeviceFlag g_gt_smem;
 
 // the tensor-core GEMM's timeout flag: cleared before a dense step, read after it
 static cavity_status gt_err_clear(cavity_ctx* ctx) {
@@ -394,7 +394,7 @@ static cavity_status cgemm(cavity_ctx* ctx, const GemmArgs& a, int cls) {
   if (!g_gt_smem) {
     CK(cudaFuncSetAttribute(k_cgemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)(2 * sizeof(GtBuf))));
-    g_gt_smem = true;
+    g_gt_smem.set();
   }
   KScope ks_(ctx, cls);
   k_cgemm_tc<<<dim3(nblk(a.N, GT_BN), nblk(a.M, 128)), 128, 2 * sizeof(GtBuf), ctx->stream>>>(a);
@@ -928,10 +928,10 @@ static cudaError_t luc_dispatch(cudaStream_t st, int R, float2* a, int lda, int 
 }
 #define LUC_RMAX 192   // 24 rows a thread; 32 spill
 // cluster size of the panels: 16 (a non-portable size) where the device runs it,
-// else 8, else 0 (none); asked once per process
+// else 8, else 0 (none); asked once per device, whose attribute it sets
 static int luc_cluster() {
-  static std::atomic<int> known{-1};
-  if (known >= 0) return known;
+  static DeviceFlag known, ok16, ok8;
+  if (known) return ok16 ? 16 : ok8 ? 8 : 0;
   auto runs = [](auto dispatch) {
     for (int R : {32, 64, 128, LUC_RMAX}) {
       int m = 0;
@@ -942,7 +942,9 @@ static int luc_cluster() {
   };
   const int k = runs(luc_dispatch<16>) ? 16 : runs(luc_dispatch<8>) ? 8 : 0;
   cudaGetLastError();   // a refused attribute is an answer, not an error
-  known = k;
+  if (k == 16) ok16.set();
+  if (k == 8) ok8.set();
+  known.set();
   return k;
 }
 
@@ -1011,7 +1013,7 @@ __global__ void k_lu_perm(const int* __restrict__ ipiv, int* __restrict__ perm, 
   for (int i = threadIdx.x; i < n; i += blockDim.x) perm[i] = pm[i];
 }
 
-static std::atomic<bool> g_lu_smem{false};
+static DeviceFlag g_lu_smem;
 
 cavity_status dense_lu(cavity_ctx* ctx, float2* a, int n, int lda, int* ipiv, int* info) {
   if (n < 1 || n > CAVITY_DENSE_MAX_N || lda < n || !a || !ipiv) {
@@ -1044,7 +1046,7 @@ cavity_status dense_lu(cavity_ctx* ctx, float2* a, int n, int lda, int* ipiv, in
                             (int)(sizeof(float2) * LU_RMAX * LU_VS)));
     CK(cudaFuncSetAttribute(k_lu_perm, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)(sizeof(int) * CAVITY_DENSE_MAX_N)));
-    g_lu_smem = true;
+    g_lu_smem.set();
   }
   for (int p = 0; p < npanel; ++p) {
     const int k0 = p * LU_NB, nb = std::min(LU_NB, n - k0), H = n - k0;
@@ -1307,7 +1309,7 @@ __global__ void __launch_bounds__(256, 1) k_trs_sweep(const float2* __restrict__
 }
 
 static const size_t TRS_SMEM = sizeof(float2) * (4 * TS_T + 2 * TS_D * (TS_B + 1));
-static std::atomic<bool> g_trs_smem{false};
+static DeviceFlag g_trs_smem;
 
 // scratch of the substitutions: a barrier counter per sweep and right-hand side
 // (a sweep uses one per chunk) and an error flag behind them
@@ -1317,12 +1319,12 @@ static size_t subst_err_offset(int nrhs) {
 static size_t subst_scratch_bytes(int nrhs) { return al256(subst_err_offset(nrhs) + sizeof(int)); }
 static size_t dinv_bytes(int n) { return sizeof(float2) * 2 * (size_t)TS_B * TS_B * ((n + TS_B - 1) / TS_B); }
 
-static std::atomic<bool> g_dinv_smem{false};
+static DeviceFlag g_dinv_smem;
 static cavity_status launch_dinv(cavity_ctx* ctx, const float2* lu, int n, int lda, float2* dinv) {
   if (!g_dinv_smem) {
     CK(cudaFuncSetAttribute(k_lu_dinv, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)(sizeof(float2) * 2 * TS_T)));
-    g_dinv_smem = true;
+    g_dinv_smem.set();
   }
   KScope ks_(ctx, KC_DENSE_LU);
   k_lu_dinv<<<(n + TS_B - 1) / TS_B, 256, sizeof(float2) * 2 * TS_T, ctx->stream>>>(lu, lda, n, dinv);
@@ -1339,7 +1341,7 @@ static cavity_status lu_substitute(cavity_ctx* ctx, const float2* lu, int n, int
   if (!g_trs_smem) {
     CK(cudaFuncSetAttribute(k_trs_sweep<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRS_SMEM));
     CK(cudaFuncSetAttribute(k_trs_sweep<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TRS_SMEM));
-    g_trs_smem = true;
+    g_trs_smem.set();
   }
   const int nch = (nrhs + TS_D - 1) / TS_D;
   unsigned int* bars = (unsigned int*)scratch;
@@ -1395,7 +1397,7 @@ cavity_status dense_lu_solve(cavity_ctx* ctx, const float2* lu, int n, int lda, 
   if (!g_lu_smem) {
     CK(cudaFuncSetAttribute(k_lu_perm, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)(sizeof(int) * CAVITY_DENSE_MAX_N)));
-    g_lu_smem = true;
+    g_lu_smem.set();
   }
   if (!perm) {
     {

@@ -19,7 +19,6 @@
 // Output per direction and level j = 1..Nz: E1 on p = 0..Nx, q = 1..Ny-1,
 // E2 on p = 1..Nx-1, q = 0..Ny, E3 on p = 1..Nx-1, q = 1..Ny-1, row-major.
 #include <algorithm>
-#include <atomic>
 
 #include "common.cuh"
 #include "fft.cuh"
@@ -295,10 +294,10 @@ cavity_status launch_field(cavity_ctx* ctx, int ndir, const double2* ap, C<T>* o
     if (!regs) {
       CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
         constexpr int LN = decltype(c)::value, L = field_lines<T>(2 << LN);
-        static std::atomic<bool> done{false};  // set once; host threads may race
+        static DeviceFlag done;
         if (!done) {
           CK(allow_max_smem(k_field_y<T, LN>));
-          done = true;
+          done.set();
         }
         KScope ks_(ctx, KC_FIELD_Y);
         k_field_y<T, LN><<<dim3((g.nx + L - 1) / L, 2, ndir * lc), FIELD_THREADS,
@@ -308,10 +307,10 @@ cavity_status launch_field(cavity_ctx* ctx, int ndir, const double2* ap, C<T>* o
       }));
       CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
         constexpr int LN = decltype(c)::value, L = field_lines<T>(2 << LN);
-        static std::atomic<bool> done{false};  // set once; host threads may race
+        static DeviceFlag done;
         if (!done) {
           CK(allow_max_smem(k_field_x<T, LN>));
-          done = true;
+          done.set();
         }
         KScope ks_(ctx, KC_FIELD_X);
         k_field_x<T, LN><<<dim3((g.ny + 1 + L - 1) / L, 2, ndir * lc), FIELD_THREADS,

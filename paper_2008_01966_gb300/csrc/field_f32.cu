@@ -26,7 +26,6 @@
 //   256 x 128 x 91, 3 directions, 3 layers   0.47 -> 0.22 ms
 //   64 x 64 x 32, 32 directions, 3 layers    0.25 -> 0.14 ms
 #include <algorithm>
-#include <atomic>
 
 #include "common.cuh"
 #include "gfft.cuh"
@@ -223,10 +222,10 @@ __global__ void __launch_bounds__(FX_NT, 2)
   }
 }
 
-template <typename K> cavity_status smem_set(cavity_ctx* ctx, K kern, std::atomic<bool>& done) {
+template <typename K> cavity_status smem_set(cavity_ctx* ctx, K kern, DeviceFlag& done) {
   if (!done) {
     CK(allow_max_smem(kern));
-    done = true;
+    done.set();
   }
   return CAVITY_OK;
 }
@@ -247,7 +246,7 @@ cavity_status launch_field_f32(cavity_ctx* ctx, int ndir, const float2* ap, floa
   CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = FShape<LN, FY_NT>;
-    static std::atomic<bool> done[2]{{false}, {false}};  // set once; host threads may race
+    static DeviceFlag done[2];
     const dim3 grid((g.nx + F::R - 1) / F::R, 2, ndir * nlev);
     CKS(smem_set(ctx, k_fy<LN, false>, done[0]));
     CKS(smem_set(ctx, k_fy<LN, true>, done[1]));
@@ -263,7 +262,7 @@ cavity_status launch_field_f32(cavity_ctx* ctx, int ndir, const float2* ap, floa
   CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = FShape<LN, FX_NT>;
-    static std::atomic<bool> done{false};
+    static DeviceFlag done;
     CKS(smem_set(ctx, k_fx<LN>, done));
     KScope ks_(ctx, KC_FIELD_X);
     k_fx<LN><<<dim3((g.ny + F::R) / F::R, 2, ndir * nlev), FX_NT, F::BYTES, ctx->stream>>>(

@@ -382,7 +382,7 @@ __global__ void __launch_bounds__(256) k_khat(double2* __restrict__ raw, double2
 cavity_status launch_khat(cavity_ctx* ctx, double kappa0) {
   const Geo& g = ctx->g;
   static std::mutex mu;   // host threads may prepare contexts at the same time
-  static bool gl_done = false;
+  static DeviceFlag gl_done;
   std::unique_lock<std::mutex> lock(mu);
   if (!gl_done) {
     std::vector<double> x, w;
@@ -396,7 +396,7 @@ cavity_status launch_khat(cavity_ctx* ctx, double kappa0) {
     std::vector<double> tab;
     j0_table(tab);
     CK(cudaMemcpyToSymbol(g_j0_tab, tab.data(), sizeof(double) * tab.size()));
-    gl_done = true;
+    gl_done.set();
   }
   lock.unlock();
   const int hx = g.Px / 2, hy = g.Py / 2;

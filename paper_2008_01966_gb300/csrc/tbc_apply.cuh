@@ -35,7 +35,6 @@
 // sides of 4 or 8 intervals, or when a pass option asks for them.
 #pragma once
 #include <algorithm>
-#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -696,10 +695,10 @@ static int last_n(const cavity_ctx* ctx) { return ctx->desc.modes_n > 0 ? ctx->d
 
 // opt every instantiation of kernel K into the device's shared-memory maximum
 // once per process
-template <typename K> static cavity_status smem_once(cavity_ctx* ctx, K kern, std::atomic<bool>& done) {
+template <typename K> static cavity_status smem_once(cavity_ctx* ctx, K kern, DeviceFlag& done) {
   if (!done) {
     CK(allow_max_smem(kern));
-    done = true;
+    done.set();
   }
   return CAVITY_OK;
 }
@@ -741,7 +740,7 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
     const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN),
                                   pair_threads<T>(4 << LN), g.nx,
                                   2LL * ndir);
-    static std::atomic<bool> done{false};  // set once; host threads may race
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_tbcA<T, LN>, done));
     KScope ks_(ctx, kclass<T>(0));
     k_tbcA<T, LN><<<dim3(cl.blocks(g.nx), 2, ndir), cl.threads, smem_a<T>(g.ny, cl.lL), st>>>(
@@ -752,7 +751,7 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
     constexpr int LN = decltype(c)::value;
     if constexpr (b1_ok<T>(LN)) {
       if (b1_use(g.Py, ndir)) {
-        static std::atomic<bool> done1{false};
+        static DeviceFlag done1;
         CKS(smem_once(ctx, k_tbcB1<T, LN>, done1));
         KScope ks_(ctx, kclass<T>(1));
         k_tbcB1<T, LN><<<dim3(g.Py, ndir), std::max(64, std::min(FftE<T>::THREADS, 6 * fft_tpl<T>(4 << LN))),
@@ -765,7 +764,7 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
     const CtaLines cl = cta_lines(clog2(pairs_per_cta<T>(4 << LN)), 2, fft_tpl<T>(4 << LN),
                                   pair_threads<T>(4 << LN), g.Py,
                                   ndir);
-    static std::atomic<bool> done{false};  // set once; host threads may race
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_tbcB<T, LN>, done));
     KScope ks_(ctx, kclass<T>(1));
     k_tbcB<T, LN><<<dim3(cl.blocks(g.Py), ndir), cl.threads, smem_b<T>(g.nx, cl.lL), st>>>(
@@ -778,7 +777,7 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
     const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(4 << LN)), 1, fft_tpl<T>(4 << LN),
                                   FftE<T>::THREADS, g.nx + 1,
                                   3LL * ndir);
-    static std::atomic<bool> done{false};  // set once; host threads may race
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_tbcC<T, LN>, done));
     KScope ks_(ctx, kclass<T>(2));
     k_tbcC<T, LN><<<dim3(cl.blocks(g.nx + 1), 3, ndir), cl.threads, smem_c<T>(g.ny, cl.lL), st>>>(
@@ -790,7 +789,7 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
     const CtaLines cl = cta_lines(clog2(lines_per_cta<T>(2 << LN)), 1, fft_tpl<T>(2 << LN),
                                   FftE<T>::THREADS, g.ny + 1,
                                   3LL * ndir);
-    static std::atomic<bool> done{false};  // set once; host threads may race
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_tbcD<T, LN>, done));
     KScope ks_(ctx, kclass<T>(3));
     k_tbcD<T, LN><<<dim3(cl.blocks(g.ny + 1), 3, ndir), cl.threads, smem_d<T>(g.nx, cl.lL), st>>>(

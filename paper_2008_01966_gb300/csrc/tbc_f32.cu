@@ -451,7 +451,7 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
   CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = F32Shape<LN>;
-    static std::atomic<bool> done{false};  // set once; host threads may race
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_opA<LN>, done));
     KScope ks_(ctx, KC_TBC_A32);
     k_opA<LN><<<dim3((g.nx + F::R - 1) / F::R, 2, ndir), F::NT, SmemA<LN>::BYTES, st>>>(
@@ -461,7 +461,7 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
   CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = F32Shape<LN>;
-    static std::atomic<bool> done{false};
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_opB<LN>, done));
     KScope ks_(ctx, KC_TBC_B32);
     k_opB<LN><<<dim3(g.Py / F::CB, ndir), F::NT, SmemB<LN>::BYTES, st>>>(
@@ -472,7 +472,7 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
   CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     constexpr int R = SmemC<LN>::R;
-    static std::atomic<bool> done{false};
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_opC<LN>, done));
     KScope ks_(ctx, KC_TBC_C32);
     k_opC<LN><<<dim3((g.nx + 1 + R - 1) / R, 3, ndir), SmemC<LN>::NT, SmemC<LN>::BYTES, st>>>(
@@ -482,7 +482,7 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
   CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     constexpr int R = SmemD<LN>::R;
-    static std::atomic<bool> done{false};
+    static DeviceFlag done;
     CKS(smem_once(ctx, k_opD<LN>, done));
     KScope ks_(ctx, KC_TBC_D32);
     k_opD<LN><<<dim3((g.ny + R - 1) / R, 3, ndir), SmemD<LN>::NT, SmemD<LN>::BYTES, st>>>(

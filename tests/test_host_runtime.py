@@ -120,3 +120,25 @@ def test_basis_of_a_group_is_as_wide_as_the_group(fake):
     (a, n_ap), (b, _) = peak(16), peak(4)
     # the same columns in all; what differs are the coefficients of more systems
     assert b - a < 0.05 * 31 * 32 * n_ap * 8
+
+
+def test_every_device_is_set_up(fake):
+    """Kernel attributes and constant tables belong to a device: the same calls
+    on two devices set up the same on both."""
+    def calls(dev):
+        fake.lib.fake_set_device(dev)
+        n = fake.lib.fake_log_size()
+        for nx, solver, modes in ((8, "krylov", 0), (64, "krylov", 0), (32, "dense", 6)):
+            for precision in ("fp64", "mixed"):
+                ctx = fake.context(nx=nx, ny=nx, precision=precision, solver=solver, modes=modes)
+                ctx.prepare()
+                use(ctx)
+                ctx.solve(20)
+                ctx.close()
+        return sorted(e.replace("device=%d" % dev, "") for e in fake.log(n)
+                      if e.startswith(("symbol", "attribute")) and e.endswith("device=%d" % dev))
+
+    first, second = calls(11), calls(12)
+    assert any("g_j0_tab" in e for e in first) and any("k_opB" in e for e in first)
+    assert any("k_lu_panel_cluster" in e for e in first)
+    assert first == second
