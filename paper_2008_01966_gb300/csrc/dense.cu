@@ -1013,7 +1013,15 @@ __global__ void k_lu_perm(const int* __restrict__ ipiv, int* __restrict__ perm, 
   for (int i = threadIdx.x; i < n; i += blockDim.x) perm[i] = pm[i];
 }
 
-static DeviceFlag g_lu_smem;
+static DeviceFlag g_lu_smem, g_perm_smem;
+// k_lu_perm is launched by the factorisation and by the solve
+static cavity_status perm_smem(cavity_ctx* ctx) {
+  if (g_perm_smem) return CAVITY_OK;
+  CK(cudaFuncSetAttribute(k_lu_perm, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                          (int)(sizeof(int) * CAVITY_DENSE_MAX_N)));
+  g_perm_smem.set();
+  return CAVITY_OK;
+}
 
 cavity_status dense_lu(cavity_ctx* ctx, float2* a, int n, int lda, int* ipiv, int* info) {
   if (n < 1 || n > CAVITY_DENSE_MAX_N || lda < n || !a || !ipiv) {
@@ -1044,10 +1052,9 @@ cavity_status dense_lu(cavity_ctx* ctx, float2* a, int n, int lda, int* ipiv, in
   if (!g_lu_smem) {
     CK(cudaFuncSetAttribute(k_lu_panel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                             (int)(sizeof(float2) * LU_RMAX * LU_VS)));
-    CK(cudaFuncSetAttribute(k_lu_perm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)(sizeof(int) * CAVITY_DENSE_MAX_N)));
     g_lu_smem.set();
   }
+  CKS(perm_smem(ctx));
   for (int p = 0; p < npanel; ++p) {
     const int k0 = p * LU_NB, nb = std::min(LU_NB, n - k0), H = n - k0;
     const int cl = luc_cluster(), RC = cl ? nblk(H, cl) : 0;
@@ -1394,11 +1401,7 @@ cavity_status dense_lu_solve(cavity_ctx* ctx, const float2* lu, int n, int lda, 
   float2* Y = (float2*)((char*)ctx->ws + bp);
   float2* dinv = (float2*)((char*)ctx->ws + bp + by);
   void* scr = (char*)ctx->ws + bp + by + bd;
-  if (!g_lu_smem) {
-    CK(cudaFuncSetAttribute(k_lu_perm, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                            (int)(sizeof(int) * CAVITY_DENSE_MAX_N)));
-    g_lu_smem.set();
-  }
+  CKS(perm_smem(ctx));
   if (!perm) {
     {
       KScope ks_(ctx, KC_DENSE_TRS);

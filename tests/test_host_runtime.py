@@ -142,3 +142,24 @@ def test_every_device_is_set_up(fake):
     assert any("g_j0_tab" in e for e in first) and any("k_opB" in e for e in first)
     assert any("k_lu_panel_cluster" in e for e in first)
     assert first == second
+
+
+def test_lu_factor_after_lu_solve(fake):
+    """A solve with given factors, as the first dense call on a device, leaves
+    the factorisation's kernel its own setting."""
+    import ctypes
+    import numpy as np
+    fake.lib.fake_set_device(21)
+    ctx = fake.context()
+    assert ctx.prepare() == 0
+    n = 4000
+    a, b = np.empty(n * n * 2, np.float32), np.empty(n * 2, np.float32)
+    piv = np.zeros(n, np.int32)
+    p = lambda v: ctypes.c_void_p(v.ctypes.data)  # noqa: E731
+    start = fake.lib.fake_log_size()
+    assert ctx.lib.cavity_lu_solve(ctx.h, p(a), 64, 64, p(piv), 1, p(b), 64) == 0
+    ctx.lib.cavity_lu_factor(ctx.h, p(a), n, n, p(piv), None)
+    log = fake.log(start)
+    assert any(e.startswith("launch k_lu_panel(") for e in log)
+    assert any(e.startswith("attribute") and "k_lu_panel(" in e for e in log)
+    ctx.close()
