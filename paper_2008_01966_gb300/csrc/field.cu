@@ -245,6 +245,13 @@ __global__ void k_ap32(const double2* __restrict__ a, float2* __restrict__ b, lo
   if (k < n) b[k] = make_float2((float)a[k].x, (float)a[k].y);
 }
 
+// Host outputs leave chunk by chunk while the next chunk is synthesised: at
+// least FIELD_HOST_CHUNKS of them, since the copy of the last one and the
+// synthesis of the first overlap with nothing, but none of less than
+// FIELD_HOST_BYTES, which the link takes in the time of a chunk's launches.
+#define FIELD_HOST_CHUNKS 8
+#define FIELD_HOST_BYTES ((size_t)4 << 20)
+
 template <typename T>
 cavity_status launch_field(cavity_ctx* ctx, int ndir, const double2* ap, C<T>* out,
                            void* host_out) {
@@ -256,6 +263,11 @@ cavity_status launch_field(cavity_ctx* ctx, int ndir, const double2* ap, C<T>* o
   // slabs are the third axis of the grids, which takes 65,535 (small grids with
   // many directions)
   lc = std::min({lc, g.nz, std::max(1, 65535 / ndir)});
+  if (host_out) {
+    const size_t level = sizeof(C<T>) * (size_t)g.field_per_level * ndir;
+    lc = std::min(lc, std::max((g.nz + FIELD_HOST_CHUNKS - 1) / FIELD_HOST_CHUNKS,
+                               (int)std::min<size_t>(g.nz, (FIELD_HOST_BYTES + level - 1) / level)));
+  }
   const size_t t1 = slab * ndir * lc;
   const size_t apb = sizeof(C<T>) == 8 ? ((sizeof(float2) * (size_t)ndir * g.nap + 255) / 256) * 256 : 0;
   CKS(ensure_ws(ctx, &ctx->ws2, &ctx->ws2_bytes, t1 + apb));
