@@ -67,7 +67,8 @@ __global__ void __launch_bounds__(256) k_dots(const C<T>* __restrict__ V, long l
 // in shared memory and forms the partial dots of that chunk with all cnt basis
 // vectors (blockIdx.z takes MDOT_VECS of them); a second kernel adds the chunk
 // partials in chunk order.  The chunk depends on n_ap and cnt alone
-// (mdot_chunk), so a direction's sums do not depend on the batch.  FP64 work is
+// (mdot_chunk), so a direction's sums do not depend on the batch (nor does the
+// operator: tbc_apply.cuh, w_first).  FP64 work is
 // scarce per SM (two lanes), so a short vector is cut into pieces for as many
 // SMs as it can feed: up to 24 vectors of 3,007 entries took 40 us in two
 // blocks, now 6.4 us in 24 to 72.

@@ -219,6 +219,23 @@ __global__ void TBC_PAIR_BOUNDS(LNY) k_tbcA(const C<T>* __restrict__ x, C<T>* __
 // the first inverse transforms).  The column gather stays a cooperative pass:
 // as a per-line first read it would load one element per 32-byte sector.
 
+// w = s0 g0 - s1 g1, the product with s0 rounded first and the other one fused
+// into the difference: said explicitly for FP64, so that the two forms of pass
+// B, which take a vector by the size of the batch, give the same bits (the pair
+// type's operations are exact about this by themselves).
+template <typename T> __device__ __forceinline__ C<T> w_first(C<T> g0, T s0) {
+  if constexpr (std::is_same<T, double>::value)
+    return make_double2(__dmul_rn(g0.x, s0), __dmul_rn(g0.y, s0));
+  else
+    return cscale<T>(g0, s0);
+}
+template <typename T> __device__ __forceinline__ C<T> w_second(C<T> w, C<T> g1, T s1) {
+  if constexpr (std::is_same<T, double>::value)
+    return make_double2(__fma_rn(-g1.x, s1, w.x), __fma_rn(-g1.y, s1, w.y));
+  else
+    return csub<T>(w, cscale<T>(g1, s1));
+}
+
 // last write of the first inverse transforms of pass B: output t (k = t mod
 // Px) of line (r, l), |t| < Px/4, times the kernel table at (|2t + r|, |j2|),
 // written to slot t mod Px/2 (other outputs are not needed), and into w
@@ -251,8 +268,8 @@ struct KhatB : LineId<T> {
     }
     line[pidx(u)] = o;
     C<T>* w = wl + (size_t)lr * padded_len(hp) + pidx(u);
-    if (F == 0) *w = cscale<T>(o, (T)j2 * scale);
-    else *w = csub<T>(*w, cscale<T>(o, (T)j1 * scale));
+    if (F == 0) *w = w_first<T>(o, (T)j2 * scale);
+    else *w = w_second<T>(*w, o, (T)j1 * scale);
   }
 };
 
@@ -455,7 +472,7 @@ __global__ void TBC_BOUNDS k_tbcB1(const C<T>* __restrict__ Vy, C<T>* __restrict
     const int j1 = 2 * (u < nx ? u : u - Px / 2) + r;
     const C<T> g0 = buf[(size_t)r * ls + pidx(u)], g1 = buf[(size_t)(2 + r) * ls + pidx(u)];
     buf[(size_t)(4 + r) * ls + pidx(u)] =
-        csub<T>(cscale<T>(g0, (T)j2 * ay), cscale<T>(g1, (T)j1 * ax));
+        w_second<T>(w_first<T>(g0, (T)j2 * ay), g1, (T)j1 * ax);
   }
   __syncthreads();
   fft_lines<T, true, LPX - 1, 6>(buf, ls, 6, tw, p.twlog);
