@@ -247,8 +247,12 @@ __global__ void k_ap32(const double2* __restrict__ a, float2* __restrict__ b, lo
 
 // Host outputs leave chunk by chunk while the next chunk is synthesised: at
 // least FIELD_HOST_CHUNKS of them, since the copy of the last one and the
-// synthesis of the first overlap with nothing, but none of less than
-// FIELD_HOST_BYTES, which the link takes in the time of a chunk's launches.
+// synthesis of the first overlap with nothing, but with at least
+// FIELD_HOST_BYTES of each direction (a copy of its own: many small ones cost
+// more than the overlap gives, 64 x 64 x 32, 64 directions 4.58 ms a solve in
+// one chunk, 5.31 in eight).  Host over device outputs of a solve on a GB300, in
+// 512 MB chunks and now: 512 x 512 x 128, one direction 3.90 -> 3.48 ms;
+// 512 x 512 x 64, two 3.92 -> 3.56; 256 x 256 x 64, eight 3.94 -> 3.71.
 #define FIELD_HOST_CHUNKS 8
 #define FIELD_HOST_BYTES ((size_t)4 << 20)
 
@@ -264,7 +268,7 @@ cavity_status launch_field(cavity_ctx* ctx, int ndir, const double2* ap, C<T>* o
   // many directions)
   lc = std::min({lc, g.nz, std::max(1, 65535 / ndir)});
   if (host_out) {
-    const size_t level = sizeof(C<T>) * (size_t)g.field_per_level * ndir;
+    const size_t level = sizeof(C<T>) * (size_t)g.field_per_level;
     lc = std::min(lc, std::max((g.nz + FIELD_HOST_CHUNKS - 1) / FIELD_HOST_CHUNKS,
                                (int)std::min<size_t>(g.nz, (FIELD_HOST_BYTES + level - 1) / level)));
   }
