@@ -147,13 +147,15 @@ cavity_status launch_rhs(cavity_ctx* ctx, int ndir, const double* theta, const d
 }
 
 // ------------------------------------------------------------------ RCS
+// (Sums and products whose fusing the compiler could choose by the kernel they are
+// inlined into are written as such: two kernels below share them to the last bit.)
 // int_0^side exp(-i s y) dy = side exp(-i s side/2) sinc(s side/2)
 __device__ __forceinline__ double2 ef(double s, double side) {
-  double x = 0.5 * s * side;
-  double sc = fabs(x) < 1e-8 ? 1.0 - x * x / 6.0 : sin(x) / x;
-  double ss, cc;
-  sincos(-x, &ss, &cc);
-  return make_double2(side * sc * cc, side * sc * ss);
+  const double x = 0.5 * s * side;
+  double sn, cs;
+  sincos(x, &sn, &cs);
+  const double sc = fabs(x) < 1e-8 ? 1.0 - x * x / 6.0 : sn / x;
+  return make_double2(__dmul_rn(side * sc, cs), __dmul_rn(-side * sc, sn));
 }
 
 struct ObsPar {
@@ -162,24 +164,45 @@ struct ObsPar {
 };
 
 // Per direction the 1-D integrals of every mode, [C1x (nx) | S2x (nx) | S1y
-// (ny) | C2y (ny)]; then each warp sums rows of E1 and E2 against them (rows
-// m of E1, then of E2: nx + nx - 1), RCS_ROWS rows a block, and a last block
-// per direction adds the blocks' parts in order.  (All modes of a direction in
-// one block used as many SMs as there are directions: 0.12 ms for 16
-// directions at 128 x 128, 0.035 ms now.)  Directions along the first axis of
-// the grids, the only one that takes more than 65,535.
-#define RCS_ROWS 16
-__global__ void k_rcs_factors(const ObsPar* __restrict__ op, double2* __restrict__ fac, int nx,
-                              int ny, double a, double b) {
-  const int d = blockIdx.x, i = blockIdx.y * blockDim.x + threadIdx.x;
-  if (i >= nx + ny) return;
+// (ny) | C2y (ny)], against which the rows of E1 and of E2 are summed by blocks
+// of 256 threads in units of RCS_PASSES passes (32 lanes a row, or as many as a
+// short row has entries).  A thread adds its parts of the units in order, then
+// the threads are added: once per direction, since with two FP64 lanes per SM
+// that takes as long as 20 terms of the sum.
+//
+// Two ways, with the same operations in the same order, which depends on the
+// grid alone (a direction's result has the same bits in any batch): one block a
+// direction for all of it (k_rcs_whole), where there are directions for two
+// blocks on every SM or little to do; else the units of a direction on blocks of
+// their own, which store every thread's part (k_rcs_factors, k_rcs_units,
+// k_rcs_final: two launches and that traffic more, but as many SMs as there are
+// units).
+// Directions go along the first axis of the grids, the only one that takes more
+// than 65,535.  Measured on a GB300, a call's us with every unit's sum reduced in
+// its block, and now: 64 x 64, 300 directions 142 -> 99; 256 x 256, 64 237 -> 139;
+// 1024 x 4, 300 988 -> 156; 64 x 64, one 48 -> 48; 1024 x 1024, one 83 -> 87.  One
+// block a direction against its units on many: 64 x 64, one direction 68 and 48,
+// 300 99 and 126; 16 x 16, one 41 and 52.
+#define RCS_PASSES 2
+struct RcsUnits {
+  int lpr, rows, n1, n2;   // lanes per row, rows per unit, units of E1 (nx rows) and of E2 (nx - 1)
+  RcsUnits(int nx, int ny) {
+    lpr = ny < 32 ? ny : 32;
+    rows = RCS_PASSES * (256 / lpr);
+    n1 = (nx + rows - 1) / rows;
+    n2 = (nx - 1 + rows - 1) / rows;
+  }
+};
+
+// integrals of mode i of [x modes | y modes] into f
+__device__ __forceinline__ void rcs_mode(int i, const ObsPar& o, double2* f, int nx, int ny, double a,
+                                         double b) {
   const bool xd = i < nx;
   const int m = xd ? i : i - nx;
-  const double side = xd ? a : b, g = xd ? op[d].g1 : op[d].g2, k = m * M_PI / side;
+  const double side = xd ? a : b, g = xd ? o.g1 : o.g2, k = m * M_PI / side;
   const double2 fm = ef(g - k, side), fp = ef(g + k, side);
-  const double2 c = make_double2(0.5 * (fm.x + fp.x), 0.5 * (fm.y + fp.y));
-  const double2 s = make_double2(0.5 * (fm.y - fp.y), -0.5 * (fm.x - fp.x));   // /(2i)
-  double2* f = fac + (size_t)d * 2 * (nx + ny);
+  const double2 c = make_double2(0.5 * __dadd_rn(fm.x, fp.x), 0.5 * __dadd_rn(fm.y, fp.y));
+  const double2 s = make_double2(0.5 * __dsub_rn(fm.y, fp.y), -0.5 * __dsub_rn(fm.x, fp.x));   // /(2i)
   if (xd) {
     f[m] = c;
     f[nx + m] = s;
@@ -189,60 +212,41 @@ __global__ void k_rcs_factors(const ObsPar* __restrict__ op, double2* __restrict
   }
 }
 
-// grid (ndir, ceil((2 nx - 1) / RCS_ROWS)), 256 threads; part[d][block]: the
-// block's parts of int E1 and int E2
-__global__ void __launch_bounds__(256) k_rcs_rows(const double2* __restrict__ ap,
-                                                  const double2* __restrict__ fac,
-                                                  double2* __restrict__ part, int nx, int ny,
-                                                  int n1, int nap) {
-  __shared__ double2 red[2][8];
-  const int d = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, N = ny - 1;
-  const double2* E = ap + (size_t)d * nap;
-  const double2* f = fac + (size_t)d * 2 * (nx + ny);
-  double2 L[2] = {make_double2(0, 0), make_double2(0, 0)};
-  for (int r = blockIdx.y * RCS_ROWS + warp; r < min((blockIdx.y + 1) * RCS_ROWS, 2 * nx - 1); r += 8) {
-    const bool first = r < nx;
-    const int m = first ? r : r - nx + 1;
-    const double2* row = first ? E + (size_t)m * N - 1 : E + n1 + (size_t)(m - 1) * ny;
-    const double2* fy = f + 2 * nx + (first ? 0 : ny);
-    double2 s = make_double2(0, 0);
-    for (int n = (first ? 1 : 0) + lane; n < ny; n += 32) s = cadd<double>(s, cmul<double>(row[n], fy[n]));
-    const double2 v = cmul<double>(s, f[(first ? 0 : nx) + m]);
-    L[first ? 0 : 1] = cadd<double>(L[first ? 0 : 1], v);
-  }
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    for (int off = 16; off > 0; off >>= 1) {
-      L[q].x += __shfl_xor_sync(0xffffffffu, L[q].x, off);
-      L[q].y += __shfl_xor_sync(0xffffffffu, L[q].y, off);
-    }
-    if (lane == 0) red[q][warp] = L[q];
-  }
-  __syncthreads();
-  if (threadIdx.x < 2) {
-    double2 s = make_double2(0, 0);
-    for (int w = 0; w < 8; ++w) s = cadd<double>(s, red[threadIdx.x][w]);
-    part[((size_t)d * gridDim.y + blockIdx.y) * 2 + threadIdx.x] = s;
-  }
+// s + a b, four multiply-adds
+__device__ __forceinline__ double2 rcs_fma(double2 a, double2 b, double2 s) {
+  return make_double2(__fma_rn(a.x, b.x, __fma_rn(-a.y, b.y, s.x)),
+                      __fma_rn(a.x, b.y, __fma_rn(a.y, b.x, s.y)));
+}
+__device__ __forceinline__ double2 rcs_add(double2 a, double2 b) {
+  return make_double2(__dadd_rn(a.x, b.x), __dadd_rn(a.y, b.y));
 }
 
-// one warp per direction
-__global__ void k_rcs_final(const double2* __restrict__ part, const ObsPar* __restrict__ op,
-                            double* __restrict__ sigma, int nblocks, double kappa0) {
-  const int d = blockIdx.x, lane = threadIdx.x;
-  double2 s1 = make_double2(0, 0), s2 = make_double2(0, 0);
-  for (int k = lane; k < nblocks; k += 32) {
-    s1 = cadd<double>(s1, part[((size_t)d * nblocks + k) * 2]);
-    s2 = cadd<double>(s2, part[((size_t)d * nblocks + k) * 2 + 1]);
+// thread t's part of unit u of E1 (FIRST) or E2
+template <bool FIRST>
+__device__ __forceinline__ double2 rcs_unit(int u, int t, const double2* __restrict__ E,
+                                            const double2* f, int nx, int ny, int n1,
+                                            const RcsUnits& un) {
+  const int lr = 31 - __clz(un.lpr);   // a power of two
+  const int sub = t >> lr, lane = t & (un.lpr - 1);
+  const double2* fy = f + 2 * nx + (FIRST ? 0 : ny);
+  double2 acc = make_double2(0, 0);
+#pragma unroll
+  for (int k = 0; k < RCS_PASSES; ++k) {
+    const int m = u * un.rows + k * (256 >> lr) + sub + (FIRST ? 0 : 1);
+    if (m >= nx) break;
+    const double2* row = FIRST ? E + (size_t)m * (ny - 1) - 1 : E + n1 + (size_t)(m - 1) * ny;
+    double2 s = make_double2(0, 0);
+#pragma unroll 4
+    for (int n = (FIRST ? 1 : 0) + lane; n < ny; n += un.lpr) s = rcs_fma(row[n], fy[n], s);
+    acc = rcs_fma(s, f[(FIRST ? 0 : nx) + m], acc);
   }
-  for (int off = 16; off > 0; off >>= 1) {
-    s1.x += __shfl_xor_sync(0xffffffffu, s1.x, off);
-    s1.y += __shfl_xor_sync(0xffffffffu, s1.y, off);
-    s2.x += __shfl_xor_sync(0xffffffffu, s2.x, off);
-    s2.y += __shfl_xor_sync(0xffffffffu, s2.y, off);
-  }
-  if (lane != 0) return;
-  const ObsPar o = op[d];
+  return acc;
+}
+
+// cross-section from int E1 and int E2
+__device__ __noinline__ double rcs_sigma(double2 s1, double2 s2, const ObsPar* __restrict__ op,
+                                         double kappa0) {
+  const ObsPar o = *op;
   // L = (-int E2, int E1, 0)
   const double2 L[3] = {make_double2(-s2.x, -s2.y), s1, make_double2(0, 0)};
   // v = e . (x_hat x L)
@@ -252,7 +256,86 @@ __global__ void k_rcs_final(const double2* __restrict__ part, const ObsPar* __re
     const double2 cr = csub<double>(cscale<double>(L[k2], o.xh[k1]), cscale<double>(L[k1], o.xh[k2]));
     v = cadd<double>(v, cscale<double>(cr, o.e[k]));
   }
-  sigma[d] = kappa0 * kappa0 / M_PI * cabs2<double>(v);
+  return kappa0 * kappa0 / M_PI * cabs2<double>(v);
+}
+// the 256 threads' int E1 (a) and int E2 (b) into direction d's cross-section
+__device__ __forceinline__ void rcs_finish(double2 a, double2 b, const ObsPar* __restrict__ op, int d,
+                                           double* __restrict__ sigma, double kappa0) {
+  __shared__ double2 red[2][8];
+  for (int off = 16; off > 0; off >>= 1) {
+    a.x += __shfl_xor_sync(0xffffffffu, a.x, off);
+    a.y += __shfl_xor_sync(0xffffffffu, a.y, off);
+    b.x += __shfl_xor_sync(0xffffffffu, b.x, off);
+    b.y += __shfl_xor_sync(0xffffffffu, b.y, off);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    red[0][threadIdx.x >> 5] = a;
+    red[1][threadIdx.x >> 5] = b;
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  double2 s1 = red[0][0], s2 = red[1][0];
+  for (int k = 1; k < 8; ++k) {
+    s1 = rcs_add(s1, red[0][k]);
+    s2 = rcs_add(s2, red[1][k]);
+  }
+  sigma[d] = rcs_sigma(s1, s2, op + d, kappa0);
+}
+
+// grid ndir, 256 threads, 2 (nx + ny) complex values of shared memory
+__global__ void __launch_bounds__(256) k_rcs_whole(const double2* __restrict__ ap,
+                                                   const ObsPar* __restrict__ op,
+                                                   double* __restrict__ sigma, int nx, int ny,
+                                                   int n1, int nap, double a, double b,
+                                                   RcsUnits un, double kappa0) {
+  extern __shared__ double2 sm_f[];
+  const int d = blockIdx.x, t = threadIdx.x;
+  for (int i = t; i < nx + ny; i += 256) rcs_mode(i, op[d], sm_f, nx, ny, a, b);
+  __syncthreads();
+  const double2* E = ap + (size_t)d * nap;
+  double2 s1 = make_double2(0, 0), s2 = make_double2(0, 0);
+  for (int u = 0; u < un.n1; ++u) s1 = rcs_add(s1, rcs_unit<true>(u, t, E, sm_f, nx, ny, n1, un));
+  for (int u = 0; u < un.n2; ++u) s2 = rcs_add(s2, rcs_unit<false>(u, t, E, sm_f, nx, ny, n1, un));
+  rcs_finish(s1, s2, op, d, sigma, kappa0);
+}
+
+// grid (ndir, ceil((nx + ny) / 128))
+__global__ void k_rcs_factors(const ObsPar* __restrict__ op, double2* __restrict__ fac, int nx,
+                              int ny, double a, double b) {
+  const int d = blockIdx.x, i = blockIdx.y * blockDim.x + threadIdx.x;
+  if (i < nx + ny) rcs_mode(i, op[d], fac + (size_t)d * 2 * (nx + ny), nx, ny, a, b);
+}
+// grid (ndir, units), 256 threads; part[d][unit][thread]
+__global__ void __launch_bounds__(256) k_rcs_units(const double2* __restrict__ ap,
+                                                   const double2* __restrict__ fac,
+                                                   double2* __restrict__ part, int nx, int ny,
+                                                   int n1, int nap, RcsUnits un) {
+  const int d = blockIdx.x, u = blockIdx.y, t = threadIdx.x;
+  const double2* E = ap + (size_t)d * nap;
+  const double2* f = fac + (size_t)d * 2 * (nx + ny);
+  part[((size_t)d * gridDim.y + u) * 256 + t] =
+      u < un.n1 ? rcs_unit<true>(u, t, E, f, nx, ny, n1, un)
+                : rcs_unit<false>(u - un.n1, t, E, f, nx, ny, n1, un);
+}
+// grid ndir, 256 threads
+__global__ void __launch_bounds__(256) k_rcs_final(const double2* __restrict__ part,
+                                                   const ObsPar* __restrict__ op,
+                                                   double* __restrict__ sigma, RcsUnits un,
+                                                   double kappa0) {
+  const int d = blockIdx.x;
+  const double2* p = part + (size_t)d * (un.n1 + un.n2) * 256 + threadIdx.x;
+  double2 s1 = make_double2(0, 0), s2 = make_double2(0, 0);
+#pragma unroll 8
+  for (int u = 0; u < un.n1; ++u) s1 = rcs_add(s1, p[(size_t)u * 256]);
+  p += (size_t)un.n1 * 256;
+#pragma unroll 8
+  for (int u = 0; u < un.n2; ++u) s2 = rcs_add(s2, p[(size_t)u * 256]);
+  rcs_finish(s1, s2, op, d, sigma, kappa0);
+}
+
+// whether one block takes a direction
+static bool rcs_whole(int ndir, int nx, int ny) {
+  return ndir >= 2 * sm_count() || nx * ny <= 512;
 }
 
 cavity_status launch_rcs(cavity_ctx* ctx, int ndir, const double2* ap, const double* th,
@@ -269,29 +352,42 @@ cavity_status launch_rcs(cavity_ctx* ctx, int ndir, const double2* ap, const dou
     else { o.e[0] = -sf; o.e[1] = cf; o.e[2] = 0.0; }
   }
   auto al = [](size_t v) { return (v + 255) / 256 * 256; };
-  const int nb = (2 * g.nx - 1 + RCS_ROWS - 1) / RCS_ROWS;
+  const RcsUnits un(g.nx, g.ny);
+  const bool whole = rcs_whole(ndir, g.nx, g.ny);
   const size_t b_op = al(sizeof(ObsPar) * ndir), b_sg = al(sizeof(double) * ndir);
-  const size_t b_fac = al(sizeof(double2) * (size_t)ndir * 2 * (g.nx + g.ny));
-  CKS(ensure_ws(ctx, &ctx->ws2, &ctx->ws2_bytes,
-                b_op + b_sg + b_fac + sizeof(double2) * 2 * (size_t)ndir * nb));
+  const size_t b_fac = whole ? 0 : al(sizeof(double2) * (size_t)ndir * 2 * (g.nx + g.ny));
+  const size_t b_part = whole ? 0 : sizeof(double2) * 256 * (size_t)ndir * (un.n1 + un.n2);
+  CKS(ensure_ws(ctx, &ctx->ws2, &ctx->ws2_bytes, b_op + b_sg + b_fac + b_part));
   char* w = (char*)ctx->ws2;
   ObsPar* op = (ObsPar*)w;
   double* sg = (double*)(w + b_op);
   double2* fac = (double2*)(w + b_op + b_sg);
   double2* part = (double2*)(w + b_op + b_sg + b_fac);
   CK(cudaMemcpyAsync(op, hp.data(), sizeof(ObsPar) * ndir, cudaMemcpyHostToDevice, ctx->stream));
-  {
+  if (whole) {
+    static DeviceFlag done;
+    if (!done) {
+      CK(allow_max_smem(k_rcs_whole));
+      done.set();
+    }
     KScope ks_(ctx, KC_RHS);
-    k_rcs_factors<<<dim3(ndir, (g.nx + g.ny + 127) / 128), 128, 0, ctx->stream>>>(op, fac, g.nx, g.ny,
-                                                                               g.a, g.b);
-  }
-  {
-    KScope ks_(ctx, KC_RHS);
-    k_rcs_rows<<<dim3(ndir, nb), 256, 0, ctx->stream>>>(ap, fac, part, g.nx, g.ny, g.n1, g.nap);
-  }
-  {
-    KScope ks_(ctx, KC_RHS);
-    k_rcs_final<<<ndir, 32, 0, ctx->stream>>>(part, op, sg, nb, ctx->kappa0);
+    k_rcs_whole<<<ndir, 256, sizeof(double2) * 2 * (g.nx + g.ny), ctx->stream>>>(
+        ap, op, sg, g.nx, g.ny, g.n1, g.nap, g.a, g.b, un, ctx->kappa0);
+  } else {
+    {
+      KScope ks_(ctx, KC_RHS);
+      k_rcs_factors<<<dim3(ndir, (g.nx + g.ny + 127) / 128), 128, 0, ctx->stream>>>(
+          op, fac, g.nx, g.ny, g.a, g.b);
+    }
+    {
+      KScope ks_(ctx, KC_RHS);
+      k_rcs_units<<<dim3(ndir, un.n1 + un.n2), 256, 0, ctx->stream>>>(ap, fac, part, g.nx, g.ny,
+                                                                      g.n1, g.nap, un);
+    }
+    {
+      KScope ks_(ctx, KC_RHS);
+      k_rcs_final<<<ndir, 256, 0, ctx->stream>>>(part, op, sg, un, ctx->kappa0);
+    }
   }
   CK(cudaGetLastError());
   CK(cudaMemcpyAsync(sigma, sg, sizeof(double) * ndir, cudaMemcpyDeviceToHost, ctx->stream));
