@@ -306,14 +306,12 @@ cavity_status cavity_lu_solve(cavity_ctx* ctx, const void* lu, int n, int lda, c
 
 /* ---- implementation options (chosen by the autotuner) ---------------------
  * Variants of the same arithmetic whose speed depends on the grid, the batch
- * and the device; results agree within the precision of the path (the FP32
- * operator variants to ~1e-7 relative, the group width within the solver
+ * and the device; results agree (the group width within the solver
  * tolerance).  Set per context, at any time between calls; the
  * paper_2008_01966_gb300.autotune module times them and caches its choice.
- *  CAVITY_OPT_PASS_B_2048, CAVITY_OPT_PASS_C_2048: FP32 operator on grids with
- *      nx = 512 (B) or ny = 512 (C): 0 = lines of 2048 points in the registers
- *      of a group of lanes (default), 1 = the generic passes with the block
- *      (Stockham) transform.
+ *  CAVITY_OPT_PASS_B_2048, CAVITY_OPT_PASS_C_2048: accept 0 and 1, as before;
+ *      the FP32 operator has one form of each pass on every grid, faster than
+ *      either of those that these values used to choose between.
  *  CAVITY_OPT_GROUP_WIDTH: directions per group of the mixed solve's block
  *      Krylov iterations (one basis per group), 1..16; default 16, taken as 8
  *      on grids of fewer than 30,000 aperture unknowns unless it is set.

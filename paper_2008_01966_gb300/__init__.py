@@ -356,12 +356,12 @@ class Cavity:
 
     # ------------------------------------------------------------ options
     def set_option(self, name, value):
-        """Implementation option (include/cavity.h, CAVITY_OPT_*): "pass_b_2048",
-        "pass_c_2048" (0 warp pairs, 1 block transform), "group_width"
+        """Implementation option (include/cavity.h, CAVITY_OPT_*): "group_width"
         (1..16 directions per block Krylov group), "coarse_modes" (0, or
         mc > 0: the mixed solve's two-level preconditioner with the exact
-        solve of the modes m, n <= mc as its coarse level) or "field_fused"
-        (0, 1 or 2: accepted, the complex64 field has one path)."""
+        solve of the modes m, n <= mc as its coarse level), "pass_b_2048",
+        "pass_c_2048" (0 or 1) or "field_fused" (0, 1 or 2): accepted, the
+        FP32 operator and the complex64 field have one path each."""
         self._check(self.lib.cavity_set_option(self.h, _lib.OPTIONS[name], int(value)))
 
     def get_option(self, name):

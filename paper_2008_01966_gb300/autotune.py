@@ -9,7 +9,9 @@ same shape reuse it without timing.
 
 Options and what is timed:
   pass_b_2048, pass_c_2048  (512-point grid sides, mixed precision): one
-      application of the FP32 operator to the batch (cavity_apply), per value;
+      application of the FP32 operator to the batch (cavity_apply), per value
+      (the library has one path for both; kept so that cached choices stay
+      complete);
   group_width (mixed precision): the aperture solve of the batch (cavity_solve
       without the field), per value among GROUP_WIDTHS; a width is kept only if
       every direction converged;

@@ -398,10 +398,9 @@ cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, vo
 template <>
 cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, float2* y, void* work,
                                   long long ystride, const ParityMap& pm);
-// sides (log2) that the FP32 operator's own passes take (tbc_f32.cu), their
-// tables (once per context) and their copy of the kernel table (per kappa0)
-#define F32_LOG_MIN 4
-inline bool f32_fast_size(int ln) { return ln >= F32_LOG_MIN; }
+// the FP32 operator's tables (once per context) and its copy of the kernel table
+// (per kappa0); sides (log2) from which the complex64 field has passes like it
+#define FIELD_F32_LOG_MIN 4
 cavity_status launch_lane_tables(cavity_ctx* ctx);
 cavity_status launch_khat_split(cavity_ctx* ctx);
 size_t apply_work_bytes(const Geo& g, int ndir, int elem_bytes);

@@ -1,19 +1,20 @@
-// Shared-memory FFTs of power-of-two length for the cavity solver.
-//
-// All transforms of the hot path -- the Fourier-series synthesis (E123F), the
-// trapezoid projections and the torus convolution of Sec. 5.2 -- are batches
-// of 1-D transforms of lines held in shared memory.
+// Shared-memory FFTs of power-of-two length for the cavity solver: batches of 1-D
+// transforms of lines held in shared memory, for the FP64 and pair-of-FP32
+// operators and the FP64 field, and for the complex64 field of sides of 4 and 8.
+// (The FP32 operator and the complex64 field of larger sides hold their lines in
+// registers: gfft.cuh.)
 //
 // Two algorithms:
+//  * block transform (FP64 and pair, and FP32 lines outside the range of the
+//    other): Stockham auto-sort, each thread owning FftE<T>::E slots of a line
+//    per pass (8 and radix 8; pair: 4 and radix 4; more at 4096 points); inputs
+//    are read from shared memory into registers, twiddled, transformed and
+//    written back in place after a barrier of the line's threads.
 //  * warp transform (FP32, 64 <= n <= 1024): the line is split as n = LW x RV
 //    (LW lanes, RV values per lane, RV = LW or 2 LW); each lane does an RV-point
 //    DFT in registers, the twiddle w_n^{l k1}, one transpose through shared
 //    memory and an LW-point DFT in registers (the "four-step" factorisation).
 //    Only warp-level synchronisation inside the transform.
-//  * block transform (FP64, and FP32 lines outside that range): Stockham
-//    auto-sort with radix-8 passes, each thread owning 8 slots of a line per
-//    pass; inputs are read from shared memory into registers, twiddled,
-//    transformed and written back in place after a CTA barrier.
 // Lines use a padded layout (one pad word per 16 elements, see pidx) so that
 // strided accesses do not collide in the shared-memory banks.  Twiddles come
 // from a table tw[k] = exp(-2 pi i k / TW) computed once in FP64 (rounded for
@@ -482,25 +483,4 @@ __device__ __forceinline__ void fft_lines(C<T>* base, int lstride, int nlines,
     for (int l0 = 0; l0 < nlines; l0 += lpg) group(l0 + lg, lg < lpg && l0 + lg < nlines);
   }
   __syncthreads();
-}
-
-// Warp-resident transform of the lines [first, first + cnt) that belong to the
-// calling warp (FP32, LineShape<T, LOGN>::WARP): 32 / LW lines at a time, each
-// on LW lanes.  Warp-level synchronisation only -- no block barrier, so the
-// warps of a block can run their chains of transforms independently.
-template <typename T, bool INV, int LOGN, typename Op = LineId<T>>
-__device__ __forceinline__ void fft_warp_lines(C<T>* base, int lstride, int first, int cnt,
-                                               const C<T>* __restrict__ tw, int twlog,
-                                               const Op& op = Op()) {
-  using S = LineShape<T, LOGN>;
-  static_assert(S::WARP, "warp transform lengths only");
-  constexpr int LW = S::LW, LPW = 32 / LW;
-  const int lane = threadIdx.x & 31;
-  const int sub = lane / LW, t = lane - sub * LW;
-  for (int l0 = 0; l0 < cnt; l0 += LPW) {
-    const int l = first + l0 + sub;
-    const bool active = l0 + sub < cnt;
-    C<T>* line = base + (size_t)(active ? l : first) * lstride;
-    fft_warp<T, INV, LW, S::RV, Op>(line, 1 << LOGN, LOGN, t, active, tw, twlog, l, op);
-  }
 }

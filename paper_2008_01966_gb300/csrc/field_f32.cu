@@ -232,7 +232,9 @@ template <typename K> cavity_status smem_set(cavity_ctx* ctx, K kern, DeviceFlag
 
 }  // namespace
 
-bool field_f32_supported(const Geo& g) { return f32_fast_size(g.lnx) && f32_fast_size(g.lny); }
+bool field_f32_supported(const Geo& g) {
+  return g.lnx >= FIELD_F32_LOG_MIN && g.lny >= FIELD_F32_LOG_MIN;
+}
 size_t field_f32_slab_bytes(const Geo& g) { return sizeof(float2) * 3 * (size_t)g.nx * g.ny; }
 
 // levels j0 .. j0 + nlev - 1 of all directions; T1: slab bytes x ndir x nlev
@@ -243,7 +245,7 @@ cavity_status launch_field_f32(cavity_ctx* ctx, int ndir, const float2* ap, floa
   p.nx = g.nx; p.ny = g.ny; p.nz = g.nz; p.M = g.M; p.N = g.N; p.n1 = g.n1; p.n2 = g.n2;
   p.nap = g.nap; p.j0 = j0; p.ndir = ndir; p.S = g.field_per_level;
   const float2* profq = ctx->layers.size() > 1 ? ctx->profq32 : nullptr;
-  CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
+  CKS(dispatch_log<FIELD_F32_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = FShape<LN, FY_NT>;
     static DeviceFlag done[2];
@@ -259,7 +261,7 @@ cavity_status launch_field_f32(cavity_ctx* ctx, int ndir, const float2* ap, floa
                                                              ctx->lane_tab_f[1]);
     return CAVITY_OK;
   }));
-  CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
+  CKS(dispatch_log<FIELD_F32_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = FShape<LN, FX_NT>;
     static DeviceFlag done;

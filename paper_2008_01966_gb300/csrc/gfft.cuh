@@ -1,7 +1,7 @@
 // Register-resident FP32 transforms by groups of lanes, for the passes of the
-// FP32 operator (tbc_f32.cu).
+// FP32 operator (tbc_f32.cu) and of the complex64 field (field_f32.cu).
 //
-// A group of LG lanes (8 .. 128) holds a line of n = LG RV points, RV values
+// A group of LG lanes (4 .. 128) holds a line of n = LG RV points, RV values
 // per lane, lane l holding x[l + LG r].  The transform is one register DFT of
 // RV points, the twiddle w_n^{l k1}, one transpose through shared memory, and
 // a DFT of LG points, and it returns its result in the SAME distribution,
@@ -24,8 +24,9 @@
 #pragma once
 #include "fft.cuh"
 
-// lanes and values per lane of a line of 2^LOGN points (6 <= LOGN <= 12)
+// lanes and values per lane of a line of 2^LOGN points
 template <int LOGN> struct GShape {
+  static_assert(LOGN >= 4 && LOGN <= 12, "lines of 16 to 4096 points");
   static constexpr int RV = LOGN >= 9 ? 32 : 1 << ((LOGN + 1) / 2);
   static constexpr int LG = (1 << LOGN) / RV;
 };
@@ -40,7 +41,6 @@ template <int LG, int RV> struct GTile {
 // lane table of one grid axis with n = 2^LOGN: [w_n^{l k1}] (k1-major, LG
 // wide), fold factors [w_LG^{h l'}] (h-major, RV wide; LG entries), the same
 // two for n/2 points (RV/2 values per lane), and exp(+2 pi i p / n), p <= n/4.
-__host__ __device__ constexpr int lane_tab_full(int) { return 0; }
 __host__ __device__ constexpr int lane_tab_half(int n, int LG) { return n + LG; }
 __host__ __device__ constexpr int lane_tab_post(int n, int LG) { return n + LG + n / 2 + LG; }
 __host__ __device__ constexpr int lane_tab_size(int n, int LG) {
@@ -78,7 +78,9 @@ __device__ __forceinline__ void dft16z(float2* v) {
 }
 template <bool INV, int R>
 __device__ __forceinline__ void dft_natz(float2* v) {
-  if constexpr (R == 8) {
+  if constexpr (R == 4) {
+    dft4sz<INV>(v, 1);
+  } else if constexpr (R == 8) {
     float2 e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
     dft4sz<INV>(e, 1);
     dft4sz<INV>(o, 1);
@@ -99,7 +101,7 @@ __device__ __forceinline__ void dft_natz(float2* v) {
 #pragma unroll
     for (int k = 0; k < 16; ++k) v[k] = u[dft16_slot(k)];
   } else {
-    static_assert(R == 32, "8, 16 or 32 values per lane");
+    static_assert(R == 32, "4, 8, 16 or 32 values per lane");
     float2 e[16], o[16];
 #pragma unroll
     for (int i = 0; i < 16; ++i) {

@@ -27,12 +27,11 @@
 //                  onto cos/sin(n pi q/Ny) (an extended FFT of length 2Ny)
 //   D  (cols n)    trapezoid projection along x1 (extended FFT of length 2Nx)
 // and a final elementwise pass adds the local part of (EJ1)/(uT1).
-// Templated on the arithmetic type: FP64 for the FP64 path and the residuals,
-// FP32 for the inner Krylov iterations of the mixed path.  Every pass kernel
-// is instantiated per grid size so that its line transforms have compile-time
-// lengths; tbc.cu instantiates the FP64 operator, tbc_df*.cu the pair-of-FP32 one.
-// The FP32 operator has passes of its own (tbc_f32.cu) and takes these only on
-// sides of 4 or 8 intervals, or when a pass option asks for them.
+// Templated on the arithmetic type: FP64 for the FP64 path, pair-of-FP32 for the
+// residuals of the mixed path.  Every pass kernel is instantiated per grid size
+// so that its line transforms have compile-time lengths; tbc.cu instantiates the
+// FP64 operator, tbc_df*.cu the pair-of-FP32 one.  The FP32 operator of the
+// mixed path's inner iterations has passes of its own (tbc_f32.cu).
 #pragma once
 #include <algorithm>
 #include <type_traits>
@@ -484,7 +483,7 @@ __global__ void TBC_BOUNDS k_tbcB1(const C<T>* __restrict__ Vy, C<T>* __restrict
   }
 }
 // sizes it is built for, and launches small enough for it
-template <typename T> __host__ __device__ constexpr bool b1_ok(int ln) { return sizeof(C<T>) == 16 && ln <= 7; }
+__host__ __device__ constexpr bool b1_ok(int ln) { return ln <= 7; }
 inline bool b1_use(int Py, int ndir) { return (long long)Py * ndir <= 4LL * sm_count(); }
 
 // ------------------------------------------------------------------ pass C
@@ -684,13 +683,6 @@ template <> struct Tabs<double> {
   static const double2* kh(cavity_ctx* c) { return c->khat64; }
   static const double2* top(cavity_ctx* c) { return c->top64; }
 };
-template <> struct Tabs<float> {
-  static const float2* tw(cavity_ctx* c) { return c->tw32; }
-  static const float2* ex(cavity_ctx* c, int k) { return c->ehat_x32[k]; }
-  static const float2* ey(cavity_ctx* c, int k) { return c->ehat_y32[k]; }
-  static const float2* kh(cavity_ctx* c) { return c->khat32; }
-  static const float2* top(cavity_ctx* c) { return c->top32; }
-};
 
 // shared memory of each pass (bytes) at 2^lL lines (or pairs) per CTA
 template <typename T> static size_t smem_a(int ny, int lL) {
@@ -722,14 +714,13 @@ template <typename K> static cavity_status smem_once(cavity_ctx* ctx, K kern, De
 
 // launch-accounting class of pass `k` (0..4: A, B, C, D, combine) for type T
 template <typename T> static int kclass(int k) {
-  if (sizeof(C<T>) == 8) return KC_TBC_A32 + k;
   if (std::is_same<T, double>::value) return KC_TBC_A64 + k;
   return KC_TBC_AP + k;
 }
 
 template <typename T>
-cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
-                                   long long ystride, const ParityMap& pm) {
+cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
+                           long long ystride, const ParityMap& pm) {
   if (!ctx->g.fft_ok) {
     ctx->err = "the FFT operator needs the convolution period 4 on both axes";
     return CAVITY_EINVAL;
@@ -766,7 +757,7 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
-    if constexpr (b1_ok<T>(LN)) {
+    if constexpr (b1_ok(LN)) {
       if (b1_use(g.Py, ndir)) {
         static DeviceFlag done1;
         CKS(smem_once(ctx, k_tbcB1<T, LN>, done1));
@@ -822,10 +813,4 @@ cavity_status launch_apply_generic(cavity_ctx* ctx, int ndir, const C<T>* x, C<T
   }
   CK(cudaGetLastError());
   return CAVITY_OK;
-}
-
-template <typename T>
-cavity_status launch_apply(cavity_ctx* ctx, int ndir, const C<T>* x, C<T>* y, void* work,
-                           long long ystride, const ParityMap& pm) {
-  return launch_apply_generic<T>(ctx, ndir, x, y, work, ystride, pm);
 }

@@ -1,6 +1,6 @@
-// The FP32 aperture operator (inner iterations of the mixed-precision solve)
-// on grids of 16 .. 1024 intervals per side: the passes of tbc_apply.cuh with
-// register-resident group transforms (gfft.cuh).
+// The FP32 aperture operator (inner iterations of the mixed-precision solve):
+// the passes of tbc_apply.cuh with register-resident group transforms
+// (gfft.cuh).
 //
 // What differs from the generic passes:
 //  * Two basis transforms instead of three.  E1 is a sine series in x2 and E2
@@ -24,6 +24,9 @@
 //   64 x 64, 64 vectors 147 -> 56;  256 x 256, 64 vectors 2624 -> 964;
 //   512 x 256, 5 vectors 496 -> 221;  512 x 512, 8 vectors 1554 -> 831;
 //   1024 x 1024, 3 vectors 2981 -> 1435.
+// Sides of 4 and 8 (lines of 16 and 32 points, 32 of them in a block of pass A),
+// us per operator, the generic passes and these: 256 x 4, 8 vectors 76 -> 54;
+// 512 x 8, 8 vectors 80 -> 63; 8 x 8, one vector 51 -> 49.
 // The three passes around it (A, C, D), 256 x 256, 64 vectors: 670 -> 410.
 // Error against 64 bits (relative, random vectors, 16 .. 1024 per side):
 // 0.9e-7 .. 2.1e-7, before 1.0e-7 .. 3.1e-7; on right-hand sides and solutions
@@ -65,19 +68,21 @@ cavity_status launch_lane_tables(cavity_ctx* ctx) {
   const Geo& g = ctx->g;
   for (int ax = 0; ax < 2; ++ax) {
     const int ln = ax == 0 ? g.lnx : g.lny, n = 4 << ln;
-    if (!f32_fast_size(ln)) continue;
-    CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(ln, [&](auto c) -> cavity_status {
-      using S = GShape<decltype(c)::value + 2>;
+    CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(ln, [&](auto c) -> cavity_status {
+      constexpr int LN = decltype(c)::value;
+      using S = GShape<LN + 2>;
       const int sz = lane_tab_size(n, S::LG);
       CK(cudaMalloc(&ctx->lane_tab[ax], sizeof(float2) * sz));
       KScope ks_(ctx, KC_SETUP);
       k_lane_tab<<<(sz + 255) / 256, 256, 0, ctx->stream>>>(ctx->lane_tab[ax], n, S::LG, S::RV);
       // the field's lines, of 2 << ln points
-      using SF = GShape<decltype(c)::value + 1>;
-      const int szf = lane_tab_size(n / 2, SF::LG);
-      CK(cudaMalloc(&ctx->lane_tab_f[ax], sizeof(float2) * szf));
-      k_lane_tab<<<(szf + 255) / 256, 256, 0, ctx->stream>>>(ctx->lane_tab_f[ax], n / 2, SF::LG,
-                                                            SF::RV);
+      if constexpr (LN >= FIELD_F32_LOG_MIN) {
+        using SF = GShape<LN + 1>;
+        const int szf = lane_tab_size(n / 2, SF::LG);
+        CK(cudaMalloc(&ctx->lane_tab_f[ax], sizeof(float2) * szf));
+        k_lane_tab<<<(szf + 255) / 256, 256, 0, ctx->stream>>>(ctx->lane_tab_f[ax], n / 2, SF::LG,
+                                                              SF::RV);
+      }
       return CAVITY_OK;
     }));
   }
@@ -89,6 +94,10 @@ cavity_status launch_lane_tables(cavity_ctx* ctx) {
 // LN = log2 of the axis' intervals; lines of n = 4 << LN points.  Blocks have
 // at least 128 threads; with 32 values (64 registers) of the line and as many
 // of its spectrum per lane, three blocks of 128 run on an SM.
+// Pitch of a line of U (nx + 1 nodes): 32-byte aligned, but packed on sides of 4
+// and 8, so that Vt and U fit what the generic passes' Vy and W take
+// (apply_work_bytes), in units of Py: 2 nx + 3 (nx + 4) <= 6 nx + 3 from nx = 9.
+__host__ __device__ constexpr int u_pitch(int nx) { return nx >= 16 ? nx + 4 : nx + 1; }
 template <int LN> struct F32Shape {
   using S = GShape<LN + 2>;
   static constexpr int N = 4 << LN, LG = S::LG, RV = S::RV, H = RV / 2, Q4 = RV / 4;
@@ -96,12 +105,12 @@ template <int LN> struct F32Shape {
   static constexpr int TILE = GTile<LG, RV>::SIZE;
   static constexpr int R = NT / LG;        // rows per block of pass A
   static constexpr int CB = NT / (2 * LG); // columns per block of pass B
-  static constexpr int CPITCH = (1 << LN) + 4;  // nodes of a line of U, 32-byte aligned
+  static constexpr int CPITCH = u_pitch(1 << LN);
 };
 #define F32_BOUNDS(LN) __launch_bounds__(F32Shape<LN>::NT, (LN) >= 10 ? 1 : 3)
 
 // ------------------------------------------------------------------ pass A
-// grid (nx / R row groups, 2 fields, ndir); field 0: E1 (sine in x2), 1: E2
+// grid (ceil(nx / R) row groups, 2 fields, ndir); field 0: E1 (sine in x2), 1: E2
 // (cosine).  Group g of the block transforms row k1 = R blockIdx.x + g; both
 // parities' results are collected in shared memory and written to
 // Vt[d][f][j2][k1], R rows (consecutive k1) at a time.
@@ -130,7 +139,7 @@ __global__ void __launch_bounds__(F32Shape<LNY>::NT, LNY >= 10 ? 1 : (LNY == 9 |
   float2* outs = sm2 + R * F::TILE;
   const float2* E1 = x + (size_t)d * p.nap;
   const float2* src = f == 0 ? E1 + (size_t)k1 * NN - 1 : E1 + p.n1 + (size_t)(k1 - 1) * ny;
-  const bool has = f == 0 || k1 >= 1;
+  const bool has = k1 < p.nx && (f == 0 || k1 >= 1);   // nx may be smaller than R
   float2 v[RV];
 #pragma unroll
   for (int r = 0; r < Q4; ++r) {
@@ -167,7 +176,8 @@ __global__ void __launch_bounds__(F32Shape<LNY>::NT, LNY >= 10 ? 1 : (LNY == 9 |
   for (int i = threadIdx.x; i < n * R; i += F::NT) {
     const int row = i % R, c = i / R, r = c / (n / 2), u = c % (n / 2);
     const int t = u < n / 4 ? u : u - n / 2;
-    dst[(size_t)((2 * t + r) & (n - 1)) * p.nx + row] = outs[(r * R + row) * OP + u];
+    if (blockIdx.x * R + row < p.nx)
+      dst[(size_t)((2 * t + r) & (n - 1)) * p.nx + row] = outs[(r * R + row) * OP + u];
   }
 }
 
@@ -319,7 +329,7 @@ __global__ void __launch_bounds__(SmemC<LNY>::NT, LNY >= 10 ? 2 : (SmemC<LNY>::N
   extern __shared__ __align__(16) float2 sm2[];
   const int f = blockIdx.y, d = blockIdx.z;
   const int g = threadIdx.x / LG, l = threadIdx.x % LG;
-  const int p0 = blockIdx.x * R, cp = p.nx + 1, up = p.nx + 4;
+  const int p0 = blockIdx.x * R, cp = p.nx + 1, up = u_pitch(p.nx);
   const float2* src = Ut + (size_t)(d * 3 + f) * n * up + p0;
 #pragma unroll 16
   for (int i = threadIdx.x; i < n * R; i += NT) {
@@ -428,7 +438,6 @@ __global__ void k_khat_split(const float2* __restrict__ in, float2* __restrict__
 }
 cavity_status launch_khat_split(cavity_ctx* ctx) {
   const Geo& g = ctx->g;
-  if (!f32_fast_size(g.lnx) || !f32_fast_size(g.lny)) return CAVITY_OK;
   const size_t n = (size_t)(g.Px / 2) * (g.Py / 2);
   CK(table_alloc(&ctx->khat32s, n));
   KScope ks_(ctx, KC_SETUP);
@@ -438,17 +447,24 @@ cavity_status launch_khat_split(cavity_ctx* ctx) {
   return CAVITY_OK;
 }
 
-static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x, float2* y,
-                                      void* work, long long ystride, const ParityMap& pm) {
+// y = A x in FP32, on every grid of the FFT operator (the options that used to
+// choose a pass by its transform are accepted and choose nothing)
+template <>
+cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, float2* y,
+                                  void* work, long long ystride, const ParityMap& pm) {
   const Geo& g = ctx->g;
+  if (!g.fft_ok) {
+    ctx->err = "the FFT operator needs the convolution period 4 on both axes";
+    return CAVITY_EINVAL;
+  }
+  if (ystride < 0) ystride = g.nap;
   TbcP p = make_params(ctx);
   cudaStream_t st = ctx->stream;
-  // Vt and Z share one region, U and O the other (each at most the size the
-  // generic passes use)
+  // Vt and Z share one region, U and O the other (u_pitch: they fit)
   const size_t vt = (size_t)ndir * 2 * g.nx * g.Py, z = (size_t)ndir * 3 * (g.nx + 1) * g.ny;
   float2* R1 = (float2*)work;
   float2* R2 = R1 + std::max(vt, z);
-  CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
+  CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = F32Shape<LN>;
     static DeviceFlag done;
@@ -458,7 +474,7 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
         x, R1, p, ctx->lane_tab[1], ctx->ehat_y32[0], ctx->ehat_y32[1]);
     return CAVITY_OK;
   }));
-  CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
+  CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     using F = F32Shape<LN>;
     static DeviceFlag done;
@@ -469,7 +485,7 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
         (float)(2.0 * M_PI / g.Lx), (float)(2.0 * M_PI / g.Ly));
     return CAVITY_OK;
   }));
-  CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
+  CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     constexpr int R = SmemC<LN>::R;
     static DeviceFlag done;
@@ -479,7 +495,7 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
         R2, R1, p, ctx->lane_tab[1]);
     return CAVITY_OK;
   }));
-  CKS(dispatch_log<F32_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
+  CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     constexpr int R = SmemD<LN>::R;
     static DeviceFlag done;
@@ -496,19 +512,4 @@ static cavity_status launch_apply_f32(cavity_ctx* ctx, int ndir, const float2* x
   }
   CK(cudaGetLastError());
   return CAVITY_OK;
-}
-
-// Sides of 4 or 8 intervals (a line has fewer points than the smallest group
-// transform), and a 512-interval side whose pass option asks for the block
-// transform, take the generic passes of tbc_apply.cuh.
-template <>
-cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, float2* y,
-                                  void* work, long long ystride, const ParityMap& pm) {
-  const Geo& g = ctx->g;
-  if (ystride < 0) ystride = g.nap;
-  const bool block = (g.lnx == 9 && ctx->opt[CAVITY_OPT_PASS_B_2048]) ||
-                     (g.lny == 9 && ctx->opt[CAVITY_OPT_PASS_C_2048]);
-  if (g.fft_ok && f32_fast_size(g.lnx) && f32_fast_size(g.lny) && !block)
-    return launch_apply_f32(ctx, ndir, x, y, work, ystride, pm);
-  return launch_apply_generic<float>(ctx, ndir, x, y, work, ystride, pm);
 }
