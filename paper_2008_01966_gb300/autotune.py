@@ -16,9 +16,9 @@ Options and what is timed:
       without the field), per value among GROUP_WIDTHS; a width is kept only if
       every direction converged;
   field_fused (mixed precision, square grids of 32..512 points per side): one
-      field synthesis of the batch (cavity_field) per value, each after a
-      prepare (the library has one path for both values; kept so that cached
-      choices stay complete).
+      field synthesis of the batch (cavity_field).  The library has one path
+      for all values; one is set and timed, so that cached choices and their
+      times stay complete.
 Values are compared by the median of `reps` timed repetitions after one
 warm-up, measured with CUDA events on the context's stream.
 """
@@ -27,7 +27,7 @@ import json
 import os
 
 GROUP_WIDTHS = (16, 8, 4)
-FIELD_PATHS = (1, 2)
+FIELD_PATHS = (1,)
 
 
 def shape_key(cav, ndir, layered):
