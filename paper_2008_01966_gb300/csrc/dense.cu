@@ -1476,7 +1476,9 @@ cavity_status dense_factor(cavity_ctx* ctx, DenseLU& f, const KeptSet& ks, bool 
       return CAVITY_ENOMEM;
     }
     const std::vector<int> map = kept_map(ks, g);
-    CK(cudaMemcpy(f.map, map.data(), sizeof(int) * ks.nk, cudaMemcpyHostToDevice));
+    // on the context's stream, which does not wait for the default stream's copies
+    CK(cudaMemcpyAsync(f.map, map.data(), sizeof(int) * ks.nk, cudaMemcpyHostToDevice, ctx->stream));
+    CK(cudaStreamSynchronize(ctx->stream));
     f.ks = ks;
     f.n = ks.nk;
     f.lda = lda;

@@ -396,6 +396,9 @@ cavity_status launch_khat(cavity_ctx* ctx, double kappa0) {
     std::vector<double> tab;
     j0_table(tab);
     CK(cudaMemcpyToSymbol(g_j0_tab, tab.data(), sizeof(double) * tab.size()));
+    // these copies are on the default stream and may still be on their way from
+    // the runtime's staging memory; a context's own stream does not wait for it
+    CK(cudaStreamSynchronize(nullptr));
     gl_done.set();
   }
   lock.unlock();

@@ -158,7 +158,10 @@ static cudaError_t copy(void* d, const void* s, size_t n) {
   if (n <= (1u << 20)) memmove(d, s, n);
   return cudaSuccess;
 }
-cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) { return copy(d, s, n); }
+cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
+  g_log.push_back("copy on the default stream");
+  return copy(d, s, n);
+}
 cudaError_t cudaMemcpyAsync(void* d, const void* s, size_t n, cudaMemcpyKind k, cudaStream_t) {
   if (k == cudaMemcpyDeviceToHost) g_log.push_back("download " + std::to_string(n));
   return copy(d, s, n);
@@ -179,7 +182,7 @@ cudaError_t cudaMemcpyToSymbol(const void* sym, const void*, size_t, size_t, cud
 }
 cudaError_t cudaMemcpyToSymbolAsync(const void* sym, const void*, size_t, size_t, cudaMemcpyKind,
                                     cudaStream_t) {
-  g_log.push_back("symbol " + names()[sym] + where());
+  g_log.push_back("symbol " + names()[sym] + " async" + where());
   return cudaSuccess;
 }
 cudaError_t cudaMemcpyFromSymbolAsync(void* d, const void*, size_t n, size_t, cudaMemcpyKind,
@@ -212,7 +215,10 @@ cudaError_t cudaOccupancyMaxActiveClusters(int* n, const void*, const cudaLaunch
 // ---- streams, events, errors
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned) { *s = (cudaStream_t)malloc(1); return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { free(s); return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+  g_log.push_back(s ? "sync own" : "sync default");
+  return cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { *e = (cudaEvent_t)malloc(1); return cudaSuccess; }
 cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned) { *e = (cudaEvent_t)malloc(1); return cudaSuccess; }

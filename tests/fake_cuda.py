@@ -50,12 +50,13 @@ class Fake:
 class Context:
     """Calls of the C ABI with host memory for every buffer; each returns its status."""
 
-    def __init__(self, fake, nx=32, ny=32, nz=8, precision="mixed", modes=0, solver="krylov"):
+    def __init__(self, fake, nx=32, ny=32, nz=8, precision="mixed", modes=0, solver="krylov",
+                 stream=None):
         self.fake, self.lib = fake, fake.lib
         d = fake.defs.CavityDesc(1.0, 1.0, 0.5, nx, ny, nz, 0 if precision == "fp64" else 1, 0, 0.0, 0,
                                  0, 0.0, 0, modes, modes, fake.defs.SOLVERS[solver], 0)
         self.h = P()
-        assert self.lib.cavity_setup(ctypes.byref(d), None, ctypes.byref(self.h)) == 0
+        assert self.lib.cavity_setup(ctypes.byref(d), P(stream), ctypes.byref(self.h)) == 0
         nap, fpd = ctypes.c_longlong(), ctypes.c_longlong()
         self.lib.cavity_sizes(self.h, ctypes.byref(nap), ctypes.byref(fpd))
         self.n_ap, self.field_per_dir, self.nz = nap.value, fpd.value, nz

@@ -181,3 +181,21 @@ def test_host_field_leaves_in_chunks(fake, nx, nz, ndir, chunks):
     sizes = [int(e.split()[1]) for e in fake.log(n) if e.startswith("download")]
     assert sum(s for s in sizes if s % level == 0) == ndir * nz * level   # every level once
     ctx.close()
+
+
+def test_no_launch_overtakes_a_copy_on_the_default_stream(fake):
+    """A context's stream may be one that does not wait for the default stream:
+    what is copied there has to be waited for before anything is launched."""
+    fake.lib.fake_set_device(31)
+    for solver, modes in (("krylov", 0), ("dense", 6)):
+        ctx = fake.context(stream=0x1000, solver=solver, modes=modes)
+        n = fake.lib.fake_log_size()
+        ctx.prepare()
+        pending = None
+        for e in fake.log(n):
+            if e.startswith("copy on the default") or (e.startswith("symbol") and " async" not in e):
+                pending = e
+            elif e == "sync default":
+                pending = None
+            assert not (pending and e.startswith("launch")), (pending, e)
+        ctx.close()
