@@ -62,11 +62,12 @@ TOL = 1e-7
 # Oracle GMRES iterations to a relative residual of 1e-12 (first direction of
 # each workload), used to size the reference arm's bounded steps.
 REF_ITERS = {"layered4": 31, "dirs16": 37}
-# DRAM traffic of one launch of a kernel class from one `ncu --set full`
-# capture, per launch of the benchmark (scaled by directions where the
-# capture had fewer; traffic is proportional to the directions).  Only valid
-# for the kernel as captured: emptied whenever the kernel changes.
-NCU_TRAFFIC = {}
+# DRAM traffic of one launch of a kernel class from one ncu capture of a small
+# case (profiles/operator_field_krylov.md), per launch of the benchmark with as
+# many directions (the pass does not depend on the depth).  Only valid for the
+# kernel as captured: emptied whenever the kernel changes.
+NCU_TRAFFIC = {("dirs16", "tbc_B_fp32"): 70.080000e6 + 52.118272e6,
+               ("layered4", "tbc_B_fp32"): 150.015488e6 + 158.286080e6}
 # FP64 FMA throughput measured on a GB300 with a throughput kernel (16
 # independent FMA chains per thread, 8 blocks of 256 threads per SM, CUDA
 # events, best of 5): 1.254 TFLOP/s (FP32 by the same kernel: 78.4 TFLOP/s).

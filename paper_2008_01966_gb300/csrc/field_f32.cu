@@ -17,7 +17,7 @@
 // columns at a time.  Chunks of 512 MB of intermediate: smaller ones that stay
 // in L2 lose more to short grids than they save in traffic (512 x 512 x 256, 8
 // directions: 16.2 ms at 64 MB, 13.1 at 256 MB, 12.5 at 512 MB).
-// Bound: the shared-memory and L1 pipe (pass Y 74 %, X 64 % busy), then issue
+// Bound: the shared-memory and L1 pipe (pass Y 75 %, X 65 % busy), then issue
 // (46, 58 %) and DRAM (46, 56 %).  Measured on a GB300, whole field, before (a
 // persistent kernel that kept the intermediate in L2 at 512 x 512, lines in
 // shared memory elsewhere) and now:

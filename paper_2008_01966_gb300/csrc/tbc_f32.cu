@@ -17,7 +17,7 @@
 //    [j2][p], so pass B reads and writes whole lines; passes A and C turn
 //    several rows at once through shared memory (32-byte pieces).
 // Bound: instruction issue (pass B at 256 x 256, 16 vectors: issue slots 65 %
-// busy, shared-memory pipe 64 %, 122 MB of DRAM traffic in 0.25 ms), three
+// busy, shared-memory and L1 pipe 64 %, 122 MB of DRAM traffic in 0.25 ms), three
 // blocks of 128 threads per SM.  Measured on a GB300, us per launch of pass B,
 // against lines kept in shared memory with three basis transforms (every
 // column's forward transform done twice):
