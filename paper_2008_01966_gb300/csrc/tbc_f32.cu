@@ -123,7 +123,9 @@ template <int LN> struct SmemA {
 };
 // (At 512 and 128 intervals three blocks per SM would spill 160-440 bytes per
 // thread: 512 x 512, 8 vectors, 193 us with three, 162 us with two.)
-template <int LNY>
+// PART: fewer rows than a block takes (nx < R); the guards of this case cost 4 %
+// of the pass at 256 x 256 and 16 vectors.
+template <int LNY, bool PART>
 __global__ void __launch_bounds__(F32Shape<LNY>::NT, LNY >= 10 ? 1 : (LNY == 9 || LNY == 7) ? 2 : 3)
     k_opA(const float2* __restrict__ x, float2* __restrict__ Vt, TbcP p,
           const float2* __restrict__ lt, const float2* __restrict__ eh_c,
@@ -139,7 +141,7 @@ __global__ void __launch_bounds__(F32Shape<LNY>::NT, LNY >= 10 ? 1 : (LNY == 9 |
   float2* outs = sm2 + R * F::TILE;
   const float2* E1 = x + (size_t)d * p.nap;
   const float2* src = f == 0 ? E1 + (size_t)k1 * NN - 1 : E1 + p.n1 + (size_t)(k1 - 1) * ny;
-  const bool has = k1 < p.nx && (f == 0 || k1 >= 1);   // nx may be smaller than R
+  const bool has = (!PART || k1 < p.nx) && (f == 0 || k1 >= 1);
   float2 v[RV];
 #pragma unroll
   for (int r = 0; r < Q4; ++r) {
@@ -176,7 +178,7 @@ __global__ void __launch_bounds__(F32Shape<LNY>::NT, LNY >= 10 ? 1 : (LNY == 9 |
   for (int i = threadIdx.x; i < n * R; i += F::NT) {
     const int row = i % R, c = i / R, r = c / (n / 2), u = c % (n / 2);
     const int t = u < n / 4 ? u : u - n / 2;
-    if (blockIdx.x * R + row < p.nx)
+    if (!PART || blockIdx.x * R + row < p.nx)
       dst[(size_t)((2 * t + r) & (n - 1)) * p.nx + row] = outs[(r * R + row) * OP + u];
   }
 }
@@ -309,7 +311,8 @@ __global__ void F32_BOUNDS(LNX)
 // torus grid, its inverse transform along x2 at the nodes q = 0..ny, and the
 // trapezoid projection onto cos/sin(n pi q / ny), n < ny, as a transform of the
 // even or odd extension (length 2 ny).  The R rows are gathered from
-// U[j2][p] through shared memory.
+// U[j2][p] through shared memory (PACKED: of the pitch of sides of 4 and 8; a
+// pitch by size or as an argument cost 1 - 3 % of the pass at 256 x 256).
 template <int LN> struct SmemC {
   using F = F32Shape<LN>;
   static constexpr int NT = F::LG == 64 ? 256 : F::NT;
@@ -319,7 +322,7 @@ template <int LN> struct SmemC {
   static constexpr int LP = (F::TILE > F::N ? F::TILE : F::N) / 16 * 16 + 16 + (R >= 16 ? 1 : 16 / R);
   static constexpr size_t BYTES = sizeof(float2) * R * LP;
 };
-template <int LNY>
+template <int LNY, bool PACKED>
 __global__ void __launch_bounds__(SmemC<LNY>::NT, LNY >= 10 ? 2 : (SmemC<LNY>::NT == 256 ? 2 : 4))
     k_opC(const float2* __restrict__ Ut, float2* __restrict__ Z, TbcP p,
           const float2* __restrict__ lt) {
@@ -329,7 +332,7 @@ __global__ void __launch_bounds__(SmemC<LNY>::NT, LNY >= 10 ? 2 : (SmemC<LNY>::N
   extern __shared__ __align__(16) float2 sm2[];
   const int f = blockIdx.y, d = blockIdx.z;
   const int g = threadIdx.x / LG, l = threadIdx.x % LG;
-  const int p0 = blockIdx.x * R, cp = p.nx + 1, up = u_pitch(p.nx);
+  const int p0 = blockIdx.x * R, cp = p.nx + 1, up = p.nx + (PACKED ? 1 : 4);   // u_pitch
   const float2* src = Ut + (size_t)(d * 3 + f) * n * up + p0;
 #pragma unroll 16
   for (int i = threadIdx.x; i < n * R; i += NT) {
@@ -468,10 +471,21 @@ cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, fl
     constexpr int LN = decltype(c)::value;
     using F = F32Shape<LN>;
     static DeviceFlag done;
-    CKS(smem_once(ctx, k_opA<LN>, done));
+    const dim3 grid((g.nx + F::R - 1) / F::R, 2, ndir);
+    if constexpr (F::R > 1 << CAV_LOG_MIN) {
+      if (g.nx < F::R) {
+        static DeviceFlag done1;
+        CKS(smem_once(ctx, k_opA<LN, true>, done1));
+        KScope ks_(ctx, KC_TBC_A32);
+        k_opA<LN, true><<<grid, F::NT, SmemA<LN>::BYTES, st>>>(x, R1, p, ctx->lane_tab[1],
+                                                              ctx->ehat_y32[0], ctx->ehat_y32[1]);
+        return CAVITY_OK;
+      }
+    }
+    CKS(smem_once(ctx, k_opA<LN, false>, done));
     KScope ks_(ctx, KC_TBC_A32);
-    k_opA<LN><<<dim3((g.nx + F::R - 1) / F::R, 2, ndir), F::NT, SmemA<LN>::BYTES, st>>>(
-        x, R1, p, ctx->lane_tab[1], ctx->ehat_y32[0], ctx->ehat_y32[1]);
+    k_opA<LN, false><<<grid, F::NT, SmemA<LN>::BYTES, st>>>(x, R1, p, ctx->lane_tab[1],
+                                                           ctx->ehat_y32[0], ctx->ehat_y32[1]);
     return CAVITY_OK;
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
@@ -488,11 +502,18 @@ cavity_status launch_apply<float>(cavity_ctx* ctx, int ndir, const float2* x, fl
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lny, [&](auto c) -> cavity_status {
     constexpr int LN = decltype(c)::value;
     constexpr int R = SmemC<LN>::R;
+    const dim3 grid((g.nx + 1 + R - 1) / R, 3, ndir);
+    if (g.nx < 16) {
+      static DeviceFlag done1;
+      CKS(smem_once(ctx, k_opC<LN, true>, done1));
+      KScope ks_(ctx, KC_TBC_C32);
+      k_opC<LN, true><<<grid, SmemC<LN>::NT, SmemC<LN>::BYTES, st>>>(R2, R1, p, ctx->lane_tab[1]);
+      return CAVITY_OK;
+    }
     static DeviceFlag done;
-    CKS(smem_once(ctx, k_opC<LN>, done));
+    CKS(smem_once(ctx, k_opC<LN, false>, done));
     KScope ks_(ctx, KC_TBC_C32);
-    k_opC<LN><<<dim3((g.nx + 1 + R - 1) / R, 3, ndir), SmemC<LN>::NT, SmemC<LN>::BYTES, st>>>(
-        R2, R1, p, ctx->lane_tab[1]);
+    k_opC<LN, false><<<grid, SmemC<LN>::NT, SmemC<LN>::BYTES, st>>>(R2, R1, p, ctx->lane_tab[1]);
     return CAVITY_OK;
   }));
   CKS(dispatch_log<CAV_LOG_MIN, CAV_LOG_MAX>(g.lnx, [&](auto c) -> cavity_status {
