@@ -252,7 +252,7 @@ __global__ void k_ap32(const double2* __restrict__ a, float2* __restrict__ b, lo
 // more than the overlap gives, 64 x 64 x 32, 64 directions 4.58 ms a solve in
 // one chunk, 5.31 in eight).  Host over device outputs of a solve on a GB300, in
 // 512 MB chunks and now: 512 x 512 x 128, one direction 3.90 -> 3.48 ms;
-// 512 x 512 x 64, two 3.92 -> 3.56; 256 x 256 x 64, eight 3.94 -> 3.71.
+// 512 x 512 x 64, two 3.92 -> 3.53; 256 x 256 x 64, eight 3.94 -> 3.70.
 #define FIELD_HOST_CHUNKS 8
 #define FIELD_HOST_BYTES ((size_t)4 << 20)
 
